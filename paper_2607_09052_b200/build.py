@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcobs.so")
 LIB_TIMING = os.path.join(HERE, "libcobs_timing.so")
-SOURCES = ["api.cu", "score_select.cu", "fused_step.cu", "summaries.cu", "exact_mass.cu", "adaptive.cu"]
+SOURCES = ["api.cu", "score_select.cu", "fused_step.cu", "summaries.cu", "build_fast.cu", "exact_mass.cu", "adaptive.cu"]
 
 
 def nvcc_path() -> str:
@@ -34,7 +34,7 @@ def build(force: bool = False, verbose: bool = False, timing: bool = False) -> s
     lib = LIB_TIMING if timing else LIB
     if not force and not needs_build(lib):
         return lib
-    cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+    cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "--threads", "0",
            "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if timing:
         cmd += ["-DCOBS_TIMING"]

@@ -21,7 +21,7 @@ cudaError_t launch_adaptive_trim(const Params &p, float tau, int k_min, cudaStre
 cudaError_t launch_fused(const Params &p, int phases, cudaStream_t stream);
 bool fused_score_supported(const Params &p);
 enum { PH_SCORE = 1, PH_ATTEND = 2 };
-cudaError_t launch_build(const Params &p, int block_begin, int block_end, cudaStream_t stream);
+cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
 cudaError_t launch_append(const Params &p, const void *k_new, const void *v_new, void *k_pages, void *v_pages, int32_t *seq_lens,
                           int32_t *old_lens, cudaStream_t stream);
 cudaError_t launch_quantise(const float *xi, long long n_vectors, int Ds, int Ds_pad, int scale_dtype, void *codes,
@@ -102,7 +102,7 @@ static int choose_splits(const cobs_config *c) {
 }
 
 struct WorkspaceLayout {
-  size_t status, ctl, e, lse_part, partial, sel_idx, sel_cnt, qtilde, q_stage, out_stage, total;
+  size_t status, ctl, e, lse_part, partial, sel_idx, sel_cnt, qtilde, u_pack, q_stage, out_stage, total;
 };
 
 static WorkspaceLayout layout_workspace(const cobs_config *c) {
@@ -120,6 +120,8 @@ static WorkspaceLayout layout_workspace(const cobs_config *c) {
   w.sel_idx = off; off = align_up(off + B * Hkv * (size_t)c->topk * sizeof(int32_t), 256);
   w.sel_cnt = off; off = align_up(off + B * Hkv * sizeof(int32_t), 256);
   w.qtilde = off; off = align_up(off + (c->sub_dim ? B * Hq * (size_t)((c->sub_dim + 31) / 32 * 32) * sizeof(float) : 0), 256);
+  w.u_pack = off;                                              // U_Q as f16 high + low parts, for the builder
+  off = align_up(off + (c->sub_dim ? Hkv * (size_t)((c->sub_dim + 15) / 16 * 16) * D * 4 : 0), 256);
   w.q_stage = off; off = align_up(off + B * Hq * D * 2, 256);
   w.out_stage = off; off = align_up(off + B * Hq * D * sizeof(float), 256);
   w.total = off;
@@ -287,7 +289,10 @@ int32_t cobs_build_summaries(const cobs_config *cfg, const cobs_kv *kv, int32_t 
   if (build_smem_bytes(p) > 227 * 1024) return COBS_ERR_UNSUPPORTED;
   // one CTA per (sequence, KV head, block of the range): the grid's x extent is 2^31 - 1 at most
   if ((long long)p.B * p.Hkv * (block_end - block_begin) > 0x7fffffffLL) return COBS_ERR_UNSUPPORTED;
-  return cuda_status(launch_build(p, block_begin, block_end, static_cast<cudaStream_t>(stream)));
+  // the score area holds at least one int per block of the range: the builder's marks
+  char *base = static_cast<char *>(workspace);
+  return cuda_status(launch_build(p, block_begin, block_end, reinterpret_cast<int *>(p.e), base + layout_workspace(cfg).u_pack,
+                                  static_cast<cudaStream_t>(stream)));
 }
 
 int32_t cobs_append_token(const cobs_config *cfg, const void *k_new, const void *v_new, void *k_pages, void *v_pages,

@@ -15,7 +15,7 @@
 //
 // One CTA per (sequence, KV head, block); everything stays in shared memory.  All reductions run in
 // a fixed order, so the output bits are a function of the input bits only.
-#include "common.cuh"
+#include "build_common.cuh"
 
 namespace cobs {
 
@@ -27,20 +27,6 @@ constexpr int kMaxSweeps = 16;
 __host__ __device__ inline int build_ldk(const Params &p) { return (((p.D > p.Ds) ? p.D : p.Ds) + 3) / 4 * 4 + 4; }
 
 // --- FP4 quantiser -------------------------------------------------------------------------------
-// code = sign bit of x, nearest E2M1 magnitude to |x| / scale with ties to the even mantissa bit.
-__device__ __forceinline__ uint32_t e2m1_encode(float x, float scale) {
-  const float t = __fdiv_rn(fabsf(x), scale);
-  uint32_t m = 0;
-  m += (t > 0.25f);
-  m += (t >= 0.75f);
-  m += (t > 1.25f);
-  m += (t >= 1.75f);
-  m += (t > 2.5f);
-  m += (t >= 3.5f);
-  m += (t > 5.0f);
-  return (signbit(x) ? 8u : 0u) | m;
-}
-
 // Quantise one factor row held in `row` (Ds floats, shared or global) by one warp.
 // codes: packed row of Ds_pad / 2 bytes (word-aligned); scale_out: element `vec` of the scale array.
 __device__ void quantise_row_warp(const float *row, int Ds, int Ds_pad, uint32_t *codes_words, void *scale_arr,
@@ -48,8 +34,7 @@ __device__ void quantise_row_warp(const float *row, int Ds, int Ds_pad, uint32_t
   float a = 0.f;
   for (int j = lane; j < Ds; j += 32) a = fmaxf(a, fabsf(row[j]));
   a = warp_max(a);
-  float scale = __fdiv_rn(a, 6.0f);
-  if (scale_dtype == COBS_SCALE_FP16) scale = __half2float(__float2half_rn(scale));
+  const float scale = fp4_scale(a, scale_dtype);
   for (int w = lane; w < Ds_pad / 8; w += 32) {
     uint32_t word = 0;
     if (scale > 0.f) {
@@ -285,8 +270,7 @@ __host__ __device__ inline BuildSmem build_smem_layout(const Params &p) {
 }
 
 template <int TL>
-__global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4) build_kernel(Params p, int block_begin, int block_end, int solver) {
-  extern __shared__ __align__(16) float sm[];
+__device__ __forceinline__ void build_block(const Params &p, float *sm, int u, int blk, int solver) {
   constexpr int L = 16 * TL;
   const int D = p.D, Dk = p.Ds, ldk = build_ldk(p);
   const BuildSmem lay = build_smem_layout(p);
@@ -300,9 +284,7 @@ __global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4) build_kernel
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int NW = kBuildThreads / 32;
-  const int n_range = block_end - block_begin;
-  const int blk = block_begin + (int)(blockIdx.x % n_range);
-  const int u = blockIdx.x / n_range, b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
+  const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
   const int T = p.seq_lens[b_idx];
   if (blk >= min(T / L, p.NB)) return;
   const size_t rec = (size_t)u * p.NB + blk;
@@ -797,30 +779,66 @@ __global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4) build_kernel
   }
 }
 
+// flags == NULL: one CTA per (unit, block of the range).  Else: the blocks whose flag is set, found by a grid that strides
+// over the flags 256 at a time (nearly always there are none).
+template <int TL>
+__global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4)
+build_kernel(Params p, int block_begin, int block_end, int solver, const int *flags, int n) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int s_flag[kBuildThreads];
+  const int n_range = block_end - block_begin, per = flags ? kBuildThreads : 1;
+  for (long long base = (long long)blockIdx.x * per; base < n; base += (long long)gridDim.x * per) {
+    if (flags) {
+      const long long i = base + threadIdx.x;
+      const int f = (i < n) ? flags[i] : 0;
+      if (!__syncthreads_or(f)) continue;
+      s_flag[threadIdx.x] = f;
+      __syncthreads();
+    }
+    for (int j = 0; j < per; ++j) {
+      if (flags && !s_flag[j]) continue;
+      const int i = (int)base + j;
+      build_block<TL>(p, sm, i / n_range, block_begin + i % n_range, solver);
+      __syncthreads();                               // the next block takes the same shared memory
+    }
+    __syncthreads();
+  }
+}
+
 size_t build_smem_bytes(const Params &p) { return (size_t)build_smem_layout(p).total * sizeof(float); }
 
 template <int TL>
-static cudaError_t launch_build_tl(const Params &p, int block_begin, int block_end, int solver, cudaStream_t stream) {
+static cudaError_t launch_build_tl(const Params &p, int block_begin, int block_end, int solver, const int *flags, cudaStream_t stream) {
   const size_t smem = build_smem_bytes(p);
   cudaError_t e = cudaFuncSetAttribute(build_kernel<TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long long n_cta = (long long)p.B * p.Hkv * (block_end - block_begin);
-  build_kernel<TL><<<(unsigned)n_cta, kBuildThreads, smem, stream>>>(p, block_begin, block_end, solver);
+  const int n = p.B * p.Hkv * (block_end - block_begin);
+  const int grid = flags ? min((n + kBuildThreads - 1) / kBuildThreads, 296) : n;
+  build_kernel<TL><<<grid, kBuildThreads, smem, stream>>>(p, block_begin, block_end, solver, flags, n);
   count_launch();
   return cudaGetLastError();
 }
 
-// COBS_BUILD_SOLVER=jacobi (read at every call) sends every block down the Jacobi route; the default is the
-// tridiagonal route with Jacobi as its fallback.
-cudaError_t launch_build(const Params &p, int block_begin, int block_end, cudaStream_t stream) {
+cudaError_t launch_build_fast(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
+
+// The main route is build_fast.cu; blocks that it marks in `flags` are solved by the kernel above.  The diagonal-skew
+// scalars exist in the kernel above only.  COBS_BUILD_SOLVER=jacobi (read at every call) sends every block down its Jacobi
+// route.
+cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream) {
   if (block_end - block_begin <= 0) return cudaSuccess;
   const char *v = getenv("COBS_BUILD_SOLVER");
   const int solver = (v && strcmp(v, "jacobi") == 0) ? 1 : 0;
+  if (solver || p.skew) {
+    flags = nullptr;
+  } else {
+    const cudaError_t e = launch_build_fast(p, block_begin, block_end, flags, u_pack, stream);
+    if (e != cudaSuccess || p.r == 0) return e;
+  }
   switch (p.L) {
-    case 16: return launch_build_tl<1>(p, block_begin, block_end, solver, stream);
-    case 32: return launch_build_tl<2>(p, block_begin, block_end, solver, stream);
-    case 64: return launch_build_tl<4>(p, block_begin, block_end, solver, stream);
-    default: return launch_build_tl<8>(p, block_begin, block_end, solver, stream);
+    case 16: return launch_build_tl<1>(p, block_begin, block_end, solver, flags, stream);
+    case 32: return launch_build_tl<2>(p, block_begin, block_end, solver, flags, stream);
+    case 64: return launch_build_tl<4>(p, block_begin, block_end, solver, flags, stream);
+    default: return launch_build_tl<8>(p, block_begin, block_end, solver, flags, stream);
   }
 }
 

@@ -942,6 +942,25 @@ def test_builder_ranks_above_eight(rank, L, D, solver, monkeypatch):
     check_builder(wl, [(0, 0), (0, 1)])
 
 
+@pytest.mark.parametrize("offset", [0.9, 1.1, 40.0])
+@pytest.mark.parametrize("L,D,rank,sub", [(16, 64, 5, 0), (64, 128, 8, 0), (128, 128, 4, 0), (128, 64, 1, 0), (32, 128, 9, 71), (128, 128, 3, 85)])
+def test_builder_keys_with_a_large_mean(L, D, rank, sub, offset, monkeypatch):
+    """Unit keys around a mean of `offset` per element: below 1 the Gram matrix is centred after the product, above 1
+    the keys are (two precisions of f16), with a subspace always.  Bounds as for any block: the mean drops out of
+    every quantity that is checked, and its own error is relative to it."""
+    wl = synth.Workload("offset", 1, 4, 2, D, 5 * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp4", sub_dim=sub,
+                        key_model="iid", shuffle_pages=True, seed=31)
+    draw = synth.generate
+
+    def moved(w, device="cpu"):
+        inp = draw(w, device)
+        inp["k_pages"] = (inp["k_pages"].float() + offset).to(torch.bfloat16)
+        return inp
+
+    monkeypatch.setattr(synth, "generate", moved)
+    check_builder(wl, [(0, 0), (0, 1)])
+
+
 @pytest.mark.parametrize("solver", ["tridiagonal", "jacobi"])
 @pytest.mark.parametrize("L", [16, 32, 64, 128])
 def test_builder_structured_spectra(L, solver, monkeypatch):
