@@ -256,9 +256,8 @@ def measure_other(B, name, dev, flush, peak, steps):
 
 def run_phase_times(args):
     """Where the time of one step goes, from the library build that carries timing code (libcobs_timing.so):
-    per-warp global-timer stamps at the phase boundaries, clock cycles per category inside the phases, and per
-    unit the moments its scores were complete and its selection was published.  One JSON line; times in
-    microseconds from the earliest warp's start.  Numbers of this build are not benchmark values."""
+    global-timer stamps of every CTA at the phase boundaries.  One JSON line; times in microseconds from the earliest
+    CTA's start.  Numbers of this build are not benchmark values."""
     import ctypes as C
     import numpy as np
     from paper_2607_09052_b200 import binding as B
@@ -283,50 +282,26 @@ def run_phase_times(args):
         flush.zero_()
         step()
     torch.cuda.synchronize()
-    acc = (C.c_ulonglong * (8 * 4096))()
-    B.lib().cobs_debug_acc(acc, 1)                          # clear the accumulators
     flush.zero_()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ev0.record(m.stream)
     step()
     ev1.record(m.stream)
     torch.cuda.synchronize()
-    buf = (C.c_ulonglong * (4 * 4096))()
-    assert B.lib().cobs_debug_times(buf) == 0 and B.lib().cobs_debug_acc(acc, 1) == 0
-    t = np.frombuffer(buf, dtype=np.uint64).reshape(4, 4096).astype(np.int64)
-    n = int((t[0] > 0).sum())
-    t = t[:, :n]
+    buf = (C.c_ulonglong * (8 * 4096))()
+    assert B.lib().cobs_debug_stamps(buf) == 0
+    t = np.frombuffer(buf, dtype=np.uint64).reshape(8, 4096).astype(np.int64)
+    t = t[:, t[0] > 0]
     t0 = int(t[0].min())
-    raw = np.frombuffer(acc, dtype=np.uint64).reshape(8, 4096).astype(np.int64)
-    mhz = 1965.0
 
     def stats(x):
         return {k: round(float(v), 2) for k, v in zip(("min", "p10", "p50", "p90", "max"),
                                                       [x.min(), *np.percentile(x, [10, 50, 90]), x.max()])}
-    out = {"phase_times": True, "workload": wl.name, "mode": args.phase_times, "streaming_warps": n,
+    names = ["start", "chunks scored", "log-sum-exp known", "scores known", "selected", "groups attended",
+             "CTA merged", "cluster merged"]
+    out = {"phase_times": True, "workload": wl.name, "mode": args.phase_times, "ctas": int(t.shape[1]),
            "step_us_this_build": round(ev0.elapsed_time(ev1) * 1e3, 2),
-           "warp_stamps_us": {name: stats((t[k] - t0) / 1e3) for k, name in
-                              enumerate(["start", "scoring_done", "attention_start", "attention_done"])}}
-    sc = raw[:, 1200:1200 + n].astype(np.float64) / mhz
-    busy = sc.sum(0) > 0.5
-    names_s = ["next position", "after issue", "wait for copies", "arithmetic", "epilogue", "issue copies", "seek", "fence + count"]
-    out["scoring_us_per_working_warp"] = {nm: round(float(sc[k][busy].mean()), 2) for k, nm in enumerate(names_s)}
-    out["scoring_working_warps"] = int(busy.sum())
-    if not score_only:
-        at = raw[:, :n].astype(np.float64) / mhz
-        names_a = ["after the draw", "item set-up", "wait for selection", "group table + query", "stream loop",
-                   "write partial + fence + count", "draw the next item", "merge (last closer of a unit)"]
-        out["attention_us_per_warp"] = {nm: round(float(at[k].mean()), 2) for k, nm in enumerate(names_a)}
-        late = np.argsort(t[3])[-8:]
-        out["latest_warps"] = [{"warp": int(w), "attention_start": round(float((t[2][w] - t0) / 1e3), 1),
-                                "attention_done": round(float((t[3][w] - t0) / 1e3), 1),
-                                **{nm: round(float(at[k][w]), 1) for k, nm in enumerate(names_a)}} for w in late]
-    nu = wl.batch * wl.n_kv_heads
-    st = [(raw[k, 3000:3000 + min(nu, 1024)] - t0) / 1e3 for k in (0, 2, 3, 4, 5, 1)]
-    out["selection_us"] = {"unit_scored_at": stats(st[0]), "unit_ready_at": stats(st[5]),
-                           "duration": stats(st[5] - st[0]),
-                           "parts_mean": {nm: round(float((st[i + 1] - st[i]).mean()), 2) for i, nm in
-                                          enumerate(["loads + lse", "scores", "bisection", "compaction", "fence + flag"])}}
+           "cta_stamps_us": {nm: stats((t[k][t[k] > 0] - t0) / 1e3) for k, nm in enumerate(names) if (t[k] > 0).any()}}
     out["status"] = B.cobs_read_status(m.ws)
     print(json.dumps(out), flush=True)
 
@@ -488,7 +463,7 @@ def run_ours(args):
                    "sharding": "independent sequences per rank, no collective"},
         "frac_of_measured_peak": round(value / (world * peak), 4), "peak_gbs": peak, "peak_kind": peak_kind,
         "frac_of_nominal_8tbs": round(value / (world * 8000.0), 4),
-        "roofline": {"bound": "hbm", "kernel": "fused_step_kernel (scoring + selection + attention + merge)",
+        "roofline": {"bound": "hbm", "kernel": "unit_step_kernel (scoring + selection + attention + merge)",
                      "achieved": round(achieved, 2), "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": TRAFFIC_BYTES.get(wl.name), "algorithmic_bytes": step_bytes,
                      "launch_ms": round(ms_per_step, 6), "kernels_per_step": kernels_per_step,

@@ -18,7 +18,7 @@
  *     `workspace` (size from cobs_workspace_bytes, 256-byte aligned).  The workspace must not be
  *     shared by calls that may overlap on the GPU.  Calls of different configurations may use one
  *     workspace in turn if it is as large as the largest of them needs (the first 1.5 MB hold the
- *     status word and the hand-off counters of the persistent kernel, at the same places for every
+ *     status word and the hand-off counters of the tcgen05 variant, at the same places for every
  *     shape; cobs_reset_status clears them).
  *   - All work is enqueued on `stream` (a cudaStream_t passed as void*, NULL = default stream) and
  *     the call returns without synchronising, except the *_host entry point and cobs_read_status.
@@ -124,7 +124,7 @@ typedef struct {
  *   c_i = g_i / lam_i^(3/2),   g_i = 1/L sum_{t in b} (u_i . (k_t - kbar))^3   (0 for a null factor),
  * adds 1/6 sum_i c_i (xi_i . q')^3 (= 1/6 sum_i (u_i . q')^3 g_i) to the block's log-mass estimate.
  * With skew != NULL: cobs_build_summaries writes the scalars (from the unrounded factors), cobs_score_select and
- * cobs_decode_step add the term; scoring then runs in the generic kernels, not in the one-launch step.  Full-space
+ * cobs_decode_step add the term (with FP4 factors scoring then runs in the generic kernels, not in the one-launch step).  Full-space
  * descriptors only (sub_dim == 0), rank >= 1: otherwise COBS_ERR_UNSUPPORTED.
  */
 
@@ -282,20 +282,14 @@ int32_t cobs_decode_step_host(const cobs_config *cfg, const void *q_host, const 
  * Who needs it: code that runs where device allocation is off limits - a decode loop inside a serving
  * process whose memory pool belongs to another component and is fully handed out, a latency-critical
  * path where cudaMalloc's device-wide synchronisation is not acceptable, a plug-in that receives only
- * its input and output tensors.  Such a caller has nowhere to get the split-KV scratch from, so this
- * variant keeps the scratch (status word, per-unit counters, split partials) in a fixed device array
- * inside the library: COBS_STATIC_SCRATCH_BYTES per GPU, held from the moment the library is loaded on
- * that GPU until the process exits.  The call allocates nothing and frees nothing.
+ * its input and output tensors.  The split-KV partials of a unit never leave the shared memory of its
+ * cluster, so the call needs no scratch in global memory: it allocates nothing, frees nothing and holds
+ * nothing.
  *
  * Limits and rules:
- *   - the configuration's scratch need, 256 + 12 * B * Hkv (rounded up to 256) + B * Hkv * slices * G *
- *     (D + 2) * 4 bytes, must fit COBS_STATIC_SCRATCH_BYTES, else COBS_ERR_WORKSPACE_TOO_SMALL is
- *     returned and nothing is launched (the benchmark's 16 x 8 units at G = 4, D = 128 need 2.4 MB);
- *   - the first call on a device looks up the array's device address (a one-off set-up step); make that
- *     first call outside any stream capture;
- *   - all calls on a device share the one array and it keeps the previous call's contents: the call
- *     itself clears the status word and the counters on `stream` before launching, but two calls that
- *     may overlap on the GPU (different streams, no dependency) race on it - serialise them;
+ *   - a configuration whose split-KV partials would not fit COBS_STATIC_SCRATCH_BYTES if they did go
+ *     through global memory, 256 + 12 * B * Hkv (rounded up to 256) + B * Hkv * slices * G * (D + 2) * 4
+ *     bytes, is refused with COBS_ERR_WORKSPACE_TOO_SMALL and nothing is launched;
  *   - device-side problems are not reported through a status word the caller can read here: an
  *     out-of-range selection entry or page id is skipped, as in cobs_sparse_decode.
  * Arguments as for cobs_sparse_decode.

@@ -240,9 +240,8 @@ def cobs_sparse_decode(cfg: Config, q: torch.Tensor, kv: KV, sel_idx: torch.Tens
 
 def cobs_sparse_decode_static(cfg: Config, q: torch.Tensor, kv: KV, sel_idx: torch.Tensor, sel_cnt: torch.Tensor,
                               out: torch.Tensor, lse: Optional[torch.Tensor], stream=None):
-    """cobs_sparse_decode without a workspace: the scratch is a fixed device array inside the library, so the
-    call allocates nothing (for callers that are not allowed to allocate device memory).  Raises CobsError(3)
-    when the configuration needs more scratch than the library holds."""
+    """cobs_sparse_decode without a workspace (for callers that are not allowed to allocate device memory).  Raises
+    CobsError(3) for a configuration beyond COBS_STATIC_SCRATCH_BYTES (see include/cobs.h)."""
     _check(lib().cobs_sparse_decode_static(C.byref(cfg), _ptr(q), C.byref(kv), _ptr(sel_idx), _ptr(sel_cnt),
                                            _ptr(out), _ptr(lse), _stream(stream)), "cobs_sparse_decode_static")
 

@@ -1,6 +1,6 @@
 """Build the CUDA library in-tree: paper_2607_09052_b200/libcobs.so (sm_100a only).
 
-`--timing` builds a second library, libcobs_timing.so, whose step kernel records per-warp phase timestamps
+`--timing` builds a second library, libcobs_timing.so, whose step kernel records phase timestamps
 (read by `bench.py --phase-times`); the production library carries no timing code."""
 
 from __future__ import annotations
@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcobs.so")
 LIB_TIMING = os.path.join(HERE, "libcobs_timing.so")
-SOURCES = ["api.cu", "score_select.cu", "fused_step.cu", "summaries.cu", "build_fast.cu", "exact_mass.cu", "adaptive.cu"]
+SOURCES = ["api.cu", "score_select.cu", "unit_step.cu", "tcgen05_step.cu", "summaries.cu", "build_fast.cu", "exact_mass.cu", "adaptive.cu"]
 
 
 def nvcc_path() -> str:

@@ -4,7 +4,7 @@
 
 #include <cstdlib>
 
-#include "common.cuh"
+#include "step_common.cuh"
 
 #include <atomic>
 
@@ -18,9 +18,10 @@ cudaError_t launch_score(const Params &p, cudaStream_t stream);
 cudaError_t launch_select(const Params &p, cudaStream_t stream);
 cudaError_t launch_exact_mass(const Params &p, cudaStream_t stream);
 cudaError_t launch_adaptive_trim(const Params &p, float tau, int k_min, cudaStream_t stream);
-cudaError_t launch_fused(const Params &p, int phases, cudaStream_t stream);
-bool fused_score_supported(const Params &p);
-enum { PH_SCORE = 1, PH_ATTEND = 2 };
+cudaError_t launch_unit_step(const Params &p, int phases, cudaStream_t stream);
+bool unit_score_supported(const Params &p);
+cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream);
+bool umma_score_supported(const Params &p);
 cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
 cudaError_t launch_append(const Params &p, const void *k_new, const void *v_new, void *k_pages, void *v_pages, int32_t *seq_lens,
                           int32_t *old_lens, cudaStream_t stream);
@@ -102,7 +103,7 @@ static int choose_splits(const cobs_config *c) {
 }
 
 struct WorkspaceLayout {
-  size_t status, ctl, e, lse_part, partial, sel_idx, sel_cnt, qtilde, u_pack, q_stage, out_stage, total;
+  size_t status, ctl, e, lse_part, partial, sel_idx, sel_cnt, u_pack, q_stage, out_stage, total;
 };
 
 static WorkspaceLayout layout_workspace(const cobs_config *c) {
@@ -114,12 +115,11 @@ static WorkspaceLayout layout_workspace(const cobs_config *c) {
   // 3 * kMaxUnits ints after set 0 whatever the shape, so that a workspace that serves calls of different shapes keeps
   // its counters in the same places and no call's scratch arrays lie over another shape's counters
   w.ctl = off; off = align_up(off + 6 * (size_t)kMaxUnits * sizeof(int), 256);
-  w.e = off; off = align_up(off + B * Hq * (size_t)c->max_blocks * sizeof(float), 256);
+  w.e = off; off = align_up(off + B * Hq * (size_t)((c->max_blocks + 15) / 16 * 16) * sizeof(float), 256);
   w.lse_part = off; off = align_up(off + B * Hq * (size_t)((c->max_blocks + 15) / 16) * 4 * 2 * sizeof(float), 256);   // up to four pairs per chunk
   w.partial = off; off = align_up(off + B * Hkv * (size_t)choose_splits(c) * G * (D + 2) * sizeof(float), 256);
   w.sel_idx = off; off = align_up(off + B * Hkv * (size_t)c->topk * sizeof(int32_t), 256);
   w.sel_cnt = off; off = align_up(off + B * Hkv * sizeof(int32_t), 256);
-  w.qtilde = off; off = align_up(off + (c->sub_dim ? B * Hq * (size_t)((c->sub_dim + 31) / 32 * 32) * sizeof(float) : 0), 256);
   w.u_pack = off;                                              // U_Q as f16 high + low parts, for the builder
   off = align_up(off + (c->sub_dim ? Hkv * (size_t)((c->sub_dim + 15) / 16 * 16) * D * 4 : 0), 256);
   w.q_stage = off; off = align_up(off + B * Hq * D * 2, 256);
@@ -148,7 +148,6 @@ static void fill_params(Params &p, const cobs_config *c, void *workspace) {
     p.ctl_set_stride = 3 * kMaxUnits;
     p.ctl_ready = p.ctl_score + (size_t)p.B * p.Hkv;
     p.ctl_att = p.ctl_ready + (size_t)p.B * p.Hkv;
-    p.qtilde_out = reinterpret_cast<float *>(base + w.qtilde);
     p.e = reinterpret_cast<float *>(base + w.e);
     p.lse_part = reinterpret_cast<float *>(base + w.lse_part);
     p.partial = reinterpret_cast<float *>(base + w.partial);
@@ -191,20 +190,18 @@ static int32_t set_kv(Params &p, const cobs_kv *kv) {
 
 static int32_t cuda_status(cudaError_t e) { return e == cudaSuccess ? COBS_OK : COBS_ERR_CUDA; }
 
-// Validated kernel parameters of an attention-only call whose scratch is not a caller workspace.
-// Fills everything except the scratch pointers (status, counters, partials); reports the attention
-// slices per unit so that the caller can lay its scratch out.
-int32_t prepare_attend_params(const cobs_config *cfg, const void *q, const cobs_kv *kv, const int32_t *sel_idx,
-                              const int32_t *sel_cnt, float *out, float *lse_or_null, Params *p) {
-  int32_t st = validate_config(cfg);
-  if (st != COBS_OK) return st;
-  if (!q || !aligned16(q) || !sel_idx || !sel_cnt || !out || !aligned16(out)) return COBS_ERR_INVALID_ARG;
-  fill_params(*p, cfg, nullptr);
-  if ((st = set_kv(*p, kv)) != COBS_OK) return st;
-  p->q = static_cast<const __nv_bfloat16 *>(q);
-  p->sel_idx = const_cast<int32_t *>(sel_idx); p->sel_cnt = const_cast<int32_t *>(sel_cnt);
-  p->out = out; p->lse = lse_or_null;
-  return COBS_OK;
+// Scoring and selection, with the attention or without: one launch.  The generic scoring and selection kernels are for what the
+// unit kernel does not cover.
+static cudaError_t launch_score_step(const Params &p, int phases, cudaStream_t s) {
+  if (umma_score_supported(p)) {
+    const cudaError_t e = launch_fused_umma(p, phases, s);
+    if (e != cudaErrorNotSupported) return e;
+  }
+  if (unit_score_supported(p)) return launch_unit_step(p, phases, s);
+  cudaError_t e = launch_score(p, s);
+  if (e == cudaSuccess) e = launch_select(p, s);
+  if (e == cudaSuccess && (phases & PH_ATTEND)) e = launch_unit_step(p, PH_ATTEND, s);
+  return e;
 }
 
 }  // namespace cobs
@@ -339,13 +336,7 @@ int32_t cobs_score_select(const cobs_config *cfg, const void *q, const cobs_summ
   p.seq_lens = seq_lens;
   p.sel_idx = sel_idx; p.sel_cnt = sel_cnt; p.scores = scores_or_null;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (fused_score_supported(p)) {
-    if (p.u_q) p.qtilde = p.qtilde_out;
-    return cuda_status(launch_fused(p, PH_SCORE, s));
-  }
-  cudaError_t e = launch_score(p, s);
-  if (e != cudaSuccess) return COBS_ERR_CUDA;
-  return cuda_status(launch_select(p, s));
+  return cuda_status(launch_score_step(p, PH_SCORE, s));
 }
 
 int32_t cobs_exact_select(const cobs_config *cfg, const void *q, const cobs_kv *kv, int32_t *sel_idx, int32_t *sel_cnt,
@@ -393,7 +384,25 @@ int32_t cobs_sparse_decode(const cobs_config *cfg, const void *q, const cobs_kv 
   p.q = static_cast<const __nv_bfloat16 *>(q);
   p.sel_idx = const_cast<int32_t *>(sel_idx); p.sel_cnt = const_cast<int32_t *>(sel_cnt);
   p.out = out; p.lse = lse_or_null;
-  return cuda_status(launch_fused(p, PH_ATTEND, static_cast<cudaStream_t>(stream)));
+  return cuda_status(launch_unit_step(p, PH_ATTEND, static_cast<cudaStream_t>(stream)));
+}
+
+int32_t cobs_sparse_decode_static(const cobs_config *cfg, const void *q, const cobs_kv *kv, const int32_t *sel_idx,
+                                  const int32_t *sel_cnt, float *out, float *lse_or_null, void *stream) {
+  int32_t st = validate_config(cfg);
+  if (st != COBS_OK) return st;
+  if (!q || !aligned16(q) || !sel_idx || !sel_cnt || !out || !aligned16(out)) return COBS_ERR_INVALID_ARG;
+  Params p;
+  fill_params(p, cfg, nullptr);
+  if ((st = set_kv(p, kv)) != COBS_OK) return st;
+  // the limit that callers were given; the kernel itself needs no scratch in global memory
+  const size_t units = (size_t)p.B * p.Hkv;
+  if (kStatusBytes + align_up(3 * units * sizeof(int), 256) + units * p.n_splits * p.G * (size_t)(p.D + 2) * sizeof(float) >
+      (size_t)COBS_STATIC_SCRATCH_BYTES) return COBS_ERR_WORKSPACE_TOO_SMALL;
+  p.q = static_cast<const __nv_bfloat16 *>(q);
+  p.sel_idx = const_cast<int32_t *>(sel_idx); p.sel_cnt = const_cast<int32_t *>(sel_cnt);
+  p.out = out; p.lse = lse_or_null;
+  return cuda_status(launch_unit_step(p, PH_ATTEND, static_cast<cudaStream_t>(stream)));
 }
 
 int32_t cobs_decode_step(const cobs_config *cfg, const void *q, const cobs_kv *kv, const cobs_summaries *summ,
@@ -412,16 +421,7 @@ int32_t cobs_decode_step(const cobs_config *cfg, const void *q, const cobs_kv *k
   if (sel_idx_or_null) { p.sel_idx = sel_idx_or_null; p.sel_cnt = sel_cnt_or_null; }
   p.out = out; p.lse = lse_or_null;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (fused_score_supported(p)) {
-    if (p.u_q) p.qtilde = p.qtilde_out;
-    return cuda_status(launch_fused(p, PH_SCORE | PH_ATTEND, s));
-  }
-  // summaries the persistent kernel's scoring phase does not cover (fp32, odd subspace widths):
-  // generic scoring and selection kernels first, then the persistent kernel for the attention
-  cudaError_t e = launch_score(p, s);
-  if (e != cudaSuccess) return COBS_ERR_CUDA;
-  if ((e = launch_select(p, s)) != cudaSuccess) return COBS_ERR_CUDA;
-  return cuda_status(launch_fused(p, PH_ATTEND, s));
+  return cuda_status(launch_score_step(p, PH_SCORE | PH_ATTEND, s));
 }
 
 int32_t cobs_decode_step_host(const cobs_config *cfg, const void *q_host, const cobs_kv *kv,

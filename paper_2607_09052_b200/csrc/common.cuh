@@ -42,8 +42,6 @@ struct Params {
   int *ctl_ready;             // [B * Hkv] 1 once the unit's selection is written
   int *ctl_att;               // [B * Hkv] attention slices finished per unit
   int ctl_set_stride;         // ints from a per-unit array of set 0 to the same array of set 1 (the same for every shape)
-  const float *qtilde;        // [B][Hq][Ds_pad] projected subspace query (what the scoring reads), or NULL
-  float *qtilde_out;          // where the step kernel's prologue writes it (workspace)
   float *e;                   // [B][Hkv][G][NB]
   float *lse_part;            // [B][Hkv][G][ceil(NB / 16)][2] per-chunk (max, sum-exp) of e
   float *partial;             // [B][Hkv][n_splits] slices of [G][D] accumulators + [G] (max, sum) pairs

@@ -1,37 +1,13 @@
-// The decode step as ONE persistent kernel: block scoring, top-k selection, block-sparse attention
-// and the split-KV merge (steps (b), (c), (d)).
+// An opt-in form of the decode step whose block scoring runs on the 5th-generation tensor cores (tcgen05), for packed E2M1
+// factors in the full key space, D = 128, r = 8.  (The step that runs by default is unit_step.cu.)
 //
-// Why one kernel.  A step moves a few hundred MiB; at HBM speed that is tens of microseconds, so
-// every kernel boundary (launch, ramp-up, tail, the idle time while a single CTA per unit selects)
-// costs a visible fraction of the step.  Here the grid is one CTA per SM, fully resident (cooperative
-// launch), with two kinds of warps:
-//
-//   streaming warps (8 per CTA), each with its own slice of shared memory:
-//     phase S  score 16-block chunks of summaries: the units are scored in waves, and inside a wave every
-//              warp takes one contiguous range of chunks; per chunk it leaves t = exp(e - chunk max) per
-//              block and head, the chunk's (max, sum) pair, and counts the chunk on its unit;
-//     phase A  attend over (unit, slice) items drawn from one global counter in unit order; a warp whose
-//              slice holds selected blocks waits (bounded) for that unit's selection, slices that hold only
-//              window blocks never wait; the warp that finishes the last slice of a unit merges the
-//              partials and writes the output;
-//   a selection team (4 warps per CTA) that selects unit u (team of CTA u mod grid) as soon as all its
-//     chunks are counted, while the streaming warps carry on with the next wave.
-//
-// Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp
-// alone (no CTA barrier anywhere in the loops).  Scoring: a chunk is three contiguous pieces of the summary
-// arrays, fetched by three bulk copies (cp.async.bulk, completion on an mbarrier) issued by one lane, two
-// stages.  Attention: K and V of a 16-token group share a stage of a three-stage cp.async ring (XOR-swizzled
-// 16-byte chunks, read back with ldmatrix / ldmatrix.trans).
-//
-// Arithmetic.  mma.sync m16n8k16 with fp32 accumulation throughout:
-//   scoring   rows = 16 block means, or factor i of 16 blocks; columns = the G query heads.  A thread
-//             owns two blocks (rows gid, gid + 8), so all results of a block land in one thread.
-//             bf16 operands multiply the raw bf16 query (exact products); FP4 codes become f16 by
-//             the hardware conversion and multiply the query scaled by a per-head power of two
-//             (exact in f16), or an f16 high + low split of the fp32 subspace query.
-//   attention S^T = q K^T with the heads as rows (zero padded to 16) and 8 tokens as columns; the S
-//             accumulators are the A fragments of P V as they sit in registers; P = bf16 high + low.
-// An opt-in variant runs phase S of the main configuration on tcgen05 (further down).
+// One persistent kernel, one CTA per SM, fully resident (cooperative launch):
+//   scoring     a producer warp, an MMA issuer warp and two epilogue sets of four warps per CTA (further down); the units are
+//               scored in waves
+//   selection   a team of four warps per CTA selects unit u (team of CTA u mod grid) as soon as all its chunks are counted
+//   attention   the epilogue warps then attend over (unit, slice) items drawn from one global counter in unit order; a warp
+//               whose slice holds selected blocks waits (bounded) for that unit's selection; the warp that finishes the last
+//               slice of a unit merges the partials and writes the output
 //
 // Cross-warp hand-offs go through global counters in the workspace (release: write, __threadfence,
 // atomicAdd; acquire: volatile read, __threadfence, .cg loads).  Every wait is bounded; on expiry the
@@ -46,7 +22,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "common.cuh"
+#include "step_common.cuh"
 
 namespace cobs {
 
@@ -54,8 +30,6 @@ constexpr int kFWarps = 8;                                   // streaming warps 
 constexpr int kSelWarps = 4;                                 // selection team of the CTA
 constexpr int kSelThreads = kSelWarps * 32;
 constexpr int kLenCache = 256;                               // sequence lengths cached in shared memory
-constexpr int kFThreads = (kFWarps + kSelWarps) * 32;        // one CTA per SM
-constexpr int kScoreStageBytes = 14080;                      // means + factor rows + scales of a 16-block chunk
 constexpr int kAttStages = 3;
 constexpr int kAttStageBytes = 2 * 16 * 128 * 2;             // K + V of one 16-token group, D = 128
 // The hand-off counters exist twice.  A launch works on the set named by bit 31 of the epoch word; the low bits of
@@ -90,153 +64,15 @@ __device__ __forceinline__ void ctl_turn(const Params &p) {           // the who
 }
 
 constexpr int kTableEntries = 256;                           // 16-token groups per attention item
-constexpr int kRingBytes = (2 * kScoreStageBytes > kAttStages * kAttStageBytes + kTableEntries * 8)
-                               ? 2 * kScoreStageBytes : kAttStages * kAttStageBytes + kTableEntries * 8;
-constexpr int kWarpSmemBytes = kRingBytes;                   // 28160
+constexpr int kWarpSmemBytes = 28160;                        // attention ring (24 KB) and group table, a multiple of 256
 constexpr int kFusedSmemBytes = kFWarps * kWarpSmemBytes;    // 225280: one CTA per SM
 constexpr long long kSpinLimit = 4000000;                    // x ~100 ns: bounded wait on another warp
 
-enum { PH_SCORE = 1, PH_ATTEND = 2 };
 constexpr int kWaves = 4;                                    // the units are scored in this many waves
-constexpr int kScoreRowGroup = 4;                            // FP4 factor rows decoded and multiplied together
-
-// Phase timing (the build with -DCOBS_TIMING, `python -m paper_2607_09052_b200.build --timing`, which makes
-// libcobs_timing.so; read by `bench.py --phase-times`): every streaming warp records the global timer at its phase
-// boundaries and accumulates clock cycles per category inside the phases; the selection teams record when a unit
-// was complete and when its selection was published.  The production library carries none of this.
-#ifdef COBS_TIMING
-__device__ unsigned long long g_dbg_times[4][4096];   // [start | scoring done | attention start | attention done][warp]
-__device__ unsigned long long g_dbg_acc[8][4096];     // accumulated clock cycles by category: attention [warp], scoring
-                                                      // [1200 + warp]; selection stamps (ns) [3000 + unit]
-__device__ __forceinline__ unsigned long long gtime() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-#define COBS_STAMP(k) do { if (lane == 0 && wg < 4096) g_dbg_times[k][wg] = gtime(); } while (0)
-#define COBS_SEL_STAMP(k) do { if (tid == 0 && u < 1024) g_dbg_acc[k][3000 + u] = gtime(); } while (0)
-#define COBS_ACC_DECL long long acc_t[8] = {0,0,0,0,0,0,0,0}; long long acc_last = clock64()
-#define COBS_ACC(k) do { long long now_ = clock64(); acc_t[k] += now_ - acc_last; acc_last = now_; } while (0)
-#define COBS_ACC_FLUSH(id) do { if ((threadIdx.x & 31) == 0 && (id) < 4096) { for (int k_ = 0; k_ < 8; ++k_) g_dbg_acc[k_][id] += acc_t[k_]; } } while (0)
-#else
-#define COBS_ACC_DECL do { } while (0)
-#define COBS_ACC(k) do { } while (0)
-#define COBS_ACC_FLUSH(id) do { } while (0)
-#define COBS_STAMP(k) do { } while (0)
-#define COBS_SEL_STAMP(k) do { } while (0)
-#endif
-
 
 // ---------------------------------------------------------------------------------------------------
-// small PTX helpers
+// waits on other warps of the grid
 // ---------------------------------------------------------------------------------------------------
-// The summaries and the selected K / V are read exactly once per step: their copies carry an L2 evict-first policy,
-// so that they do not push the step's small shared state (block scores, chunk pairs, selections, split partials,
-// flags: written by one warp, read by another a few microseconds later) out of L2 and into the HBM queues.
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(pol));
-  return pol;
-}
-__device__ __forceinline__ void cpa16(uint32_t dst, const void *src, uint64_t pol) {
-  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "l"(pol));
-}
-__device__ __forceinline__ void cpa16z(uint32_t dst, const void *src, int bytes, uint64_t pol) {
-  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;\n" ::"r"(dst), "l"(src), "r"(bytes), "l"(pol));
-}
-__device__ __forceinline__ void cpa4(uint32_t dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src));
-}
-__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t addr) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ void mma16816_bf16(float &c0, float &c1, float &c2, float &c3, uint32_t a0, uint32_t a1,
-                                              uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-               : "+f"(c0), "+f"(c1), "+f"(c2), "+f"(c3)
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma16816_f16(float &c0, float &c1, float &c2, float &c3, uint32_t a0, uint32_t a1,
-                                             uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-               : "+f"(c0), "+f"(c1), "+f"(c2), "+f"(c3)
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void ldsm_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
-// Eight E2M1 codes -> four f16x2 (code 2 i in the low half of h[i], code 2 i + 1 in the high half).
-__device__ __forceinline__ void e2m1x8_to_f16(uint32_t w, uint32_t (&h)[4]) {
-  asm("{\n .reg .b8 b0, b1, b2, b3;\n mov.b32 {b0, b1, b2, b3}, %4;\n cvt.rn.f16x2.e2m1x2 %0, b0;\n"
-      " cvt.rn.f16x2.e2m1x2 %1, b1;\n cvt.rn.f16x2.e2m1x2 %2, b2;\n cvt.rn.f16x2.e2m1x2 %3, b3;\n}\n"
-      : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]) : "r"(w));
-}
-__device__ __forceinline__ uint32_t f16x2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&h);
-}
-__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(addr));
-  return v;
-}
-// ---- mbarrier + bulk copy (global -> shared, completion counted in bytes on an mbarrier) -----------------
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar, uint64_t pol) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(pol) : "memory");
-}
-// Wait for the phase with the given parity to complete.  Bounded; false on expiry.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int it = 0; it < 20000000; ++it) {
-    uint32_t done;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
-  }
-  return false;
-}
 __device__ __forceinline__ int ld_volatile(const int *p) { return *reinterpret_cast<const volatile int *>(p); }
 
 // Wait until *flag != 0 (set by another warp of the grid).  Bounded; false on expiry.
@@ -365,7 +201,6 @@ __device__ void select_unit(const Params &p, int u, int n_sum, int n_cand, int t
     }
   }
   }
-  COBS_SEL_STAMP(2);
   if (real) team_sync();
   // ---- scores of this thread's blocks: score_b = sum_g t[g][b] * exp(part max[g] - lse_g) -----------------------
   if (real || part == 1) {
@@ -402,7 +237,6 @@ __device__ void select_unit(const Params &p, int u, int n_sum, int n_cand, int t
     keys[j] = (b < n_cand) ? __float_as_uint(sc[j]) : 0u;
   }
   }
-  COBS_SEL_STAMP(3);
   // ---- top-k ------------------------------------------------------------------------------------------------
   int32_t *out = p.sel_idx + (size_t)u * p.topk;
   const int k = min(p.topk, n_cand);
@@ -461,7 +295,6 @@ __device__ void select_unit(const Params &p, int u, int n_sum, int n_cand, int t
     if (na >= ku) theta = ta; else if (nb >= ku) theta = tb; else if (nc >= ku) theta = tc;
   }
   }
-  COBS_SEL_STAMP(4);
   if (real || part == 3) {
   // keep every key above theta and the lowest-index `need_eq` keys equal to it, in index order: one scan of the
   // packed (above, equal) counts gives both the totals and this thread's position
@@ -494,7 +327,6 @@ __device__ void select_unit(const Params &p, int u, int n_sum, int n_cand, int t
     }
   }
   }
-  COBS_SEL_STAMP(5);
 }
 
 // count_mult: how often the scoring path counts a chunk on its unit; empty_need: the count a unit without
@@ -530,7 +362,6 @@ __device__ void select_team(const Params &p, const int *seq_lens, int tid, int c
       team_sync();
       if (!ok) { u += gridDim.x; continue; }     // never scored: leave the unit unselected (its attention times out too)
       __threadfence();
-      COBS_SEL_STAMP(0);
     }
     const int part = rehearsal ? (tid >> 5) : -1;
     if (n_sum <= kSelThreads * 4) select_unit<PPC, 4>(p, u, n_sum, n_cand, tid, part);
@@ -541,482 +372,8 @@ __device__ void select_team(const Params &p, const int *seq_lens, int tid, int c
     __threadfence();
     team_sync();
     if (tid == 0) atomicExch(CTL_UNIT(p.ctl_ready) + u, 1);
-    COBS_SEL_STAMP(1);
     u += gridDim.x;
   }
-}
-
-// Curvature term of a 16-block chunk whose packed E2M1 rows are full width (128 codes: one 16-byte read per thread and
-// row) and whose rank R is a multiple of four: no clamps or row tests, four rows (four independent accumulator chains) at
-// a time, the four scales of a block read in one go.  xa / xb: this thread's 16 bytes of row 0 of blocks 2 gid and
-// 2 gid + 1 (rows 64 bytes apart); sp: the scales of block 2 gid (those of block 2 gid + 1 follow them).
-// Adds sum_i (scale_i * (xi_i . q))^2 per block and head; the query's per-head factor is applied by the caller.
-template <int R, bool SCALE_F32>
-__device__ __forceinline__ void fp4_rows_full_width(uint32_t xa, uint32_t xb, uint32_t sp, const uint32_t (&bq)[8][2], float &sA0,
-                                                    float &sA1, float &sB0, float &sB1) {
-  static_assert(R % 4 == 0, "whole groups of four rows");
-#pragma unroll 1                                 // rolled: half the code at rank 8 (instruction fetch is a visible stall of this kernel)
-  for (int i0 = 0; i0 < R; i0 += 4) {
-    uint4 wa[4], wb[4];
-    float d[4][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      wa[k] = lds128(xa + (i0 + k) * 64);
-      wb[k] = lds128(xb + (i0 + k) * 64);
-      d[k][0] = d[k][1] = d[k][2] = d[k][3] = 0.f;
-    }
-    float sa[4], sb[4];
-    if (SCALE_F32) {
-      const uint4 a = lds128(sp + i0 * 4), b = lds128(sp + R * 4 + i0 * 4);
-      sa[0] = __uint_as_float(a.x); sa[1] = __uint_as_float(a.y); sa[2] = __uint_as_float(a.z); sa[3] = __uint_as_float(a.w);
-      sb[0] = __uint_as_float(b.x); sb[1] = __uint_as_float(b.y); sb[2] = __uint_as_float(b.z); sb[3] = __uint_as_float(b.w);
-    } else {
-      const uint2 a = lds64(sp + i0 * 2), b = lds64(sp + R * 2 + i0 * 2);
-      const float2 a0 = __half22float2(*reinterpret_cast<const __half2 *>(&a.x)), a1 = __half22float2(*reinterpret_cast<const __half2 *>(&a.y));
-      const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&b.x)), b1 = __half22float2(*reinterpret_cast<const __half2 *>(&b.y));
-      sa[0] = a0.x; sa[1] = a0.y; sa[2] = a1.x; sa[3] = a1.y;
-      sb[0] = b0.x; sb[1] = b0.y; sb[2] = b1.x; sb[3] = b1.y;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        uint32_t ha[4], hb[4];
-        e2m1x8_to_f16(j == 0 ? wa[k].x : j == 1 ? wa[k].y : j == 2 ? wa[k].z : wa[k].w, ha);
-        e2m1x8_to_f16(j == 0 ? wb[k].x : j == 1 ? wb[k].y : j == 2 ? wb[k].z : wb[k].w, hb);
-        mma16816_f16(d[k][0], d[k][1], d[k][2], d[k][3], ha[0], hb[0], ha[1], hb[1], bq[2 * j][0], bq[2 * j][1]);
-        mma16816_f16(d[k][0], d[k][1], d[k][2], d[k][3], ha[2], hb[2], ha[3], hb[3], bq[2 * j + 1][0], bq[2 * j + 1][1]);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float d0 = d[k][0] * sa[k], d1 = d[k][1] * sa[k], d2 = d[k][2] * sb[k], d3 = d[k][3] * sb[k];
-      sA0 = fmaf(d0, d0, sA0); sA1 = fmaf(d1, d1, sA1); sB0 = fmaf(d2, d2, sB0); sB1 = fmaf(d3, d3, sB1);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------------
-// phase S: scoring (+ selection by the warp that completes a unit)
-// DT: COBS_SUMM_BF16 | COBS_SUMM_FP4_E2M1.  WPT: 32-bit words of codes per thread per FP4 row
-// (Ds_pad / 32).  NT: f16 terms of the query (1: full space, 2: fp32 subspace query).
-// ---------------------------------------------------------------------------------------------------
-// Returns false when a wait for this warp's own copies ran out (COBS_ERR_TIMEOUT is recorded): copies may then still
-// be on their way into the warp's ring, so the caller must not reuse it.
-template <int DT, int D, int WPT, int NT>
-__device__ bool score_phase(const Params &p, const int *seq_lens, unsigned char *wsm, uint64_t *bars, int wg, int n_wg,
-                            int lane) {
-  constexpr bool FP4 = (DT == COBS_SUMM_FP4_E2M1);
-  constexpr int MCH = D / 32;                 // 16-byte chunks of a bf16 row per thread
-  constexpr int KSM = D / 16;                 // k-steps of a bf16 row
-  constexpr int KSQ = FP4 ? WPT * 2 : 1;      // k-steps of an FP4 row
-  // stage layout: [16 block means, row stride MROW][16 blocks x rows of factors, block stride XS][scales]
-  // The +32 bytes of padding per row / block put the rows of neighbouring quads in different bank halves.
-  constexpr int MROW = D * 2 + 32;
-  constexpr int MEAN_BYTES = 16 * MROW;
-  constexpr int ROWB = FP4 ? WPT * 16 : D * 2;                 // bytes of one factor row
-  constexpr int ROWS_CAP = (kScoreStageBytes - 16 * 32) / (16 * ROWB);
-  constexpr int ROWS_MAX = ROWS_CAP < COBS_MAX_RANK ? ROWS_CAP : COBS_MAX_RANK;   // rows a batch can hold at most
-  static_assert((kScoreStageBytes - MEAN_BYTES - 16 * 32 - 16 * COBS_MAX_RANK * 4) / (16 * ROWB) >= 1, "stage too small");
-  const int gid = lane >> 2, tig = lane & 3;
-  const int G = p.G, r = p.r, NB = p.NB, L = p.L;
-  const int units = p.B * p.Hkv;
-  const int cpu = (NB + 15) / 16;             // chunks per unit
-  const int scale_sz = (p.scale_dtype == COBS_SCALE_FP16) ? 2 : 4;
-  const int scale_bytes = FP4 ? 16 * r * scale_sz : 0;        // scales of a chunk, at the end of the stage
-  // Common case: means, all r factor rows and scales of the 16 blocks fit one stage.  Then a chunk is three
-  // contiguous pieces of the summary arrays and is fetched by three bulk copies in memory layout (`single`).
-  // Otherwise the factor rows go in batches, each block copied on its own to a padded position.
-  const bool single = 16 * D * 2 + 16 * r * ROWB + scale_bytes <= kScoreStageBytes && r <= ROWS_MAX;
-  const int ROWS0 = single ? r : min(ROWS_MAX, (kScoreStageBytes - MEAN_BYTES - 16 * 32 - scale_bytes) / (16 * ROWB));
-  const int ROWSN = min(ROWS_MAX, (kScoreStageBytes - 16 * 32 - scale_bytes) / (16 * ROWB));
-  const int mrow = single ? D * 2 : MROW;                                  // row stride of the mean area
-  const int mean_bytes = 16 * mrow;
-  const int XS0 = single ? r * ROWB : ROWS0 * ROWB + 32, XSN = ROWSN * ROWB + 32;   // block stride of the factor area
-  const int n_batches = (r <= ROWS0) ? 1 : 1 + (r - ROWS0 + ROWSN - 1) / ROWSN;
-  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(wsm);
-  const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(bars);
-  const float inv_sqrt_d = 1.0f / sqrtf((float)D);
-  const float ln_l = (float)(31 - __clz(L)) * 0.6931471805599453f;      // L is a power of two
-
-  // Work order.  The units are scored in kWaves waves (first half, second half); within a wave every streaming
-  // warp takes one contiguous range of the wave's chunks (mostly one unit: its query fragments are built once, and
-  // its finished chunks are counted once).  The selection teams pick up a wave's units while the next wave is being
-  // scored - or, for the last wave, while the first wave's units are being attended.
-  // A position is (unit, chunk-in-unit, blocks of the unit); 32-bit arithmetic throughout.
-  auto unit_blocks = [&](int u) -> int { return min(seq_lens[u / p.Hkv] / L, NB); };
-  // waves only when there is enough work to keep every warp busy in each of them: with fewer chunks than warps a
-  // wave would serialise chunks on a few warps while the rest idle
-  const int n_waves = max(1, min(min(kWaves, units / 2), (units * cpu) / n_wg));
-  int wave = 0, c_end = 0;
-  auto wave_range = [&](int w, int &cb, int &ce) {          // this warp's chunk range [cb, ce) in wave w
-    const int u0 = (units * w) / n_waves, u1 = (units * (w + 1)) / n_waves;
-    const int tot = (u1 - u0) * cpu;                       // the host refuses configurations where this overflows
-    // ceil-sized ranges: at the benchmark's size this leaves the last 20 CTAs without scoring work; they start on the
-    // attention of the first selected units while the others still score.  Equal shares for every warp end the
-    // scoring 5 us earlier and the step 4 us later (measured, several forms): the warps then reach the attention
-    // phase together, before most selections are published, and move through it in lockstep.
-    const int per = (tot + n_wg - 1) / n_wg;
-    cb = u0 * cpu + min(wg * per, tot);
-    ce = u0 * cpu + min(wg * per + per, tot);
-  };
-  // first position at or after (u, ck) that holds work, moving on to the next wave's range when this one is
-  // exhausted; u = units when there is nothing left.  Chunk 0 of a unit without summarised blocks counts as work:
-  // its warp counts it, so that the selection sees the unit as scored.
-  auto seek = [&](int &u, int &ck, int &n_sum) {
-    for (;;) {
-      while (u < units && u * cpu + ck < c_end) {
-        if (ck * 16 < n_sum || ck == 0) return;
-        ++u; ck = 0;                           // rest of this unit has no summaries
-        if (u < units) n_sum = unit_blocks(u);
-      }
-      if (++wave >= n_waves) { u = units; return; }
-      int cb;
-      wave_range(wave, cb, c_end);
-      u = cb / cpu; ck = cb - u * cpu;
-      if (u < units) n_sum = unit_blocks(u);
-    }
-  };
-
-  COBS_ACC_DECL;
-  const uint64_t pol = l2_evict_first_policy();
-  // ---- bulk copies of (chunk c, batch b) into stage st; completion is counted on the stage's mbarrier ----
-  // lanes 0-15 copy the factor rows of block `lane`, lanes 16-31 the mean of block `lane - 16`, lane 0 the scales
-  auto issue = [&](int u, int ck, int n_sum, int b, int st) {
-    if (u >= units) return;
-    if (ck * 16 >= n_sum) return;
-    const int nblk = min(16, NB - ck * 16);
-    const size_t rec0 = (size_t)u * NB + ck * 16;
-    const int row0 = (b == 0) ? 0 : ROWS0 + (b - 1) * ROWSN;
-    const int rows = min(r - row0, (b == 0) ? ROWS0 : ROWSN);
-    const uint32_t sbase = ring + st * kScoreStageBytes;
-    const uint32_t xoff = (b == 0) ? mean_bytes : 0;
-    const uint32_t xs = (b == 0) ? XS0 : XSN;
-    const uint32_t soff = kScoreStageBytes - scale_bytes;
-    const bool scales_bulk = FP4 && nblk == 16 && r > 0;
-    const uint32_t bar = bar0 + st * 8;
-    if (lane == 0) {
-      uint32_t tx = (uint32_t)nblk * (uint32_t)(rows > 0 ? rows * ROWB : 0);
-      if (b == 0) tx += (uint32_t)nblk * (D * 2);
-      if (scales_bulk) tx += (uint32_t)(16 * r * scale_sz);
-      mbar_expect_tx(bar, tx);
-      if (single) {                            // the whole chunk: three contiguous pieces, one lane issues them
-        bulk_g2s(sbase, (const char *)p.mean + rec0 * (size_t)(D * 2), nblk * D * 2, bar, pol);
-        if (rows > 0) bulk_g2s(sbase + xoff, (const char *)p.xi + rec0 * r * (size_t)ROWB, nblk * r * ROWB, bar, pol);
-        if (scales_bulk) bulk_g2s(sbase + soff, (const char *)p.scale + rec0 * (size_t)(r * scale_sz), 16 * r * scale_sz, bar, pol);
-      }
-    }
-    COBS_ACC(5);
-    if (single) {
-      if (FP4 && r > 0 && !scales_bulk) {      // ragged last chunk of the array: plain loads, 4 bytes at a time
-        const char *ssrc = (const char *)p.scale + rec0 * (size_t)(r * scale_sz);
-        for (int w = lane * 4; w < nblk * r * scale_sz; w += 128)
-          *reinterpret_cast<uint32_t *>(wsm + st * kScoreStageBytes + soff + w) = *reinterpret_cast<const uint32_t *>(ssrc + w);
-      }
-      return;
-    }
-    __syncwarp();
-    if (lane < 16) {
-      if (lane < nblk && rows > 0)
-        bulk_g2s(sbase + xoff + lane * xs, (const char *)p.xi + ((rec0 + lane) * r + row0) * (size_t)ROWB, rows * ROWB, bar, pol);
-    } else if (b == 0 && lane - 16 < nblk) {
-      bulk_g2s(sbase + (lane - 16) * mrow, (const char *)p.mean + (rec0 + lane - 16) * (size_t)(D * 2), D * 2, bar, pol);
-    }
-    if (FP4 && r > 0) {
-      const char *ssrc = (const char *)p.scale + rec0 * (size_t)(r * scale_sz);
-      if (scales_bulk) {
-        if (lane == 2) bulk_g2s(sbase + soff, ssrc, 16 * r * scale_sz, bar, pol);
-      } else {                                // ragged last chunk of the array: plain loads, 4 bytes at a time
-        for (int w = lane * 4; w < nblk * r * scale_sz; w += 128)
-          *reinterpret_cast<uint32_t *>(wsm + st * kScoreStageBytes + soff + w) = *reinterpret_cast<const uint32_t *>(ssrc + w);
-      }
-    }
-  };
-
-  int cu, cck, cn = 0;                                        // current position and its unit's block count
-  {
-    int cb;
-    wave_range(0, cb, c_end);
-    cu = cb / cpu; cck = cb - cu * cpu;
-    if (cu < units) cn = unit_blocks(cu);
-    seek(cu, cck, cn);
-  }
-  int cur_b = 0, st = 0;
-  uint32_t phase_bits = 0;                  // bit st = parity to wait for on stage st
-  int pend_u = -1, pend_n = 0;              // chunks finished but not yet counted (counted once per unit run)
-  issue(cu, cck, cn, 0, 0);
-  // per-chunk state
-  uint32_t bm[KSM][2];
-  uint32_t bq[FP4 ? NT : 1][KSQ][2];
-  float m0 = 0.f, m1 = 0.f;
-  float fA0 = 0.f, fA1 = 0.f, fB0 = 0.f, fB1 = 0.f, sA0 = 0.f, sA1 = 0.f, sB0 = 0.f, sB1 = 0.f;
-  int cur_u = -1;
-  bool alive = true;
-
-  while (cu < units && alive) {
-    COBS_ACC(0);
-    // ---- prefetch the next batch of this warp --------------------------------------------------------
-    int nu = cu, nck = cck, nn = cn, nxt_b = cur_b + 1;
-    if (nxt_b >= n_batches) {
-      nxt_b = 0;
-      if (++nck >= cpu) { ++nu; nck = 0; if (nu < units) nn = unit_blocks(nu); }
-      seek(nu, nck, nn);
-    }
-    COBS_ACC(6);
-    issue(nu, nck, nn, nxt_b, st ^ 1);
-    COBS_ACC(1);
-
-    const int u = cu, ck = cck, n_sum = cn;
-    const uint32_t sbase = ring + st * kScoreStageBytes;
-    if (ck * 16 < n_sum) {
-      if (!mbar_wait(bar0 + st * 8, (phase_bits >> st) & 1u)) {     // bounded: the copies never landed
-        if (lane == 0) report(p.status, COBS_ERR_TIMEOUT);
-        alive = false;
-        break;
-      }
-      phase_bits ^= 1u << st;
-      __syncwarp();
-      COBS_ACC(2);
-        if (cur_b == 0) {
-        if (u != cur_u) {
-          cur_u = u;
-          const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;      // a division: once per unit, not per chunk
-          // ---- query fragments of this unit ------------------------------------------------------------
-          const __nv_bfloat16 *qg = p.q + ((size_t)b_idx * p.Hq + h * G) * D;
-#pragma unroll
-          for (int m = 0; m < KSM / 2; ++m) {
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (gid < G) v = *reinterpret_cast<const uint4 *>(qg + gid * D + (tig + 4 * m) * 8);
-            bm[2 * m][0] = v.x; bm[2 * m][1] = v.y; bm[2 * m + 1][0] = v.z; bm[2 * m + 1][1] = v.w;
-          }
-          if (FP4) {
-            // this thread's WPT * 8 query elements of head gid: the raw bf16 query (full space; the
-            // 1/sqrt(D) factor is applied to the tile result) or the prepared fp32 q~ (subspace)
-            float e[WPT][8];
-            float mx = 0.f;
-#pragma unroll
-            for (int j = 0; j < WPT; ++j) {
-              if (p.qtilde) {
-                const float4 *src = reinterpret_cast<const float4 *>(
-                    p.qtilde + ((size_t)b_idx * p.Hq + h * G + gid) * p.Ds_pad + tig * (WPT * 8) + j * 8);
-                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-                if (gid < G) { lo = __ldcg(src); hi = __ldcg(src + 1); }
-                e[j][0] = lo.x; e[j][1] = lo.y; e[j][2] = lo.z; e[j][3] = lo.w;
-                e[j][4] = hi.x; e[j][5] = hi.y; e[j][6] = hi.z; e[j][7] = hi.w;
-              } else {
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (gid < G) v = *reinterpret_cast<const uint4 *>(qg + gid * D + tig * (WPT * 8) + j * 8);
-                e[j][0] = bf16_lo(v.x); e[j][1] = bf16_hi(v.x); e[j][2] = bf16_lo(v.y); e[j][3] = bf16_hi(v.y);
-                e[j][4] = bf16_lo(v.z); e[j][5] = bf16_hi(v.z); e[j][6] = bf16_lo(v.w); e[j][7] = bf16_hi(v.w);
-              }
-#pragma unroll
-              for (int n = 0; n < 8; ++n) mx = fmaxf(mx, fabsf(e[j][n]));
-            }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            // mx in [2^(ex-1), 2^ex), from its exponent field (clamped: an all-zero or absurdly large query keeps
-            // the powers of two below in range)
-            const int ex = (int)(__float_as_uint(fminf(fmaxf(mx, 1e-30f), 1e30f)) >> 23) - 126;
-            const float inv_s = __uint_as_float((uint32_t)(128 - ex) << 23);       // 2^(1-ex): brings max |q| into [1, 2)
-            const float mult = __uint_as_float((uint32_t)(126 + ex) << 23) * (p.qtilde ? 1.0f : inv_sqrt_d);
-#pragma unroll
-            for (int j = 0; j < WPT; ++j) {
-#pragma unroll
-              for (int t = 0; t < NT; ++t) {
-                float hi[8];
-#pragma unroll
-                for (int n = 0; n < 8; ++n) {
-                  const float x = (t == 0) ? e[j][n] * inv_s : e[j][n];
-                  hi[n] = __half2float(__float2half_rn(x));
-                  e[j][n] = x - hi[n];
-                }
-                bq[t][2 * j][0] = f16x2(hi[0], hi[1]); bq[t][2 * j][1] = f16x2(hi[2], hi[3]);
-                bq[t][2 * j + 1][0] = f16x2(hi[4], hi[5]); bq[t][2 * j + 1][1] = f16x2(hi[6], hi[7]);
-              }
-            }
-            // result columns 2 tig, 2 tig + 1 are heads whose factor sits in the lanes gid = 2 tig, 2 tig + 1
-            m0 = __shfl_sync(0xffffffffu, mult, (2 * tig) * 4);
-            m1 = __shfl_sync(0xffffffffu, mult, (2 * tig + 1) * 4);
-          }
-        }
-            // ---- first-order term: block means against the raw bf16 query ------------------------------------
-        float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f, e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;   // two chains
-        const uint32_t ma = sbase + (2 * gid) * mrow + tig * 16, mb = ma + mrow;
-#pragma unroll
-        for (int m = 0; m < MCH; ++m) {
-          const uint4 va = lds128(ma + m * 64), vb = lds128(mb + m * 64);
-          mma16816_bf16(c0, c1, c2, c3, va.x, vb.x, va.y, vb.y, bm[2 * m][0], bm[2 * m][1]);
-          mma16816_bf16(e0, e1, e2, e3, va.z, vb.z, va.w, vb.w, bm[2 * m + 1][0], bm[2 * m + 1][1]);
-        }
-        fA0 = (c0 + e0) * inv_sqrt_d; fA1 = (c1 + e1) * inv_sqrt_d;
-        fB0 = (c2 + e2) * inv_sqrt_d; fB1 = (c3 + e3) * inv_sqrt_d;
-        sA0 = sA1 = sB0 = sB1 = 0.f;
-      }
-      // ---- curvature term: rows of this batch ----------------------------------------------------------
-      const int row0 = (cur_b == 0) ? 0 : ROWS0 + (cur_b - 1) * ROWSN;
-      const int rows = min(r - row0, (cur_b == 0) ? ROWS0 : ROWSN);
-      const uint32_t xs = (cur_b == 0) ? XS0 : XSN;
-      const uint32_t xa = sbase + ((cur_b == 0) ? mean_bytes : 0) + (2 * gid) * xs + tig * (FP4 ? WPT * 4 : 16), xb = xa + xs;
-      bool rows_done = false;
-      if constexpr (FP4 && WPT == 4 && NT == 1) {
-        // the benchmark's descriptors (full key space, rank 4 or 8, the whole chunk in one stage): straight-line code
-        if (single && (r == 8 || r == 4)) {
-          const uint32_t spa = sbase + (kScoreStageBytes - scale_bytes) + (2 * gid) * r * scale_sz;
-          if (r == 8) {
-            if (scale_sz == 4) fp4_rows_full_width<8, true>(xa, xb, spa, bq[0], sA0, sA1, sB0, sB1);
-            else fp4_rows_full_width<8, false>(xa, xb, spa, bq[0], sA0, sA1, sB0, sB1);
-          } else {
-            if (scale_sz == 4) fp4_rows_full_width<4, true>(xa, xb, spa, bq[0], sA0, sA1, sB0, sB1);
-            else fp4_rows_full_width<4, false>(xa, xb, spa, bq[0], sA0, sA1, sB0, sB1);
-          }
-          rows_done = true;
-        }
-      }
-      if (rows_done) {
-      } else if (FP4) {
-        // RG factor rows at a time: RG independent accumulator chains keep the tensor pipe busy
-        constexpr int RG = kScoreRowGroup;
-        const unsigned char *sp = wsm + st * kScoreStageBytes + (kScoreStageBytes - scale_bytes) + (2 * gid) * r * scale_sz;
-#pragma unroll 1
-        for (int i0 = 0; i0 < ROWS_MAX; i0 += RG) {
-          if (i0 < rows) {
-            float d[RG][4];
-            uint32_t wa[RG][4], wb[RG][4];
-#pragma unroll
-            for (int k = 0; k < RG; ++k) {
-              // neighbouring quads walk the group's rows in a rotated order (their rows then sit in different
-              // bank halves); a row past the end of the batch is read from the last row and weighted by zero
-              const int i = min(i0 + ((k + gid) & (RG - 1)), rows - 1);
-              if (WPT == 4) {
-                const uint4 a = lds128(xa + i * ROWB), bb = lds128(xb + i * ROWB);
-                wa[k][0] = a.x; wa[k][1] = a.y; wa[k][2] = a.z; wa[k][3] = a.w;
-                wb[k][0] = bb.x; wb[k][1] = bb.y; wb[k][2] = bb.z; wb[k][3] = bb.w;
-              } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  wa[k][j] = (j < WPT) ? lds_u32(xa + i * ROWB + j * 4) : 0u;
-                  wb[k][j] = (j < WPT) ? lds_u32(xb + i * ROWB + j * 4) : 0u;
-                }
-              }
-              d[k][0] = d[k][1] = d[k][2] = d[k][3] = 0.f;
-            }
-#pragma unroll
-            for (int j = 0; j < WPT; ++j) {
-#pragma unroll
-              for (int k = 0; k < RG; ++k) {
-                uint32_t ha[4], hb[4];
-                e2m1x8_to_f16(wa[k][j], ha);
-                e2m1x8_to_f16(wb[k][j], hb);
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                  mma16816_f16(d[k][0], d[k][1], d[k][2], d[k][3], ha[0], hb[0], ha[1], hb[1], bq[t][2 * j][0], bq[t][2 * j][1]);
-                  mma16816_f16(d[k][0], d[k][1], d[k][2], d[k][3], ha[2], hb[2], ha[3], hb[3], bq[t][2 * j + 1][0],
-                               bq[t][2 * j + 1][1]);
-                }
-              }
-            }
-            // scales of this lane's rows of the group (clamped like the rows themselves; a row past the end weighs
-            // zero).  The per-head query factors m0, m1 are applied once per chunk, to the sums of squares.
-            auto accumulate = [&](auto f32) {
-#pragma unroll
-              for (int k = 0; k < RG; ++k) {
-                const int io = i0 + ((k + gid) & (RG - 1));
-                const int ri = row0 + min(io, rows - 1);
-                float sa, sb;
-                if (decltype(f32)::value) {
-                  sa = reinterpret_cast<const float *>(sp)[ri];
-                  sb = reinterpret_cast<const float *>(sp)[r + ri];
-                } else {
-                  sa = __half2float(reinterpret_cast<const __half *>(sp)[ri]);
-                  sb = __half2float(reinterpret_cast<const __half *>(sp)[r + ri]);
-                }
-                if (io >= rows) { sa = 0.f; sb = 0.f; }
-                const float d0 = d[k][0] * sa, d1 = d[k][1] * sa, d2 = d[k][2] * sb, d3 = d[k][3] * sb;
-                sA0 = fmaf(d0, d0, sA0); sA1 = fmaf(d1, d1, sA1); sB0 = fmaf(d2, d2, sB0); sB1 = fmaf(d3, d3, sB1);
-              }
-            };
-            if (scale_sz == 4) accumulate(std::true_type{}); else accumulate(std::false_type{});
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < ROWS_MAX; ++i) {
-          if (i < rows) {
-            float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
-#pragma unroll
-            for (int m = 0; m < MCH; ++m) {
-              const uint4 va = lds128(xa + i * ROWB + m * 64), vb = lds128(xb + i * ROWB + m * 64);
-              mma16816_bf16(d0, d1, d2, d3, va.x, vb.x, va.y, vb.y, bm[2 * m][0], bm[2 * m][1]);
-              mma16816_bf16(d0, d1, d2, d3, va.z, vb.z, va.w, vb.w, bm[2 * m + 1][0], bm[2 * m + 1][1]);
-            }
-            d0 *= inv_sqrt_d; d1 *= inv_sqrt_d; d2 *= inv_sqrt_d; d3 *= inv_sqrt_d;
-            sA0 = fmaf(d0, d0, sA0); sA1 = fmaf(d1, d1, sA1); sB0 = fmaf(d2, d2, sB0); sB1 = fmaf(d3, d3, sB1);
-          }
-        }
-      }
-    }
-
-    COBS_ACC(3);
-    // ---- end of a chunk: publish t = exp(e - chunk max) per block and the chunk's (max, sum of t) per head ----
-    if (cur_b == n_batches - 1) {
-      if (pend_u != u && pend_n > 0) {       // moving on to another unit: count the finished one's chunks
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) atomicAdd(CTL_UNIT(p.ctl_score) + pend_u, pend_n);
-        pend_n = 0;
-        COBS_ACC(7);
-      }
-      pend_u = u;
-      if (ck * 16 < n_sum) {
-        const int bA = ck * 16 + 2 * gid, bB = bA + 1, g0 = 2 * tig, g1 = g0 + 1;
-        // 1/2 of the sums of squared projections; for FP4 the squares still lack the query's per-head factor
-        const float h0 = FP4 ? 0.5f * m0 * m0 : 0.5f, h1 = FP4 ? 0.5f * m1 * m1 : 0.5f;
-        const float eA0 = (bA < n_sum) ? ln_l + fA0 + h0 * sA0 : -INFINITY;
-        const float eB0 = (bB < n_sum) ? ln_l + fB0 + h0 * sB0 : -INFINITY;
-        const float eA1 = (bA < n_sum) ? ln_l + fA1 + h1 * sA1 : -INFINITY;
-        const float eB1 = (bB < n_sum) ? ln_l + fB1 + h1 * sB1 : -INFINITY;
-        // max over the chunk's 16 blocks (over gid), per head
-        float mx0 = fmaxf(eA0, eB0), mx1 = fmaxf(eA1, eB1);
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
-          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
-        }
-        const float tA0 = __expf(eA0 - mx0), tB0 = __expf(eB0 - mx0), tA1 = __expf(eA1 - mx1), tB1 = __expf(eB1 - mx1);
-        float *e0 = p.e + ((size_t)u * G + g0) * NB, *e1 = p.e + ((size_t)u * G + g1) * NB;
-        // blocks bA (even) and bA + 1 are neighbours in memory: one 8-byte store when both exist
-        if (bB < n_sum) {
-          if (g0 < G) __stcg(reinterpret_cast<float2 *>(e0 + bA), make_float2(tA0, tB0));
-          if (g1 < G) __stcg(reinterpret_cast<float2 *>(e1 + bA), make_float2(tA1, tB1));
-        } else if (bA < n_sum) {
-          if (g0 < G) __stcg(e0 + bA, tA0);
-          if (g1 < G) __stcg(e1 + bA, tA1);
-        }
-        float sm0 = tA0 + tB0, sm1 = tA1 + tB1;
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-          sm0 += __shfl_xor_sync(0xffffffffu, sm0, o);
-          sm1 += __shfl_xor_sync(0xffffffffu, sm1, o);
-        }
-        if (gid == 0) {
-          if (g0 < G) __stcg(reinterpret_cast<float2 *>(p.lse_part) + ((size_t)u * G + g0) * cpu + ck, make_float2(mx0, sm0));
-          if (g1 < G) __stcg(reinterpret_cast<float2 *>(p.lse_part) + ((size_t)u * G + g1) * cpu + ck, make_float2(mx1, sm1));
-        }
-      }
-      ++pend_n;
-    }
-    __syncwarp();                           // all lanes are done with stage st before it is refilled
-    COBS_ACC(4);
-    cu = nu; cck = nck; cn = nn; cur_b = nxt_b; st ^= 1;
-  }
-  if (pend_n > 0) {
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) atomicAdd(CTL_UNIT(p.ctl_score) + pend_u, pend_n);
-  }
-  COBS_ACC(0);
-  COBS_ACC_FLUSH(1200 + wg);
-  return alive;
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1058,7 +415,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
   // items are handed out in unit order from a global counter: a warp that arrives late simply takes fewer
   const int n_items = units * n_splits;
   const uint64_t pol = l2_evict_first_policy();
-  COBS_ACC_DECL;
 
   // Closing an item = making its partial visible, counting it, and merging the unit if it was the last slice.
   // (Drawing the next item before this one is closed was measured and is slower: a warp that turns out to be the
@@ -1069,7 +425,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
     int last = 0;
     if (lane == 0) last = (atomicAdd(CTL_UNIT(p.ctl_att) + u, 1) + 1 == n_splits);
     last = __shfl_sync(0xffffffffu, last, 0);
-    COBS_ACC(5);
     if (!last) return;
     // ---- merge the unit's partials: o = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s -------------------
     // A slice is [G][D] accumulators followed by [G] (max, sum) pairs.  Few round trips: all pairs at once, then the
@@ -1162,7 +517,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
   if (lane == 0) item = atomicAdd(CTL_MISC(p.ctl_item), 1);
   item = __shfl_sync(0xffffffffu, item, 0);
   for (;;) {
-    COBS_ACC(0);
     if (item >= n_items) break;
     const int u = item / n_splits, split = item - u * n_splits;
     const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
@@ -1188,7 +542,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
       }
     }
     bool ok = true;
-    COBS_ACC(1);
     if (g0 < n_sel * gpb && n_groups > 0) {
       if (wait_select) {
         ok = wait_flag(CTL_UNIT(p.ctl_ready) + u);
@@ -1198,7 +551,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
         n_sel = min(n_sel, min(__ldcg(p.sel_cnt + u), p.topk));
       }
     }
-    COBS_ACC(2);
     // ---- table of this item's groups -----------------------------------------------------------------
     __syncwarp();
     for (int g = lane; g < n_groups; g += 32) {
@@ -1254,8 +606,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
       }
       cpa_commit();
     };
-
-    COBS_ACC(3);
     issue(0, 0);
     issue(1, 1);
     int st = 0, st2 = 2;
@@ -1316,7 +666,6 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
       st2 = (st2 == kAttStages - 1) ? 0 : st2 + 1;
     }
     cpa_wait<0>();
-    COBS_ACC(4);
 
     // ---- this warp's partial: [G][D] acc, then [G] (running max in natural log units, running sum) ---------
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
@@ -1331,13 +680,10 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
                make_float2((l_run > 0.f) ? m_run * (sl2 * 0.6931471805599453f) : -INFINITY, l_run));
     }
     close_item(u);
-    COBS_ACC(7);
     int next_item = 0;
     if (lane == 0) next_item = atomicAdd(CTL_MISC(p.ctl_item), 1);
     item = __shfl_sync(0xffffffffu, next_item, 0);
-    COBS_ACC(6);
   }
-  COBS_ACC_FLUSH(wg);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1493,7 +839,6 @@ __device__ void umma_producer(const Params &p, const int *seq_lens, const UmmaLi
   const uint32_t scale_bytes = kUBlocks * 8 * scale_sz;
   const uint32_t sm = (uint32_t)__cvta_generic_to_shared(fsm);
   int w = 0, o = lane;
-  COBS_ACC_DECL;
   for (int k = 0;; ++k) {
     while (w < l.n_waves && o >= l.len[w]) { o -= l.len[w]; ++w; }
     const int slot = (lane & (kUAccBufs - 1)) + kUAccBufs * (k & 1);
@@ -1508,16 +853,13 @@ __device__ void umma_producer(const Params &p, const int *seq_lens, const UmmaLi
       valid = ck * kUBlocks < n_sum;
       tile = l.tile0[w] + (u - l.start[w] / cpu);
     }
-    COBS_ACC(0);
     bool ok = true;
     if (has && k > 1) ok = mbar_wait_lim(bars + (kBEmpty + slot) * 8, ((k >> 1) - 1) & 1);
     if (!__all_sync(0xffffffffu, ok)) { umma_abort(p, abort_flag, lane); break; }
-    COBS_ACC(1);
     if (has) *reinterpret_cast<int4 *>(fsm + slot * kUStageBytes + kUHdrOff) = make_int4(u, ck, n_sum, (valid ? 1 : 0) | (tile << 8));
     __syncwarp();
     const unsigned hm = __ballot_sync(0xffffffffu, has), vm = __ballot_sync(0xffffffffu, valid);
     const uint32_t rec0 = (uint32_t)(u * NB + ck * kUBlocks);    // < 2^28 (checked on the host)
-    COBS_ACC(2);
 #pragma unroll
     for (int sl = 0; sl < kUAccBufs; ++sl) {
       const uint32_t rec = __shfl_sync(0xffffffffu, rec0, sl);
@@ -1535,10 +877,8 @@ __device__ void umma_producer(const Params &p, const int *seq_lens, const UmmaLi
         }
       }
     }
-    COBS_ACC(3);
     o += kUAccBufs;
   }
-  COBS_ACC_FLUSH((int)blockIdx.x);
 }
 
 // MMA issuer warp.  Lane a < kUAccBufs waits for and decodes the list positions a, a + kUAccBufs, ... (accumulator
@@ -1548,7 +888,6 @@ __device__ void umma_issuer(const Params &p, const UmmaList &l, unsigned char *f
                             volatile int *abort_flag) {
   const uint64_t desc0 = umma_desc((uint32_t)__cvta_generic_to_shared(fsm));   // the whole region lies below 2^18
   int n = lane;
-  COBS_ACC_DECL;
   if (!mbar_wait_lim(bars + kBTiles * 8, 0)) { umma_abort(p, abort_flag, lane); return; }
   for (int k = 0;; ++k) {
     const int slot = (lane & (kUAccBufs - 1)) + kUAccBufs * (k & 1), fpar = (k >> 1) & 1;
@@ -1556,16 +895,13 @@ __device__ void umma_issuer(const Params &p, const UmmaList &l, unsigned char *f
     if (!__any_sync(0xffffffffu, has) || *abort_flag) break;
     bool ok = true;
     int4 hdr = make_int4(0, 0, 0, 0);
-    COBS_ACC(0);
     if (has) {
       ok = mbar_wait_lim(bars + (kBFull + slot) * 8, fpar);
       hdr = *reinterpret_cast<const int4 *>(fsm + slot * kUStageBytes + kUHdrOff);
     }
-    COBS_ACC(1);
     const bool valid = has && (hdr.w & 1);
     const int tile = (hdr.w >> 8) & 0xff;
     if (has && ok && k > 0) ok = mbar_wait_lim(bars + (kBTEmpty + lane) * 8, (k - 1) & 1);
-    COBS_ACC(2);
     if (!__all_sync(0xffffffffu, ok)) { umma_abort(p, abort_flag, lane); break; }
     tc_fence_after();
     const unsigned hm = __ballot_sync(0xffffffffu, has), vm = __ballot_sync(0xffffffffu, valid);
@@ -1594,10 +930,8 @@ __device__ void umma_issuer(const Params &p, const UmmaList &l, unsigned char *f
         }
       }
     }
-    COBS_ACC(3);
     n += kUAccBufs;
   }
-  COBS_ACC_FLUSH(200 + (int)blockIdx.x);
 }
 
 // Epilogue warp (streaming warps 0-7; set = warp / 4 takes the list positions of its parity, warp mod 4 = TMEM lane
@@ -1626,15 +960,12 @@ __device__ void umma_epilogue(const Params &p, const UmmaList &l, unsigned char 
       pend_n = 0;
     }
   };
-  COBS_ACC_DECL;
   if (!mbar_wait_lim(bars + kBTiles * 8, 0)) { umma_abort(p, abort_flag, lane); return; }
   for (int n = set, j = 0; n < l.total; n += 2, ++j) {
     if (*abort_flag) break;
     const int slot = n & (kUStages - 1), fpar = (n / kUStages) & 1, tfpar = j & 1;
     const uint32_t bar_empty = bars + (kBEmpty + slot) * 8, bar_tfull = bars + (kBTFull + set) * 8, bar_tempty = bars + (kBTEmpty + set) * 8;
-    COBS_ACC(0);
     if (!mbar_wait_lim(bars + (kBFull + slot) * 8, fpar)) { umma_abort(p, abort_flag, lane); break; }
-    COBS_ACC(1);
     const unsigned char *stg = fsm + slot * kUStageBytes;
     const int4 hdr = *reinterpret_cast<const int4 *>(stg + kUHdrOff);
     const int u = hdr.x, ck = hdr.y, n_sum = hdr.z;
@@ -1659,7 +990,6 @@ __device__ void umma_epilogue(const Params &p, const UmmaList &l, unsigned char 
       const float fac = (i < G) ? reinterpret_cast<const float *>(fsm + kUFacOff)[tile * 8 + i] : 0.f;
       fac2 = fac * fac;
     }
-    COBS_ACC(2);
     // ---- first-order term: rows 0-3 of an m16n8k16 tile = blocks 4 q .. of half 0, rows 8-11 = those of half 1 -----
     float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f, e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
     {
@@ -1681,10 +1011,8 @@ __device__ void umma_epilogue(const Params &p, const UmmaList &l, unsigned char 
       sc[hf] = scale_f16 ? __half2float(reinterpret_cast<const __half *>(stg + kUScaleOff)[srow])
                          : reinterpret_cast<const float *>(stg + kUScaleOff)[srow];
     }
-    COBS_ACC(3);
     // ---- the stage's products from tensor memory ----------------------------------------------------------------
     if (!mbar_wait_lim(bar_tfull, tfpar)) { umma_abort(p, abort_flag, lane); break; }
-    COBS_ACC(4);
     tc_fence_after();
     uint32_t r[32];
     {
@@ -1741,124 +1069,16 @@ __device__ void umma_epilogue(const Params &p, const UmmaList &l, unsigned char 
       if (bl == 0 && i < G && (2 * ck + hf) * 16 < n_sum)
         __stcg(reinterpret_cast<float2 *>(p.lse_part) + (((size_t)u * G + i) * cpu16 + 2 * ck + hf) * 4 + q, make_float2(wm, ws));
     }
-    COBS_ACC(5);
     if (pend_u != u) flush();
     pend_u = u;
     pend_n += 1 + (((2 * ck + 1) * 16 < n_sum) ? 1 : 0);
-    COBS_ACC(6);
   }
   flush();
-  COBS_ACC_FLUSH(400 + (int)blockIdx.x * 8 + warp);
-}
-
-// ---------------------------------------------------------------------------------------------------
-// Prologue of the subspace descriptor: q~ = U_Q^T (q / sqrt(D)) for every query head, zero padded to Ds_pad - the
-// one O(s D) projection per step and head that the scoring then shares across all blocks (Method, "Per-step
-// scoring").  Teams of four warps take (head, 32 consecutive subspace coordinates) tasks: lane = coordinate, so the
-// reads of U_Q [Hkv][D][Ds] are coalesced; each warp sums a quarter of the head dimension (all its loads in flight at
-// once) and the quarters are added in a fixed order.  The result goes to the workspace; a grid barrier (the launch
-// is cooperative, so every CTA is resident) makes it visible before any warp scores.
-// ---------------------------------------------------------------------------------------------------
-__device__ void project_queries(const Params &p) {
-  __shared__ float s_part[16][32];                // partial sums of the CTA's warps (at most 16 warps)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int teams = (int)(blockDim.x >> 5) / 4;   // four warps share a task: each sums a quarter of the head dimension
-  const int team = warp >> 2, quarter = warp & 3;
-  const int nsb = p.Ds_pad / 32, n_tasks = p.B * p.Hq * nsb;
-  const int dq = p.D / 4;                         // 32 or 16 coordinates per quarter: all their loads fly together
-  const float inv_sqrt_d = 1.0f / sqrtf((float)p.D);
-  for (int base = blockIdx.x * teams; base < n_tasks; base += gridDim.x * teams) {
-    const int t = base + team;
-    const bool active = team < teams && t < n_tasks;
-    float v = 0.f;
-    int bh = 0, sidx = 0;
-    if (active) {
-      bh = t / nsb;
-      const int sb = t - bh * nsb, hq = bh % p.Hq, h = hq / p.G;
-      sidx = sb * 32 + lane;
-      const float qv = (lane < dq) ? __bfloat162float(p.q[(size_t)bh * p.D + quarter * dq + lane]) * inv_sqrt_d : 0.f;
-      const bool live = sidx < p.Ds;              // padding coordinates take part in the shuffles and end as 0
-      const float *uq = p.u_q + ((size_t)h * p.D + quarter * dq) * p.Ds + (live ? sidx : 0);
-      float x[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) x[j] = (live && j < dq) ? __ldg(uq + (size_t)j * p.Ds) : 0.f;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v = fmaf(x[j], __shfl_sync(0xffffffffu, qv, j), v);
-    }
-    if (warp < 16) s_part[warp][lane] = v;
-    __syncthreads();
-    if (active && quarter == 0)                   // fixed order: the same bits every time
-      __stcg(p.qtilde_out + (size_t)bh * p.Ds_pad + sidx,
-             ((s_part[warp][lane] + s_part[warp + 1][lane]) + s_part[warp + 2][lane]) + s_part[warp + 3][lane]);
-    __syncthreads();
-  }
-}
-
-// Every CTA of the (cooperatively launched, hence fully resident) grid has arrived and its writes are visible.
-// Bounded: on expiry COBS_ERR_TIMEOUT is recorded and the caller goes on (its results are then undefined).
-__device__ void grid_barrier(const Params &p) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(CTL_MISC(p.ctl_bar), 1);
-    bool ok = false;
-    for (long long it = 0; it < kSpinLimit; ++it) {
-      if (ld_volatile(CTL_MISC(p.ctl_bar)) >= (int)gridDim.x) { ok = true; break; }
-      __nanosleep(50);
-    }
-    if (!ok) report(p.status, COBS_ERR_TIMEOUT);
-    __threadfence();
-  }
-  __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------------------------------
-template <int DT, int D, int WPT, int NT>
-__global__ void __launch_bounds__(kFThreads, 1) fused_step_kernel(Params p, int phases) {
-  extern __shared__ __align__(256) unsigned char fsm[];
-  __shared__ __align__(8) uint64_t s_bars[kFWarps][2];     // one mbarrier per scoring stage per streaming warp
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * kFWarps + warp, n_wg = gridDim.x * kFWarps;
-  // sequence lengths are consulted at every change of unit: keep them in shared memory when they fit
-  __shared__ int s_len[kLenCache];
-  const int *seq_lens = p.seq_lens;
-  if (threadIdx.x == 0) ctl_begin(p);          // (its round trip overlaps the loads of the lengths)
-  if (p.B <= kLenCache) {
-    for (int i = threadIdx.x; i < p.B; i += kFThreads) s_len[i] = p.seq_lens[i];
-    seq_lens = s_len;
-  }
-  __syncthreads();
-  if (s_ctl[2]) ctl_turn(p);
-  if ((phases & PH_SCORE) && p.u_q) {
-    project_queries(p);
-    grid_barrier(p);
-  }
-  if (warp < kFWarps) {
-    // ---- streaming warps: score their chunks, then attend their items -------------------------------------
-    unsigned char *wsm = fsm + warp * kWarpSmemBytes;
-    if (lane == 0) {
-      mbar_init((uint32_t)__cvta_generic_to_shared(&s_bars[warp][0]), 1);
-      mbar_init((uint32_t)__cvta_generic_to_shared(&s_bars[warp][1]), 1);
-      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    __syncwarp();
-    COBS_STAMP(0);
-    bool ring_free = true;
-    if (phases & PH_SCORE) ring_free = score_phase<DT, D, WPT, NT>(p, seq_lens, wsm, &s_bars[warp][0], wg, n_wg, lane);
-    COBS_STAMP(1);
-    COBS_STAMP(2);
-    // after a timeout in scoring the step's outputs are undefined; this warp leaves its items to the others
-    if ((phases & PH_ATTEND) && ring_free) attend_phase<D>(p, seq_lens, wsm, wg, n_wg, lane, (phases & PH_SCORE) != 0);
-    COBS_STAMP(3);
-  } else if (phases & PH_SCORE) {
-    // ---- selection team ----------------------------------------------------------------------------------------
-    select_team<1>(p, seq_lens, (int)threadIdx.x - kFWarps * 32, 1, 1);
-  }
-  // (nothing to clean up: the next launch works on the other set of counters, see ctl_begin)
-}
-
 // The step with phase S on tcgen05 (packed E2M1, full key space, D = 128, r = 8); phases must include PH_SCORE.
 __global__ void __launch_bounds__(kUThreads, 1) fused_step_umma_kernel(Params p, int phases, const __grid_constant__ CUtensorMap tmap_xi) {
   extern __shared__ unsigned char fsm_raw[];
@@ -1897,14 +1117,10 @@ __global__ void __launch_bounds__(kUThreads, 1) fused_step_umma_kernel(Params p,
   const uint32_t tmem = s_tmem;
   volatile int *abort_flag = &s_abort;
   if (warp < kFWarps) {
-    COBS_STAMP(0);
     umma_epilogue(p, s_list, fsm, bars, tmem, warp, lane, abort_flag);
-    COBS_STAMP(1);
     // every streaming warp is done with the scoring stages before any of them reuses the memory for attention
     asm volatile("bar.sync 4, %0;\n" ::"n"(kFWarps * 32) : "memory");
-    COBS_STAMP(2);
     if (phases & PH_ATTEND) attend_phase<128>(p, seq_lens, fsm + warp * kWarpSmemBytes, wg, n_wg, lane, true);
-    COBS_STAMP(3);
   } else if (warp < kFWarps + kSelWarps) {
     umma_build_tiles(p, s_list, fsm, bars, warp - kFWarps, lane);
     select_team<4>(p, seq_lens, (int)threadIdx.x - kFWarps * 32, 4, 0);
@@ -1925,55 +1141,18 @@ __global__ void __launch_bounds__(kUThreads, 1) fused_step_umma_kernel(Params p,
 // ---------------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------------
-template <int DT, int D, int WPT, int NT>
-static cudaError_t launch_fused_t(Params p, int phases, cudaStream_t stream) {
-  auto kern = fused_step_kernel<DT, D, WPT, NT>;
-  static int grid_cache[64] = {0};             // resident grid size of this instantiation, per device
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (grid_cache[dev] == 0) {
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmemBytes)) != cudaSuccess) return e;
-    int sms = 0, occ = 0;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kFThreads, kFusedSmemBytes)) != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorLaunchOutOfResources;
-    grid_cache[dev] = sms * occ;
-  }
-  void *args[] = {&p, &phases};
-  // cooperative launch: the grid is resident as a whole (or the launch fails), which the cross-warp waits rely on
-  e = cudaLaunchCooperativeKernel((const void *)kern, dim3(grid_cache[dev]), dim3(kFThreads), args, kFusedSmemBytes,
-                                  stream);
-  count_launch();
-  return e;
-}
-
-// Whether the persistent kernel covers this configuration's scoring phase.
-bool fused_score_supported(const Params &p) {
-  if (p.skew) return false;                                     // the third-cumulant variant is scored by the generic kernel
-  if (p.NB > kSelThreads * 16 || p.NB % 4 != 0) return false;   // the selection team holds at most 16 blocks per thread
-  if (p.summ_dtype == COBS_SUMM_BF16) return p.u_q == nullptr;
-  if (p.summ_dtype == COBS_SUMM_FP4_E2M1) {
-    if (p.Ds_pad % 32 != 0) return false;
-    const int scale_sz = (p.scale_dtype == COBS_SCALE_FP16) ? 2 : 4;
-    if ((p.r * scale_sz) % 4 != 0) return false;
-    return true;
-  }
-  return false;
-}
-
-// The tcgen05 scoring path is parity-tested but, as measured, not faster than the mma.sync path (its unpacked
-// 4-bit rows take twice the shared memory per byte in flight, which halves the copy depth of a bandwidth-bound
-// stream), so it is opt-in: environment variable COBS_SCORE_PATH=tcgen05, read at every call.
+// The tcgen05 scoring path is parity-tested but, as measured, slower than mma.sync scoring (its unpacked 4-bit rows take
+// twice the shared memory per byte in flight, which halves the copy depth of a bandwidth-bound stream: 157 us for sixteen
+// sequences of 128k, 98 by default), so it is opt-in: environment variable COBS_SCORE_PATH=tcgen05, read at every call.
 static bool umma_requested() {
   const char *v = getenv("COBS_SCORE_PATH");
   return v != nullptr && strcmp(v, "tcgen05") == 0;
 }
 
 // Whether phase S of this configuration runs on tcgen05 (see the section on it above).
-static bool umma_score_supported(const Params &p) {
-  if (!umma_requested() || !fused_score_supported(p)) return false;
+bool umma_score_supported(const Params &p) {
+  if (!umma_requested() || p.skew) return false;
+  if (p.NB > kSelThreads * 16) return false;                 // the selection team holds at most 16 blocks per thread
   if (p.summ_dtype != COBS_SUMM_FP4_E2M1 || p.u_q != nullptr) return false;
   if (p.D != 128 || p.Ds_pad != 128 || p.r != 8 || p.G > 8) return false;
   if (p.NB % kUBlocks != 0) return false;                    // whole 32-block stages
@@ -1987,7 +1166,8 @@ typedef CUresult (*cobs_tmap_encode_fn)(CUtensorMap *, CUtensorMapDataType, cuui
                                         const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                         CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-static cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream) {
+// cudaErrorNotSupported: too many units per CTA, or no encoder (nothing was launched).
+cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream) {
   static cobs_tmap_encode_fn encode = nullptr;
   static std::mutex mu;
   static int grid_cache[64] = {0};
@@ -2036,95 +1216,4 @@ static cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream) 
   return e;
 }
 
-cudaError_t launch_fused(const Params &p, int phases, cudaStream_t stream) {
-  if ((phases & PH_SCORE) && umma_score_supported(p)) {
-    const cudaError_t e = launch_fused_umma(p, phases, stream);
-    if (e != cudaErrorNotSupported) return e;                // not supported: too many units per CTA, or no encoder
-  }
-  const bool fp4 = p.summ_dtype == COBS_SUMM_FP4_E2M1 && (phases & PH_SCORE);
-  if (!fp4) {
-    return p.D == 128 ? launch_fused_t<COBS_SUMM_BF16, 128, 1, 1>(p, phases, stream)
-                      : launch_fused_t<COBS_SUMM_BF16, 64, 1, 1>(p, phases, stream);
-  }
-  const int wpt = p.Ds_pad / 32;
-  const bool sub = p.u_q != nullptr;
-#define COBS_CASE(DD, WW)                                                                                   \
-  if (p.D == DD && wpt == WW)                                                                               \
-    return sub ? launch_fused_t<COBS_SUMM_FP4_E2M1, DD, WW, 2>(p, phases, stream)                           \
-               : launch_fused_t<COBS_SUMM_FP4_E2M1, DD, WW, 1>(p, phases, stream);
-  COBS_CASE(128, 4) COBS_CASE(128, 3) COBS_CASE(128, 2) COBS_CASE(128, 1) COBS_CASE(64, 2) COBS_CASE(64, 1)
-#undef COBS_CASE
-  return cudaErrorInvalidValue;
-}
-
-int32_t prepare_attend_params(const cobs_config *cfg, const void *q, const cobs_kv *kv, const int32_t *sel_idx,
-                              const int32_t *sel_cnt, float *out, float *lse_or_null, Params *p);
-
-// ---------------------------------------------------------------------------------------------------
-// cobs_sparse_decode_static: the attention step with its scratch in device memory the library itself
-// owns, for callers that may not allocate.
-// ---------------------------------------------------------------------------------------------------
-// The scratch lives here, in a file-scope device array.  Every GPU that loads the library holds these
-// bytes until the process exits.  In host code the name below is only a handle: the device address is
-// obtained once per device with cudaGetSymbolAddress and that pointer is what the kernel is given.
-static __device__ __align__(256) unsigned char g_static_scratch[COBS_STATIC_SCRATCH_BYTES];
-
-static void *static_scratch_address(cudaError_t *err) {
-  static void *addr[64] = {nullptr};
-  static std::mutex mu;
-  int dev = 0;
-  *err = cudaGetDevice(&dev);
-  if (*err != cudaSuccess) return nullptr;
-  if (dev < 0 || dev >= 64) { *err = cudaErrorInvalidDevice; return nullptr; }
-  std::lock_guard<std::mutex> lock(mu);
-  if (!addr[dev]) {
-    void *ptr = nullptr;
-    *err = cudaGetSymbolAddress(&ptr, g_static_scratch);     // the current device's copy of the array
-    if (*err != cudaSuccess) return nullptr;
-    addr[dev] = ptr;
-  }
-  return addr[dev];
-}
-
 }  // namespace cobs
-
-extern "C" int32_t cobs_sparse_decode_static(const cobs_config *cfg, const void *q, const cobs_kv *kv,
-                                             const int32_t *sel_idx, const int32_t *sel_cnt, float *out,
-                                             float *lse_or_null, void *stream) {
-  using namespace cobs;
-  Params p;
-  int32_t st = prepare_attend_params(cfg, q, kv, sel_idx, sel_cnt, out, lse_or_null, &p);
-  if (st != COBS_OK) return st;
-  // scratch layout: [status word, epoch word, item / barrier words: 256 B][3 counters per unit][split partials]
-  const size_t units = (size_t)p.B * p.Hkv;
-  const size_t ctl_bytes = (3 * units * sizeof(int) + 255) / 256 * 256;     // every call starts from cleared words: set 0 only
-  const size_t partial_bytes = units * p.n_splits * p.G * (size_t)(p.D + 2) * sizeof(float);
-  if (kStatusBytes + ctl_bytes + partial_bytes > (size_t)COBS_STATIC_SCRATCH_BYTES) return COBS_ERR_WORKSPACE_TOO_SMALL;
-  cudaError_t e = cudaSuccess;
-  unsigned char *base = static_cast<unsigned char *>(static_scratch_address(&e));
-  if (!base) return COBS_ERR_CUDA;
-  p.status = reinterpret_cast<int32_t *>(base);
-  p.ctl_epoch = reinterpret_cast<int *>(base) + 1;
-  p.ctl_item = reinterpret_cast<int *>(base) + 2;
-  p.ctl_bar = reinterpret_cast<int *>(base) + 3;
-  p.ctl_set_stride = 0;                       // (the extent word is cleared with the rest: the other set is never touched)
-  p.ctl_score = reinterpret_cast<int *>(base + kStatusBytes);
-  p.ctl_ready = p.ctl_score + units;
-  p.ctl_att = p.ctl_ready + units;
-  p.partial = reinterpret_cast<float *>(base + kStatusBytes + ctl_bytes);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the array keeps whatever the previous call left: the status word and the counters must start at zero
-  if (cudaMemsetAsync(base, 0, kStatusBytes + ctl_bytes, s) != cudaSuccess) return COBS_ERR_CUDA;
-  return launch_fused(p, PH_ATTEND, s) == cudaSuccess ? COBS_OK : COBS_ERR_CUDA;
-}
-
-#ifdef COBS_TIMING
-extern "C" int cobs_debug_times(unsigned long long *host_out) {
-  return (int)cudaMemcpyFromSymbol(host_out, cobs::g_dbg_times, sizeof(unsigned long long) * 4 * 4096);
-}
-extern "C" int cobs_debug_acc(unsigned long long *host_out, int clear) {
-  int e = (int)cudaMemcpyFromSymbol(host_out, cobs::g_dbg_acc, sizeof(unsigned long long) * 8 * 4096);
-  if (clear) { static unsigned long long z[8 * 4096]; cudaMemcpyToSymbol(cobs::g_dbg_acc, z, sizeof(z)); }
-  return e;
-}
-#endif

@@ -43,7 +43,7 @@ def main():
     variants = [
         ("packed E2M1, rank 8 (step kernel scores)", base),
         ("bf16, rank 4 (step kernel scores)", base.replace(summary_dtype="bf16", rank=4)),
-        ("fp32, rank 4 (generic scoring + selection kernels)", base.replace(summary_dtype="fp32", rank=4)),
+        ("fp32, rank 4", base.replace(summary_dtype="fp32", rank=4)),
         ("packed E2M1 subspace 85, rank 4 (projection prologue)", base.replace(sub_dim=85, rank=4, query_model="spectrum")),
     ]
     for label, wl in variants:

@@ -91,7 +91,7 @@ def main():
     for s in (42, 56, 71, 85, 108):
         variants.append((f"subspace s={s}, r=4, fp4", base.replace(sub_dim=s, rank=4, summary_dtype="fp4")))
     variants.append(("subspace s=85, r=4, bf16", base.replace(sub_dim=85, rank=4, summary_dtype="bf16")))
-    # the diagonal-skew variant (Appendix, Cheap diagonal skew): r more scalars per block, scored by the generic kernels
+    # the diagonal-skew variant (Appendix, Cheap diagonal skew): r more scalars per block
     skewed = [(f"full space, r={rank}, bf16 + skew", base.replace(sub_dim=0, query_model="iid", rank=rank,
                                                                   summary_dtype="bf16")) for rank in (4, 8)]
     print(f"shape: B={base.batch}, {base.n_q_heads} query / {base.n_kv_heads} KV heads, D={base.head_dim}, "

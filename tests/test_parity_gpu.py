@@ -292,6 +292,28 @@ def test_shape_grid(summary_dtype, scale_dtype, G, D, L, P):
     run_stage_s(wl)
 
 
+# units x blocks x options at the edges of the step kernel's plan: clusters of 16, 5, 2 and 1 CTAs and two CTAs per SM; block
+# counts of every residue mod 16 and 4, up to the three selection layouts (2, 8, any number of keys per thread); scales that
+# start on any 2-byte boundary; the rows that are read element by element (fp32, bf16 in a subspace of odd width)
+@pytest.mark.parametrize("batch,hkv,G,D,nb,L,rank,sub,dtype,scale,topk", [
+    (1, 1, 4, 128, 4101, 16, 3, 0, "fp4", "fp16", 128),
+    (1, 2, 2, 64, 1027, 16, 5, 0, "fp4", "fp32", 100),
+    (1, 1, 8, 128, 517, 16, 8, 0, "bf16", "fp32", 31),
+    (3, 5, 1, 64, 61, 32, 7, 0, "fp4", "fp16", 9),
+    (3, 9, 4, 128, 30, 32, 1, 33, "fp4", "fp16", 4),
+    (2, 20, 2, 128, 18, 64, 6, 77, "bf16", "fp32", 3),
+    (5, 16, 2, 64, 33, 16, 4, 41, "fp32", "fp32", 7),
+    (19, 8, 1, 64, 35, 16, 16, 0, "fp32", "fp32", 6),
+    (40, 8, 1, 64, 47, 16, 3, 0, "fp4", "fp16", 5),
+])
+def test_unit_step_plan_edges(batch, hkv, G, D, nb, L, rank, sub, dtype, scale, topk):
+    lens = [nb * L - (7 * b) % L if b % 3 else nb * L for b in range(batch)]
+    wl = synth.Workload("plan", batch, hkv * G, hkv, D, nb * L, L, 16, rank=rank, topk=topk, window=3 * L + 5, sub_dim=sub,
+                        summary_dtype=dtype, scale_dtype=scale, key_model="block_offset", shuffle_pages=True, seed=17, seq_lens=lens)
+    units = [(b, h) for b in range(batch) for h in range(hkv)]
+    run_stage_s(wl, units=units if len(units) <= 32 else [units[0], units[1], units[len(units) // 2], units[-1]])
+
+
 def test_ragged_lengths_and_degenerate_cases():
     L = 64
     # T < L (no summarised block), T inside the window only, partial last block, k larger than candidates
