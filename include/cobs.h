@@ -167,8 +167,7 @@ int32_t cobs_build_summaries(const cobs_config *cfg, const cobs_kv *kv, int32_t 
  * (Method, Cost: a block's summary is built when the block fills, so the caller then rebuilds block
  * seq_len / L - 1 with cobs_build_summaries whenever the new length is a multiple of L).  A sequence whose page
  * table has no room for the position, or names a page outside [0, n_pages), leaves COBS_ERR_BOUNDS in the status
- * word and is not touched.  Uses the first batch * 4 bytes of the workspace's staging area for a snapshot of the
- * lengths.
+ * word and is not touched.
  */
 int32_t cobs_append_token(const cobs_config *cfg, const void *k_new, const void *v_new, void *k_pages, void *v_pages,
                           const int32_t *page_table, int32_t *seq_lens, int64_t n_pages, void *workspace,
@@ -264,10 +263,10 @@ int32_t cobs_decode_step(const cobs_config *cfg, const void *q, const cobs_kv *k
  * The fused step for a caller whose per-step tensors live in HOST memory: copies q_host to the device,
  * runs cobs_decode_step, copies the output back and synchronises `stream`.  The KV cache, page table and
  * summaries stay on the device (they are the state a decode loop keeps there).  q_host [B][Hq][D] bf16 and
- * out_host [B][Hq][D] fp32 should be pinned for the copies to be asynchronous; when out_host is pinned memory that
- * is mapped into the device's address space (cudaHostAlloc / cudaHostRegister under unified addressing) and 16-byte
- * aligned, the kernel writes the output rows straight into it and no device-to-host copy is made (measured: 10 us
- * less per step); other host memory goes through a staging buffer in the workspace.  sel_idx_host_or_null
+ * out_host [B][Hq][D] fp32 should be pinned memory that is mapped into the device's address space (cudaHostAlloc /
+ * cudaHostRegister under unified addressing) on a 16-byte boundary: the query is then fetched, and the output rows (and the
+ * selection, if its arrays are pinned too) written, by kernels, and no copy is made; other host memory goes through staging
+ * buffers in the workspace.  sel_idx_host_or_null
  * [B][Hkv][topk] and sel_cnt_host_or_null [B][Hkv] receive the selection when given.  On return the stream has been
  * synchronised and out_host holds the result.
  */

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kAThreads) adaptive_trim_kernel(Params p, floa
   __shared__ int s_id[kAThreads];
   __shared__ int s_warp[kAThreads / 32];
   __shared__ int s_k;
+  pdl_begin();
   const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b_idx = u / p.Hkv;
   const int T = p.seq_lens[b_idx];
@@ -95,9 +96,7 @@ __global__ void __launch_bounds__(kAThreads) adaptive_trim_kernel(Params p, floa
 }  // namespace
 
 cudaError_t launch_adaptive_trim(const Params &p, float tau, int k_min, cudaStream_t stream) {
-  adaptive_trim_kernel<<<p.B * p.Hkv, kAThreads, 0, stream>>>(p, tau, k_min);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(adaptive_trim_kernel, dim3(p.B * p.Hkv), dim3(kAThreads), 0, stream, p, tau, k_min);
 }
 
 }  // namespace cobs

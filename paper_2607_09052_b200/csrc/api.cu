@@ -24,10 +24,11 @@ cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream);
 bool umma_score_supported(const Params &p);
 cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
 cudaError_t launch_append(const Params &p, const void *k_new, const void *v_new, void *k_pages, void *v_pages, int32_t *seq_lens,
-                          int32_t *old_lens, cudaStream_t stream);
+                          cudaStream_t stream);
 cudaError_t launch_quantise(const float *xi, long long n_vectors, int Ds, int Ds_pad, int scale_dtype, void *codes,
                             void *scale, cudaStream_t stream);
 size_t build_smem_bytes(const Params &p);
+cudaError_t launch_stage(const void *src, void *dst, size_t bytes, cudaStream_t stream);
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -190,6 +191,17 @@ static int32_t set_kv(Params &p, const cobs_kv *kv) {
 
 static int32_t cuda_status(cudaError_t e) { return e == cudaSuccess ? COBS_OK : COBS_ERR_CUDA; }
 
+// The device address of pinned, device-mapped host memory on a 16-byte boundary, or NULL.
+static void *mapped(const void *host) {
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, host) == cudaSuccess) {
+    if (attr.type == cudaMemoryTypeHost && attr.devicePointer != nullptr && aligned16(attr.devicePointer)) return attr.devicePointer;
+  } else {
+    (void)cudaGetLastError();                  // unregistered host memory reports an error on some drivers: clear it
+  }
+  return nullptr;
+}
+
 // Scoring and selection, with the attention or without: one launch.  The generic scoring and selection kernels are for what the
 // unit kernel does not cover.
 static cudaError_t launch_score_step(const Params &p, int phases, cudaStream_t s) {
@@ -305,9 +317,7 @@ int32_t cobs_append_token(const cobs_config *cfg, const void *k_new, const void 
   fill_params(p, cfg, workspace);
   p.page_table = page_table;
   p.n_pages = n_pages;
-  // the snapshot of the lengths lives in the query staging area of the workspace (batch * 4 bytes of it)
-  int32_t *old_lens = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(workspace) + layout_workspace(cfg).q_stage);
-  return cuda_status(launch_append(p, k_new, v_new, k_pages, v_pages, seq_lens, old_lens, static_cast<cudaStream_t>(stream)));
+  return cuda_status(launch_append(p, k_new, v_new, k_pages, v_pages, seq_lens, static_cast<cudaStream_t>(stream)));
 }
 
 int32_t cobs_quantise_xi(const cobs_config *cfg, const float *xi_fp32, int64_t n_vectors, void *codes, void *scale,
@@ -437,27 +447,34 @@ int32_t cobs_decode_step_host(const cobs_config *cfg, const void *q_host, const 
   void *q_dev = base + w.q_stage;
   float *out_dev = reinterpret_cast<float *>(base + w.out_stage);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const size_t n = (size_t)cfg->batch * cfg->n_q_heads * cfg->head_dim;
-  if (cudaMemcpyAsync(q_dev, q_host, n * 2, cudaMemcpyHostToDevice, s) != cudaSuccess) return COBS_ERR_CUDA;
-  // Pinned, device-mapped output memory: the merge writes its rows straight into it (posted writes over PCIe, 256 KB
-  // spread over the tail of the kernel), which saves a device-to-host copy and its latency after the kernel.  Any
-  // other host memory goes through the staging buffer.
-  float *out_direct = nullptr;
-  {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, out_host) == cudaSuccess && attr.type == cudaMemoryTypeHost &&
-        attr.devicePointer != nullptr && aligned16(attr.devicePointer))
-      out_direct = static_cast<float *>(attr.devicePointer);
-    else
-      (void)cudaGetLastError();                  // unregistered host memory reports an error on some drivers: clear it
-  }
-  st = cobs_decode_step(cfg, q_dev, kv, summ, out_direct ? out_direct : out_dev, nullptr, nullptr, nullptr, workspace,
-                        workspace_bytes, stream);
-  if (st != COBS_OK) return st;
-  if (!out_direct && cudaMemcpyAsync(out_host, out_dev, n * sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  const size_t n = (size_t)cfg->batch * cfg->n_q_heads * cfg->head_dim, units = (size_t)cfg->batch * cfg->n_kv_heads;
+  // Pinned, device-mapped memory is read and written in place: the query by a small kernel that the step is chained to (a
+  // copy-engine transfer and the hand-over to it cost more than the 131 KB over the bus), the output rows and the selection
+  // by posted writes of the step kernel, which saves their copies after it.  Any other host memory goes through copies.
+  const void *q_map = mapped(q_host);
+  float *out_map = static_cast<float *>(mapped(out_host));
+  if (q_map) {
+    if (launch_stage(q_map, q_dev, n * 2, s) != cudaSuccess) return COBS_ERR_CUDA;
+  } else if (cudaMemcpyAsync(q_dev, q_host, n * 2, cudaMemcpyHostToDevice, s) != cudaSuccess) {
     return COBS_ERR_CUDA;
+  }
+  int32_t *sel_map = nullptr, *cnt_map = nullptr;
   if (sel_idx_host_or_null) {
-    const size_t units = (size_t)cfg->batch * cfg->n_kv_heads;
+    Params p;
+    fill_params(p, cfg, workspace);
+    if ((st = set_summaries(p, cfg, summ)) != COBS_OK) return st;
+    if (unit_score_supported(p) && !umma_score_supported(p)) {       // (the other paths read the selection back)
+      sel_map = static_cast<int32_t *>(mapped(sel_idx_host_or_null));
+      cnt_map = static_cast<int32_t *>(mapped(sel_cnt_host_or_null));
+    }
+  }
+  const bool sel_direct = sel_map && cnt_map;
+  st = cobs_decode_step(cfg, q_dev, kv, summ, out_map ? out_map : out_dev, nullptr, sel_direct ? sel_map : nullptr,
+                        sel_direct ? cnt_map : nullptr, workspace, workspace_bytes, stream);
+  if (st != COBS_OK) return st;
+  if (!out_map && cudaMemcpyAsync(out_host, out_dev, n * sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    return COBS_ERR_CUDA;
+  if (sel_idx_host_or_null && !sel_direct) {
     if (cudaMemcpyAsync(sel_idx_host_or_null, base + w.sel_idx, units * cfg->topk * sizeof(int32_t),
                         cudaMemcpyDeviceToHost, s) != cudaSuccess) return COBS_ERR_CUDA;
     if (cudaMemcpyAsync(sel_cnt_host_or_null, base + w.sel_cnt, units * sizeof(int32_t), cudaMemcpyDeviceToHost,

@@ -56,6 +56,28 @@ struct Params {
 void count_launch(int n = 1);
 void count_tcgen05_launch();
 
+// Programmatic dependent launch: every kernel of the library begins with pdl_begin and is launched by launch_chained, so that
+// in a chain of calls on one stream (append, build, step; score, trim, attend; step after step) a kernel's CTAs are set up
+// while the last ones of the kernel before it still run.  The wait returns when that kernel has completed and its writes are
+// visible: nothing is read or written before it.  (A kernel launched without the attribute is not overtaken, nor does one
+// that does not say launch_dependents let its successor in early.)
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+template <class... KArgs, class... Args>
+static cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  count_launch();
+  return e;
+}
+
 __device__ __forceinline__ void report(int32_t *status, int code) {
   if (status) atomicCAS(status, 0, code);
 }

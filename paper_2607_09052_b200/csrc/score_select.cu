@@ -44,6 +44,7 @@ __device__ void prepare_query(const Params &p, int b_idx, int h, float *qs, floa
 template <int G, int DT>
 __global__ void __launch_bounds__(256) score_generic_kernel(Params p, int blocks_per_cta) {
   extern __shared__ float smem[];
+  pdl_begin();
   float *qs = smem;                 // [G][D]
   float *qt = smem + G * p.D;       // [G][Ds_pad]
   const int u = blockIdx.y, b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
@@ -148,6 +149,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(Params p) {
   __shared__ uint32_t s_prefix;
   __shared__ int s_need;
 
+  pdl_begin();
   const int u = blockIdx.x, b_idx = u / p.Hkv, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int T = p.seq_lens[b_idx];
   const int n_sum = min(T / p.L, p.NB);
@@ -273,12 +275,10 @@ static cudaError_t launch_score_g(const Params &p, cudaStream_t stream) {
   dim3 grid((p.NB + blocks_per_cta - 1) / blocks_per_cta, p.B * p.Hkv);
   size_t smem = (size_t)G * (p.D + p.Ds_pad) * sizeof(float);
   switch (p.summ_dtype) {
-    case COBS_SUMM_FP32: score_generic_kernel<G, COBS_SUMM_FP32><<<grid, 256, smem, stream>>>(p, blocks_per_cta); break;
-    case COBS_SUMM_BF16: score_generic_kernel<G, COBS_SUMM_BF16><<<grid, 256, smem, stream>>>(p, blocks_per_cta); break;
-    default: score_generic_kernel<G, COBS_SUMM_FP4_E2M1><<<grid, 256, smem, stream>>>(p, blocks_per_cta); break;
+    case COBS_SUMM_FP32: return launch_chained(score_generic_kernel<G, COBS_SUMM_FP32>, grid, dim3(256), smem, stream, p, blocks_per_cta);
+    case COBS_SUMM_BF16: return launch_chained(score_generic_kernel<G, COBS_SUMM_BF16>, grid, dim3(256), smem, stream, p, blocks_per_cta);
+    default: return launch_chained(score_generic_kernel<G, COBS_SUMM_FP4_E2M1>, grid, dim3(256), smem, stream, p, blocks_per_cta);
   }
-  count_launch();
-  return cudaGetLastError();
 }
 
 cudaError_t launch_score(const Params &p, cudaStream_t stream) {
@@ -296,9 +296,7 @@ cudaError_t launch_select(const Params &p, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  select_kernel<<<p.B * p.Hkv, kSelThreads, smem, stream>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(select_kernel, dim3(p.B * p.Hkv), dim3(kSelThreads), smem, stream, p);
 }
 
 }  // namespace cobs

@@ -54,6 +54,7 @@ __device__ void quantise_row_warp(const float *row, int Ds, int Ds_pad, uint32_t
 
 __global__ void quantise_kernel(const float *xi, long long n_vectors, int Ds, int Ds_pad, int scale_dtype,
                                 uint8_t *codes, void *scale) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long vec = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (vec >= n_vectors) return;
@@ -786,6 +787,7 @@ __global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4)
 build_kernel(Params p, int block_begin, int block_end, int solver, const int *flags, int n) {
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_flag[kBuildThreads];
+  pdl_begin();
   const int n_range = block_end - block_begin, per = flags ? kBuildThreads : 1;
   for (long long base = (long long)blockIdx.x * per; base < n; base += (long long)gridDim.x * per) {
     if (flags) {
@@ -814,9 +816,7 @@ static cudaError_t launch_build_tl(const Params &p, int block_begin, int block_e
   if (e != cudaSuccess) return e;
   const int n = p.B * p.Hkv * (block_end - block_begin);
   const int grid = flags ? min((n + kBuildThreads - 1) / kBuildThreads, 296) : n;
-  build_kernel<TL><<<grid, kBuildThreads, smem, stream>>>(p, block_begin, block_end, solver, flags, n);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(build_kernel<TL>, dim3(grid), dim3(kBuildThreads), smem, stream, p, block_begin, block_end, solver, flags, n);
 }
 
 cudaError_t launch_build_fast(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
@@ -842,44 +842,38 @@ cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *f
   }
 }
 
-// One new token per sequence into the paged cache: 16 bytes per thread, one CTA per (sequence, KV head); the
-// CTAs of KV head 0 also advance the sequence lengths once every CTA of the sequence has read the old one.
-__global__ void append_kernel(Params p, const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bfloat16 *k_pages,
-                              __nv_bfloat16 *v_pages, int32_t *seq_lens, const int32_t *old_lens) {
-  const int b = blockIdx.x / p.Hkv, h = blockIdx.x - b * p.Hkv;
-  const int T = old_lens[b];
-  if (T < 0 || T >= p.mpp * p.P) { if (threadIdx.x == 0) report(p.status, COBS_ERR_BOUNDS); return; }
-  const int pg = p.page_table[(size_t)b * p.mpp + T / p.P];
-  if (pg < 0 || pg >= p.n_pages) { if (threadIdx.x == 0) report(p.status, COBS_ERR_BOUNDS); return; }
-  const size_t dst = (((size_t)pg * p.Hkv + h) * p.P + (T % p.P)) * p.D, src = ((size_t)b * p.Hkv + h) * p.D;
-  for (int i = threadIdx.x; i < p.D / 8; i += blockDim.x) {
-    reinterpret_cast<uint4 *>(k_pages + dst)[i] = reinterpret_cast<const uint4 *>(k_new + src)[i];
-    reinterpret_cast<uint4 *>(v_pages + dst)[i] = reinterpret_cast<const uint4 *>(v_new + src)[i];
+// One new token per sequence into the paged cache: one CTA per sequence, 16 bytes per thread and turn; the CTA that has read the
+// length is the one that advances it.
+__global__ void __launch_bounds__(256) append_kernel(Params p, const uint4 *k_new, const uint4 *v_new, uint4 *k_pages, uint4 *v_pages, int32_t *seq_lens) {
+  pdl_begin();
+  const int b = blockIdx.x, T = seq_lens[b], d8 = p.D / 8;
+  const int pg = (T >= 0 && T < p.mpp * p.P) ? p.page_table[(size_t)b * p.mpp + T / p.P] : -1;
+  if (pg < 0 || pg >= p.n_pages) {
+    if (threadIdx.x == 0) report(p.status, COBS_ERR_BOUNDS);
+    return;
   }
-  if (h == 0 && threadIdx.x == 0) seq_lens[b] = T + 1;
+  for (int i = threadIdx.x; i < p.Hkv * d8; i += blockDim.x) {
+    const int h = i / d8, j = i - h * d8;
+    const size_t dst = (((size_t)pg * p.Hkv + h) * p.P + (T % p.P)) * d8 + j, src = (size_t)b * p.Hkv * d8 + i;
+    k_pages[dst] = k_new[src];
+    v_pages[dst] = v_new[src];
+  }
+  __syncthreads();                               // every thread has used the old length
+  if (threadIdx.x == 0) seq_lens[b] = T + 1;
 }
 
-// old_lens: a snapshot of the lengths taken on the stream before the launch (the kernel reads the snapshot and
-// writes the live array, so no CTA can see a length another CTA has already advanced).
 cudaError_t launch_append(const Params &p, const void *k_new, const void *v_new, void *k_pages, void *v_pages, int32_t *seq_lens,
-                          int32_t *old_lens, cudaStream_t stream) {
-  cudaError_t e = cudaMemcpyAsync(old_lens, seq_lens, sizeof(int32_t) * p.B, cudaMemcpyDeviceToDevice, stream);
-  if (e != cudaSuccess) return e;
-  append_kernel<<<p.B * p.Hkv, 32, 0, stream>>>(p, static_cast<const __nv_bfloat16 *>(k_new), static_cast<const __nv_bfloat16 *>(v_new),
-                                                 static_cast<__nv_bfloat16 *>(k_pages), static_cast<__nv_bfloat16 *>(v_pages), seq_lens,
-                                                 old_lens);
-  count_launch();
-  return cudaGetLastError();
+                          cudaStream_t stream) {
+  return launch_chained(append_kernel, dim3(p.B), dim3(256), 0, stream, p, static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
+                        static_cast<uint4 *>(k_pages), static_cast<uint4 *>(v_pages), seq_lens);
 }
 
 cudaError_t launch_quantise(const float *xi, long long n_vectors, int Ds, int Ds_pad, int scale_dtype, void *codes,
                             void *scale, cudaStream_t stream) {
   if (n_vectors <= 0) return cudaSuccess;
   const int wpb = 8;
-  quantise_kernel<<<(unsigned)((n_vectors + wpb - 1) / wpb), wpb * 32, 0, stream>>>(xi, n_vectors, Ds, Ds_pad,
-                                                                                 scale_dtype, (uint8_t *)codes, scale);
-  count_launch();
-  return cudaGetLastError();
+  return launch_chained(quantise_kernel, dim3((unsigned)((n_vectors + wpb - 1) / wpb)), dim3(wpb * 32), 0, stream, xi, n_vectors, Ds, Ds_pad, scale_dtype,
+                        (uint8_t *)codes, scale);
 }
 
 // The GPU's own float -> E2M1 conversion instruction, one code per input value: what the threshold chain of

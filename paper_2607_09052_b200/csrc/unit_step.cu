@@ -18,7 +18,8 @@
 // Measured against the persistent kernel with counters in global memory that this one replaced (a step among others, us):
 // one sequence of 32k 31.9 -> 20.5, four of 32k with a subspace 37.0 -> 26.7, sixteen of 128k 115 -> 98 (80 % of the measured
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
-// summaries at 2k (three launches before) 36.4 -> 18.5.
+// summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
+// search: 17.1, 23.4, 95-98, 43.5, 16.9.
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
 // chunk is three contiguous pieces of the summary arrays, fetched by three bulk copies (cp.async.bulk, completion on an
@@ -481,9 +482,11 @@ struct Scorer {
 };
 
 // ---------------------------------------------------------------------------------------------------
-// Scoring from rows that bulk copies cannot fetch or whose factors need more than squares: fp32 summaries, bf16 factors in a
-// subspace (rows of 2 * Ds bytes start anywhere), the diagonal-skew variant.  A thread reads its eight elements of a row
-// straight from global memory (a quad takes 128 or 64 consecutive bytes; 16 loads in flight per row of 16 blocks).
+// Scoring from rows of floats: fp32 summaries, bf16 factors in a subspace, the diagonal-skew variant.  Rows of Ds elements start
+// on any element; a block's rows are fetched by one bulk copy of the 16-byte units that hold them, in batches of as many rows
+// as fit a stage, and read back 16 bytes or (rows that are no multiple of 16 bytes) one element at a time.
+// (Reading them straight from global memory, one row of 16 blocks in flight per warp, took 1366 us for 2.4 GB of fp32 summaries,
+// 288 units; this way 688.  A single sequence of 2k does not gain: 16.9 us, 15.7 that way.)
 // ---------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void split3(float x, float y, uint32_t &a, uint32_t &b, uint32_t &c) {
   a = bf16x2(x, y);
@@ -492,52 +495,108 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t &a, uint32_t &
   c = bf16x2(x1 - bf16_lo(b), y1 - bf16_hi(b));
 }
 template <int DT, int D>
-struct DirectScorer {
+struct RowScorer {
   static constexpr bool F32 = (DT == COBS_SUMM_FP32);
+  static constexpr int ES = F32 ? 4 : 2;
   static constexpr int KS = D / 32;               // groups of 32 elements (8 per lane of a quad)
   static constexpr int XT = F32 ? 3 : 1;          // bf16 terms of a stored value
-  using El = typename std::conditional<F32, float, uint16_t>::type;
+  static constexpr int PAD = 32;                  // rows of neighbouring blocks start in different banks
+  static constexpr int MROW = D * ES + PAD;
+  static constexpr int ROOM = kStage / 16 - PAD - 32;       // bytes of a block's rows in a batch (the copy takes up to 15 more at either end)
+  static_assert(ROOM >= D * ES, "a stage must hold a row of every block");
   const Params &p;
-  int lane;
-  __device__ __forceinline__ DirectScorer(const Params &p_, const Unit &, unsigned char *, uint64_t *, int lane_) : p(p_), lane(lane_) {}
-  __device__ __forceinline__ void start(int, int) {}
+  unsigned char *wsm;
+  uint32_t ring, bar0;
+  int lane, rowb, rows0, rows_n, n_batches;
+  uint64_t pol;
+  size_t rec_u, xi_total;
 
-  // eight elements j .. j + 7 of a row of n elements, as bf16 pairs in XT terms (zeros beyond the row)
-  __device__ __forceinline__ void load8(const El *row, int j, int n, bool vec, bool live, uint32_t (&t)[XT][4]) const {
+  __device__ __forceinline__ RowScorer(const Params &p_, const Unit &x, unsigned char *wsm_, uint64_t *bars, int lane_) : p(p_), wsm(wsm_), lane(lane_) {
+    ring = smem_u32(wsm);
+    bar0 = smem_u32(bars);
+    rowb = p.Ds * ES;
+    rows0 = min(p.r, max(0, ROOM - MROW) / rowb);            // rows beside the means
+    rows_n = ROOM / rowb;
+    n_batches = 1 + (p.r - rows0 + rows_n - 1) / rows_n;
+    pol = l2_evict_first_policy();
+    rec_u = (size_t)x.u * p.NB;
+    xi_total = (size_t)p.B * p.Hkv * p.NB * p.r * rowb;
+  }
+  __device__ __forceinline__ int first_row(int b) const { return (b == 0) ? 0 : rows0 + (b - 1) * rows_n; }
+  __device__ __forceinline__ int n_rows(int b) const { return (b == 0) ? rows0 : min(p.r - first_row(b), rows_n); }
+  __device__ __forceinline__ int stride(int b) const { return (((b == 0) ? rows0 : rows_n) * rowb + 16 + 15) / 16 * 16 + PAD; }
+  __device__ __forceinline__ int shift(size_t rec, int b) const { return (int)(((rec * p.r + first_row(b)) * rowb) & 15); }
+
+  __device__ __forceinline__ void issue(int ck, int b, int st) {
+    const int nblk = min(16, p.NB - ck * 16), i = lane & 15;
+    const size_t rec = rec_u + ck * 16 + i;
+    const bool on = i < nblk, mean = lane >= 16;
+    const int rows = n_rows(b);
+    const uint32_t sbase = ring + st * kStage, bar = bar0 + st * 8;
+    const char *src = nullptr;
+    uint32_t dst = 0, bytes = 0;
+    if (on && mean && b == 0) {
+      src = (const char *)p.mean + rec * (size_t)(D * ES);
+      dst = sbase + i * MROW;
+      bytes = D * ES;
+    } else if (on && !mean && rows > 0) {
+      const size_t s0 = (rec * p.r + first_row(b)) * (size_t)rowb;
+      const int sh = (int)(s0 & 15);
+      src = (const char *)p.xi + (s0 - sh);
+      dst = sbase + ((b == 0) ? 16 * MROW : 0) + i * stride(b);
+      bytes = (sh + rows * rowb + 15) & ~15;
+      if (s0 - sh + bytes > xi_total) {             // the end of the array: what is left of its last 16 bytes, element by element
+        bytes = (uint32_t)(xi_total - (s0 - sh)) & ~15u;
+        for (int k = (int)bytes / ES; k < (sh + rows * rowb) / ES; ++k) {
+          if (F32) reinterpret_cast<float *>(wsm + (dst - ring))[k] = reinterpret_cast<const float *>(src)[k];
+          else reinterpret_cast<uint16_t *>(wsm + (dst - ring))[k] = reinterpret_cast<const uint16_t *>(src)[k];
+        }
+      }
+    }
+    const uint32_t tx = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) mbar_expect_tx(bar, tx);
+    __syncwarp();
+    if (bytes) bulk_g2s(dst, src, bytes, bar, pol);
+  }
+  __device__ __forceinline__ void start(int cb, int ce) {
+    if (cb < ce) issue(cb, 0, 0);
+  }
+
+  // eight elements from element j on of a row of n elements at address a, as bf16 pairs in XT terms (zeros beyond the row)
+  __device__ __forceinline__ void load8(uint32_t a, int j, int n, bool vec, bool swap, uint32_t (&t)[XT][4]) const {
     if constexpr (F32) {
       float f[8];
-      if (vec) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        if (live && j < n) a = __ldg(reinterpret_cast<const float4 *>(row + j));
-        if (live && j + 4 < n) b = __ldg(reinterpret_cast<const float4 *>(row + j + 4));
-        f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+      if (vec) {                                    // (n is a multiple of 4; odd gid reads the second half first: no bank conflicts)
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        const int jx = j + (swap ? 4 : 0), jy = j + (swap ? 0 : 4);
+        const uint4 v = (jx < n) ? lds128(a + jx * 4) : z, w = (jy < n) ? lds128(a + jy * 4) : z;
+        const uint4 lo = swap ? w : v, hi = swap ? v : w;
+        f[0] = __uint_as_float(lo.x); f[1] = __uint_as_float(lo.y); f[2] = __uint_as_float(lo.z); f[3] = __uint_as_float(lo.w);
+        f[4] = __uint_as_float(hi.x); f[5] = __uint_as_float(hi.y); f[6] = __uint_as_float(hi.z); f[7] = __uint_as_float(hi.w);
       } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = (live && j + i < n) ? __ldg(row + j + i) : 0.f;
+        for (int i = 0; i < 8; ++i) f[i] = (j + i < n) ? lds_f32(a + (j + i) * 4) : 0.f;
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) split3(f[2 * i], f[2 * i + 1], t[0][i], t[XT > 1 ? 1 : 0][i], t[XT - 1][i]);
     } else {
       if (vec) {
-        uint4 a = make_uint4(0u, 0u, 0u, 0u);
-        if (live && j < n) a = __ldg(reinterpret_cast<const uint4 *>(row + j));
-        t[0][0] = a.x; t[0][1] = a.y; t[0][2] = a.z; t[0][3] = a.w;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (j < n) v = lds128(a + j * 2);
+        t[0][0] = v.x; t[0][1] = v.y; t[0][2] = v.z; t[0][3] = v.w;
       } else {
+        const uint16_t *q = reinterpret_cast<const uint16_t *>(wsm + (a - ring)) + j;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t a = (live && j + 2 * i < n) ? __ldg(row + j + 2 * i) : 0u;
-          const uint32_t b = (live && j + 2 * i + 1 < n) ? __ldg(row + j + 2 * i + 1) : 0u;
-          t[0][i] = a | (b << 16);
-        }
+        for (int i = 0; i < 4; ++i)
+          t[0][i] = ((j + 2 * i < n) ? (uint32_t)q[2 * i] : 0u) | ((j + 2 * i + 1 < n) ? (uint32_t)q[2 * i + 1] << 16 : 0u);
       }
     }
   }
 
   __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, Run (&rn)[2]) {
     if (cb >= ce) return true;
-    const int gid = lane >> 2, tig = lane & 3, G = p.G, Ds = p.Ds, r = p.r;
-    const bool sub = p.u_q != nullptr;
-    const bool vec = (Ds % (F32 ? 4 : 8)) == 0;
+    const int gid = lane >> 2, tig = lane & 3, G = p.G, Ds = p.Ds;
+    const bool sub = p.u_q != nullptr, vec = (rowb & 15) == 0, swap = gid & 1;
     const float inv_sqrt_d = 1.0f / sqrtf((float)D);
     const float ln_l = (float)(31 - __clz(p.L)) * 0.6931471805599453f;
     uint32_t bm[KS][4], bs[3][KS][4];               // the raw query; the subspace query in three bf16 terms
@@ -558,60 +617,76 @@ struct DirectScorer {
         split3(a, b, bs[0][m][i], bs[1][m][i], bs[2][m][i]);
       }
     }
-    // products of one row kind of the two blocks; `full` = against the raw query, else against the subspace query
-    auto row_product = [&](const El *ra, const El *rb, int n, bool v, bool la, bool lb, bool full, float (&d)[4]) {
-      uint32_t ta[KS][XT][4], tb[KS][XT][4];
-#pragma unroll
-      for (int m = 0; m < KS; ++m) {
-        load8(ra, (tig + 4 * m) * 8, n, v, la, ta[m]);
-        load8(rb, (tig + 4 * m) * 8, n, v, lb, tb[m]);
-      }
+    // products of one row of the two blocks; `full` = against the raw query, else against the subspace query
+    auto row_product = [&](uint32_t ra, uint32_t rb, int n, bool v, bool full, float (&d)[4]) {
       d[0] = d[1] = d[2] = d[3] = 0.f;
       float e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int m = 0; m < KS; ++m) {
+        uint32_t ta[XT][4], tb[XT][4];
+        load8(ra, (tig + 4 * m) * 8, n, v, swap, ta);
+        load8(rb, (tig + 4 * m) * 8, n, v, swap, tb);
         if (full) {
 #pragma unroll
           for (int t = XT - 1; t >= 0; --t) {
-            mma16816_bf16(d[0], d[1], d[2], d[3], ta[m][t][0], tb[m][t][0], ta[m][t][1], tb[m][t][1], bm[m][0], bm[m][1]);
-            mma16816_bf16(e[0], e[1], e[2], e[3], ta[m][t][2], tb[m][t][2], ta[m][t][3], tb[m][t][3], bm[m][2], bm[m][3]);
+            mma16816_bf16(d[0], d[1], d[2], d[3], ta[t][0], tb[t][0], ta[t][1], tb[t][1], bm[m][0], bm[m][1]);
+            mma16816_bf16(e[0], e[1], e[2], e[3], ta[t][2], tb[t][2], ta[t][3], tb[t][3], bm[m][2], bm[m][3]);
           }
         } else {
 #pragma unroll
           for (int t = XT - 1; t >= 0; --t)
 #pragma unroll
             for (int s = 2 - t; s >= 0; --s) {        // terms below 2^-24 of the product are left out
-              mma16816_bf16(d[0], d[1], d[2], d[3], ta[m][t][0], tb[m][t][0], ta[m][t][1], tb[m][t][1], bs[s][m][0], bs[s][m][1]);
-              mma16816_bf16(e[0], e[1], e[2], e[3], ta[m][t][2], tb[m][t][2], ta[m][t][3], tb[m][t][3], bs[s][m][2], bs[s][m][3]);
+              mma16816_bf16(d[0], d[1], d[2], d[3], ta[t][0], tb[t][0], ta[t][1], tb[t][1], bs[s][m][0], bs[s][m][1]);
+              mma16816_bf16(e[0], e[1], e[2], e[3], ta[t][2], tb[t][2], ta[t][3], tb[t][3], bs[s][m][2], bs[s][m][3]);
             }
         }
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) d[i] += e[i];
     };
-    for (int ck = cb; ck < ce; ++ck) {
-      const int bA = ck * 16 + 2 * gid;
-      const bool la = bA < x.n_sum, lb = bA + 1 < x.n_sum;
-      const size_t rec = (size_t)x.u * p.NB + bA;
+    const float qs = sub ? 1.0f : inv_sqrt_d;
+    float fA0 = 0.f, fA1 = 0.f, fB0 = 0.f, fB1 = 0.f, sA0 = 0.f, sA1 = 0.f, sB0 = 0.f, sB1 = 0.f;
+    int ck = cb, b = 0, st = 0;
+    uint32_t phase_bits = 0;
+    while (ck < ce) {
+      int nck = ck, nb = b + 1;
+      if (nb >= n_batches) { nb = 0; ++nck; }
+      if (nck < ce) issue(nck, nb, st ^ 1);
+      if (!mbar_wait(bar0 + st * 8, (phase_bits >> st) & 1u)) {     // bounded: the copies never landed
+        if (lane == 0) report(p.status, COBS_ERR_TIMEOUT);
+        return false;
+      }
+      phase_bits ^= 1u << st;
+      __syncwarp();
+      const uint32_t sbase = ring + st * kStage;
+      const size_t rec = rec_u + ck * 16 + 2 * gid;
       float d[4];
-      row_product((const El *)p.mean + rec * D, (const El *)p.mean + (rec + 1) * D, D, true, la, lb, true, d);
-      const float fA0 = d[0] * inv_sqrt_d, fA1 = d[1] * inv_sqrt_d, fB0 = d[2] * inv_sqrt_d, fB1 = d[3] * inv_sqrt_d;
-      float sA0 = 0.f, sA1 = 0.f, sB0 = 0.f, sB1 = 0.f;
-      const El *xa = (const El *)p.xi + rec * r * Ds, *xb = xa + (size_t)r * Ds;
-      const float qs = sub ? 1.0f : inv_sqrt_d;
+      if (b == 0) {
+        const uint32_t ma = sbase + 2 * gid * MROW;
+        row_product(ma, ma + MROW, D, true, true, d);
+        fA0 = d[0] * inv_sqrt_d; fA1 = d[1] * inv_sqrt_d; fB0 = d[2] * inv_sqrt_d; fB1 = d[3] * inv_sqrt_d;
+        sA0 = sA1 = sB0 = sB1 = 0.f;
+      }
+      const uint32_t xo = sbase + ((b == 0) ? 16 * MROW : 0) + 2 * gid * stride(b);
+      const uint32_t xa = xo + shift(rec, b), xb = xo + stride(b) + shift(rec + 1, b);
+      const int rows = n_rows(b), row0 = first_row(b);
 #pragma unroll 1
-      for (int i = 0; i < r; ++i) {
-        row_product(xa + (size_t)i * Ds, xb + (size_t)i * Ds, Ds, vec, la, lb, !sub, d);
+      for (int i = 0; i < rows; ++i) {
+        row_product(xa + i * rowb, xb + i * rowb, Ds, vec, !sub, d);
         float cA = 0.f, cB = 0.f;                    // (c / 6) / (1 / 2): folded into the sums that are halved below
         if (p.skew) {
-          if (la) cA = __ldg(p.skew + rec * r + i) * (1.0f / 3.0f);
-          if (lb) cB = __ldg(p.skew + (rec + 1) * r + i) * (1.0f / 3.0f);
+          if (ck * 16 + 2 * gid < x.n_sum) cA = __ldg(p.skew + rec * p.r + row0 + i) * (1.0f / 3.0f);
+          if (ck * 16 + 2 * gid + 1 < x.n_sum) cB = __ldg(p.skew + (rec + 1) * p.r + row0 + i) * (1.0f / 3.0f);
         }
         const float d0 = d[0] * qs, d1 = d[1] * qs, d2 = d[2] * qs, d3 = d[3] * qs;
         sA0 = fmaf(d0 * d0, fmaf(cA, d0, 1.0f), sA0); sA1 = fmaf(d1 * d1, fmaf(cA, d1, 1.0f), sA1);
         sB0 = fmaf(d2 * d2, fmaf(cB, d2, 1.0f), sB0); sB1 = fmaf(d3 * d3, fmaf(cB, d3, 1.0f), sB1);
       }
-      put_e(x, G, ck, gid, tig, ln_l + fA0 + 0.5f * sA0, ln_l + fB0 + 0.5f * sB0, ln_l + fA1 + 0.5f * sA1, ln_l + fB1 + 0.5f * sB1, rn);
+      if (b == n_batches - 1)
+        put_e(x, G, ck, gid, tig, ln_l + fA0 + 0.5f * sA0, ln_l + fB0 + 0.5f * sB0, ln_l + fA1 + 0.5f * sA1, ln_l + fB1 + 0.5f * sB1, rn);
+      __syncwarp();                           // all lanes are done with stage st before it is refilled
+      ck = nck; b = nb; st ^= 1;
     }
     return true;
   }
@@ -677,7 +752,7 @@ __device__ __forceinline__ void select_topk(const float *keys_s, int n, int k, i
       for (int j = 0; j < per; ++j) f((b0 + j < n) ? __float_as_uint(keys_s[b0 + j]) : 0u, b0 + j);
     }
   };
-  // theta = the largest T with #(key >= T) >= k, found two bits at a time: three trial values whose counts travel packed, 10
+  // theta = the largest T with #(key >= T) >= k (or any with exactly k), found two bits at a time: three trial counts packed, 10
   // bits each in one word while there are fewer than 1024 keys (BPT <= 2), else 16 bits each in two
   constexpr bool ONE = BPT == 1 || BPT == 2;
   uint32_t theta = 0u;
@@ -702,7 +777,9 @@ __device__ __forceinline__ void select_topk(const float *keys_s, int n, int k, i
     par ^= 1;
     const uint32_t ku = (uint32_t)k;
     const uint32_t na = ONE ? n0 & 1023u : n0 & 0xffffu, nb = ONE ? (n0 >> 10) & 1023u : n0 >> 16, nc = ONE ? n0 >> 20 : n1;
+    const uint32_t at = (na >= ku) ? na : (nb >= ku) ? nb : (nc >= ku) ? nc : 0u;
     if (na >= ku) theta = ta; else if (nb >= ku) theta = tb; else if (nc >= ku) theta = tc;
+    if (at == ku) break;                             // (uniform) exactly k keys are >= theta: the bits below do not matter
   }
   // keep every key above theta and the lowest-index `need_eq` keys equal to it, in index order: one scan of the
   // packed (above, equal) counts gives both the totals and this thread's position
@@ -917,8 +994,18 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, W = pl.W, C = pl.C, nthr = W * 32;
   const int u = blockIdx.x / C, rank = blockIdx.x - u * C;
   const int G = p.G, L = p.L, NB = p.NB;
-  COBS_STAMP(0);
   if (C > 1) cluster_arrive();                             // (waited for before the first access to another CTA's memory)
+  if (tid < 2 * 2 * kMaxW) (&s_cnt[0][0][0])[tid] = 0u;
+  if (tid < kMaxW) s_scan[tid] = 0;
+  if (tid == 0) s_lost = 0;
+  if (lane == 0) {
+    mbar_init(smem_u32(&s_bars[warp][0]), 1);
+    mbar_init(smem_u32(&s_bars[warp][1]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+  pdl_begin();
+  COBS_STAMP(0);
   Unit x;
   x.u = u; x.b_idx = u / p.Hkv; x.h = u - x.b_idx * p.Hkv;
   const int T = p.seq_lens[x.b_idx];
@@ -929,18 +1016,8 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   unsigned char *wsm = fsm + warp * kRing;
   const int nw = C * W, wi = rank * W + warp;
   int n_sel = min(p.topk, n_cand);
-  if (tid < 2 * 2 * kMaxW) (&s_cnt[0][0][0])[tid] = 0u;
-  if (tid < kMaxW) s_scan[tid] = 0;
-  if (tid == 0) s_lost = 0;
-  __syncthreads();
 
   if (phases & PH_SCORE) {
-    if (lane == 0) {
-      mbar_init(smem_u32(&s_bars[warp][0]), 1);
-      mbar_init(smem_u32(&s_bars[warp][1]), 1);
-      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    __syncwarp();
     const int n_chunks = (x.n_sum + 15) / 16;
     const int cb = (int)((long long)n_chunks * wi / nw), ce = (int)((long long)n_chunks * (wi + 1) / nw);
     x.c0 = (int)((long long)n_chunks * (rank * W) / nw);
@@ -1117,9 +1194,11 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see pdl_begin
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
   if (!ready[dev].load(std::memory_order_acquire)) {       // (two threads may fill it with the same values)
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOne)) != cudaSuccess) return e;
@@ -1157,12 +1236,25 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   cfg.blockDim = dim3((unsigned)(W * 32));
   cfg.dynamicSmemBytes = (size_t)off;
   cfg.stream = stream;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, kern, p, phases, pl);
   count_launch();
   return e;
 }
 
+// The query from mapped host memory into the workspace: 16 bytes per thread, all of them on the bus at once.
+__global__ void __launch_bounds__(256) stage_kernel(const uint4 *src, uint4 *dst, int n) {
+  pdl_begin();
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i < n) dst[i] = src[i];
+}
+
 }  // namespace
+
+cudaError_t launch_stage(const void *src, void *dst, size_t bytes, cudaStream_t stream) {
+  const int n = (int)(bytes / 16);                         // (a whole number of rows of 128 bytes at least)
+  return launch_chained(stage_kernel, dim3((n + 255) / 256), dim3(256), 0, stream, static_cast<const uint4 *>(src), static_cast<uint4 *>(dst), n);
+}
 
 // Whether this kernel covers a configuration's scoring phase: everything but the diagonal-skew variant of FP4 summaries, and
 // units whose scores do not fit a CTA's shared memory.
@@ -1176,9 +1268,9 @@ cudaError_t launch_unit_step(const Params &p, int phases, cudaStream_t stream) {
   if (!(phases & PH_SCORE) || bf16_full)
     return p.D == 128 ? launch_t<Scorer<COBS_SUMM_BF16, 128, 1, 1>, 128>(p, phases, stream) : launch_t<Scorer<COBS_SUMM_BF16, 64, 1, 1>, 64>(p, phases, stream);
   if (p.summ_dtype == COBS_SUMM_FP32)
-    return p.D == 128 ? launch_t<DirectScorer<COBS_SUMM_FP32, 128>, 128>(p, phases, stream) : launch_t<DirectScorer<COBS_SUMM_FP32, 64>, 64>(p, phases, stream);
+    return p.D == 128 ? launch_t<RowScorer<COBS_SUMM_FP32, 128>, 128>(p, phases, stream) : launch_t<RowScorer<COBS_SUMM_FP32, 64>, 64>(p, phases, stream);
   if (p.summ_dtype == COBS_SUMM_BF16)
-    return p.D == 128 ? launch_t<DirectScorer<COBS_SUMM_BF16, 128>, 128>(p, phases, stream) : launch_t<DirectScorer<COBS_SUMM_BF16, 64>, 64>(p, phases, stream);
+    return p.D == 128 ? launch_t<RowScorer<COBS_SUMM_BF16, 128>, 128>(p, phases, stream) : launch_t<RowScorer<COBS_SUMM_BF16, 64>, 64>(p, phases, stream);
   const int wpt = p.Ds_pad / 32;
   if (!p.u_q)
     return p.D == 128 ? launch_t<Scorer<COBS_SUMM_FP4_E2M1, 128, 4, 1>, 128>(p, phases, stream) : launch_t<Scorer<COBS_SUMM_FP4_E2M1, 64, 2, 1>, 64>(p, phases, stream);
