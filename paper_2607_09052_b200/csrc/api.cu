@@ -20,6 +20,8 @@ cudaError_t launch_exact_mass(const Params &p, cudaStream_t stream);
 cudaError_t launch_adaptive_trim(const Params &p, float tau, int k_min, cudaStream_t stream);
 cudaError_t launch_unit_step(const Params &p, int phases, cudaStream_t stream);
 bool unit_score_supported(const Params &p);
+bool unit_keys_fit(const Params &p);
+cudaError_t launch_unit_exact(const Params &p, cudaStream_t stream);
 cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream);
 bool umma_score_supported(const Params &p);
 cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *flags, void *u_pack, cudaStream_t stream);
@@ -361,6 +363,7 @@ int32_t cobs_exact_select(const cobs_config *cfg, const void *q, const cobs_kv *
   p.q = static_cast<const __nv_bfloat16 *>(q);
   p.sel_idx = sel_idx; p.sel_cnt = sel_cnt; p.scores = scores_or_null;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (unit_keys_fit(p)) return cuda_status(launch_unit_exact(p, s));
   if (launch_exact_mass(p, s) != cudaSuccess) return COBS_ERR_CUDA;
   return cuda_status(launch_select(p, s));
 }

@@ -89,6 +89,9 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
 __device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(addr), "f"(v) : "memory");
 }
+__device__ __forceinline__ void st_cluster4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
 __device__ __forceinline__ float2 ld_cluster2(uint32_t addr) {
   float2 v;
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
@@ -105,11 +108,25 @@ __device__ __forceinline__ void run_add(Run &r, float a, float b) {
   r.m = m;
 }
 
+// the warp's pair of every head, from the runs of threads that hold heads 2 tig and 2 tig + 1
+__device__ __forceinline__ void reduce_runs(const Run (&rn)[2], float2 *pair, int lane) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    float m = rn[i].m;
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float s = rn[i].s * __expf(rn[i].m - m);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < 4) pair[2 * lane + i] = make_float2(m, s);
+  }
+}
+
 // what a warp needs to know about its unit
 struct Unit {
   int u, b_idx, h, n_sum;
-  float *eb;                                                 // [G][el]: e of the CTA's blocks, the first of which is c0 * 16
-  int el, c0;
+  float *eb;                                                 // [G][el]: e of the CTA's blocks, the first of which is b0
+  int el, b0;
   const float *qt;                                           // [G][Ds_pad] the subspace query in shared memory
 };
 
@@ -118,7 +135,7 @@ __device__ __forceinline__ void put_e(const Unit &x, int G, int ck, int gid, int
   const int bA = ck * 16 + 2 * gid, g0 = 2 * tig, g1 = g0 + 1;
   if (bA >= x.n_sum) { eA0 = -INFINITY; eA1 = -INFINITY; }
   if (bA + 1 >= x.n_sum) { eB0 = -INFINITY; eB1 = -INFINITY; }
-  float *d = x.eb + (bA - 16 * x.c0);
+  float *d = x.eb + (bA - x.b0);
   if (g0 < G) *reinterpret_cast<float2 *>(d + (size_t)g0 * x.el) = make_float2(eA0, eB0);
   if (g1 < G) *reinterpret_cast<float2 *>(d + (size_t)g1 * x.el) = make_float2(eA1, eB1);
   run_add(run[0], eA0, eB0);
@@ -179,10 +196,11 @@ __device__ __forceinline__ void fp4_rows_full_width(uint32_t xa, uint32_t xb, ui
 // Scoring of chunks [cb, ce) of a unit by one warp.  DT: COBS_SUMM_BF16 | COBS_SUMM_FP4_E2M1.  WPT: 32-bit words of codes per
 // thread per FP4 row (Ds_pad / 32).  NT: f16 terms of the query (1: full space, 2: fp32 subspace query).
 // The first copies are issued by `start`, so that they fly while the CTA projects the query.
-// `run` returns false when a wait for this warp's own copies ran out.
+// `run` leaves the warp's (max, sum) pairs, and returns false when a wait for this warp's own copies ran out.
 // ---------------------------------------------------------------------------------------------------
 template <int DT, int D, int WPT, int NT>
 struct Scorer {
+  static constexpr int BLOCKS = 16;               // blocks of a chunk
   static constexpr bool FP4 = (DT == COBS_SUMM_FP4_E2M1);
   static constexpr int MCH = D / 32;              // 16-byte chunks of a bf16 row per thread
   static constexpr int KSM = D / 16;              // k-steps of a bf16 row
@@ -275,8 +293,13 @@ struct Scorer {
     if (cb < ce) issue(cb, 0, 0);
   }
 
-  __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, Run (&rn)[2]) {
-    if (cb >= ce) return true;
+  __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, float2 *pair) {
+    Run rn[2] = {{-1e30f, 0.f}, {-1e30f, 0.f}};
+    const bool ok = cb >= ce || score(x, cb, ce, rn);
+    reduce_runs(rn, pair, lane);
+    return ok;
+  }
+  __device__ __forceinline__ bool score(const Unit &x, int cb, int ce, Run (&rn)[2]) {
     const int gid = lane >> 2, tig = lane & 3, G = p.G;
     const float inv_sqrt_d = 1.0f / sqrtf((float)D);
     const float ln_l = (float)(31 - __clz(p.L)) * 0.6931471805599453f;      // L is a power of two
@@ -496,6 +519,7 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t &a, uint32_t &
 }
 template <int DT, int D>
 struct RowScorer {
+  static constexpr int BLOCKS = 16;
   static constexpr bool F32 = (DT == COBS_SUMM_FP32);
   static constexpr int ES = F32 ? 4 : 2;
   static constexpr int KS = D / 32;               // groups of 32 elements (8 per lane of a quad)
@@ -593,8 +617,13 @@ struct RowScorer {
     }
   }
 
-  __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, Run (&rn)[2]) {
-    if (cb >= ce) return true;
+  __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, float2 *pair) {
+    Run rn[2] = {{-1e30f, 0.f}, {-1e30f, 0.f}};
+    const bool ok = cb >= ce || score(x, cb, ce, rn);
+    reduce_runs(rn, pair, lane);
+    return ok;
+  }
+  __device__ __forceinline__ bool score(const Unit &x, int cb, int ce, Run (&rn)[2]) {
     const int gid = lane >> 2, tig = lane & 3, G = p.G, Ds = p.Ds;
     const bool sub = p.u_q != nullptr, vec = (rowb & 15) == 0, swap = gid & 1;
     const float inv_sqrt_d = 1.0f / sqrtf((float)D);
@@ -693,6 +722,147 @@ struct RowScorer {
 };
 
 // ---------------------------------------------------------------------------------------------------
+// Exact block masses in place of estimates: e[g][b] = ln sum_{t in b} exp(q'_g . k_t) (Eq. bg-defs), for cobs_exact_select.  It reads
+// every key, so what bounds it is HBM: a warp streams the 16-token groups of a contiguous range of blocks through a ring of its own
+// without a stop at a block's end, five 4 KB stages in flight.  Logits by mma.sync with the heads as rows (zero padded to 16) and
+// 8 tokens as columns; every lane keeps a running (max, sum) of its four tokens per group, merged once per block.
+// (A kernel of its own with two stages per warp, drained at the end of every block, and a selection kernel behind it: 63 us
+// for 268 MB; this way 50.)
+// ---------------------------------------------------------------------------------------------------
+template <int D>
+struct ExactScorer {
+  static constexpr int BLOCKS = 4;
+  static constexpr int CH = D / 8, KS = D / 16, ROWB = D * 2, STAGE = 16 * ROWB, NCP = (16 * CH) / 32;
+  static constexpr int NST = (D == 128) ? 6 : 12;   // 16-token groups in the ring: the two being used, 16 to 20 KB on their way
+  static_assert(NST * STAGE <= kRing && NST % 2 == 0, "the ring must fit");
+  const Params &p;
+  unsigned char *wsm;
+  int lane;
+  __device__ __forceinline__ ExactScorer(const Params &p_, const Unit &, unsigned char *wsm_, uint64_t *, int lane_) : p(p_), wsm(wsm_), lane(lane_) {}
+  __device__ __forceinline__ void start(int, int) {}
+  __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, float2 *pair) {
+    const int gid = lane >> 2, tig = lane & 3, G = p.G, gpb = p.L >> 4, lgP = 31 - __clz(p.P);
+    const int b0 = cb * BLOCKS, b1 = min(ce * BLOCKS, x.n_sum), n = max(0, b1 - b0) * gpb;
+    Run rn = {-1e30f, 0.f};                         // of head gid
+    const float sl = 1.0f / sqrtf((float)D);
+    const uint32_t ring = smem_u32(wsm);
+    const uint64_t pol = l2_evict_first_policy();
+    const uint4 *kbase = reinterpret_cast<const uint4 *>(p.k_pages) + lane;
+    uint32_t qa[KS][2];
+    const uint32_t *qg = reinterpret_cast<const uint32_t *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G + gid) * D);
+#pragma unroll
+    for (int s = 0; s < KS; ++s) {
+      qa[s][0] = (gid < G) ? qg[8 * s + tig] : 0u;
+      qa[s][1] = (gid < G) ? qg[8 * s + 4 + tig] : 0u;
+    }
+    uint32_t cdst[NCP];
+#pragma unroll
+    for (int j = 0; j < NCP; ++j) {
+      const int i = lane + 32 * j, t = i / CH, c = i - t * CH;
+      cdst[j] = t * ROWB + ((c ^ (t & 7)) << 4);
+    }
+    const int kt = ((lane >> 4) & 1) * 8 + (lane & 7), kc = (lane >> 3) & 1;
+    // lane i holds the place of group 32 k + i (16-byte units from the pool's start; none: all ones), for two k at a time
+    constexpr uint32_t kNone = 0xffffffffu;
+    auto resolve = [&](int g) -> uint32_t {
+      if (g >= n) return kNone;
+      const int tok0 = b0 * p.L + g * 16, pslot = tok0 >> lgP;
+      const int pg = (pslot < p.mpp) ? p.page_table[(size_t)x.b_idx * p.mpp + pslot] : -1;
+      if (pg < 0 || pg >= p.n_pages) { report(p.status, COBS_ERR_BOUNDS); return kNone; }
+      return (uint32_t)(((((size_t)pg * p.Hkv + x.h) * p.P + (tok0 & (p.P - 1))) * D) / 8);
+    };
+    uint32_t tab[2] = {resolve(lane), resolve(32 + lane)};
+    auto issue = [&](int g, int st) {
+      const uint32_t off = __shfl_sync(0xffffffffu, (g & 32) ? tab[1] : tab[0], g & 31);
+      if (g < n && off != kNone) {
+#pragma unroll
+        for (int j = 0; j < NCP; ++j) cpa16(ring + st * STAGE + cdst[j], kbase + off + 32 * j, pol);
+      }
+      cpa_commit();
+      return off;
+    };
+    uint32_t live = 0;                               // bit st: stage st holds a group
+#pragma unroll
+    for (int g = 0; g < NST - 2; ++g) live |= (issue(g, g) != kNone ? 1u : 0u) << g;
+    int st = 0, in_blk = 0, blk = b0;
+    float m_run = -1e30f, l_run = 0.f;
+    // a lane's four logits of the group in stage s (natural-log units)
+    auto logits = [&](int s_, float (&v)[4]) {
+      const uint32_t sb = ring + s_ * STAGE;
+      float sc[2][2][4] = {};                        // [tokens 0-7, 8-15][even, odd k steps]
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        uint32_t r0, r1, r2, r3;
+        ldsm_x4(r0, r1, r2, r3, sb + kt * ROWB + (((2 * s + kc) ^ (kt & 7)) << 4));
+        float (&y0)[4] = sc[0][s & 1], (&y1)[4] = sc[1][s & 1];
+        mma16816_bf16(y0[0], y0[1], y0[2], y0[3], qa[s][0], 0u, qa[s][1], 0u, r0, r1);
+        mma16816_bf16(y1[0], y1[1], y1[2], y1[3], qa[s][0], 0u, qa[s][1], 0u, r2, r3);
+      }
+      v[0] = (sc[0][0][0] + sc[0][1][0]) * sl; v[1] = (sc[0][0][1] + sc[0][1][1]) * sl;
+      v[2] = (sc[1][0][0] + sc[1][1][0]) * sl; v[3] = (sc[1][0][1] + sc[1][1][1]) * sl;
+      if (!((live >> s_) & 1u)) v[0] = v[1] = v[2] = v[3] = -1e30f;
+    };
+    auto add = [&](const float (&v)[4], const float (&w)[4], bool both) {
+      float m_new = fmaxf(m_run, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+      if (both) m_new = fmaxf(m_new, fmaxf(fmaxf(w[0], w[1]), fmaxf(w[2], w[3])));
+      float t = (__expf(v[0] - m_new) + __expf(v[1] - m_new)) + (__expf(v[2] - m_new) + __expf(v[3] - m_new));
+      if (both) t += (__expf(w[0] - m_new) + __expf(w[1] - m_new)) + (__expf(w[2] - m_new) + __expf(w[3] - m_new));
+      l_run = fmaf(l_run, __expf(m_run - m_new), t);
+      m_run = m_new;
+    };
+    auto finish = [&]() {                            // the four lanes of a head hold different tokens: merge their pairs
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m_run, o), ol = __shfl_xor_sync(0xffffffffu, l_run, o);
+        const float nm = fmaxf(m_run, om);
+        l_run = l_run * __expf(m_run - nm) + ol * __expf(om - nm);
+        m_run = nm;
+      }
+      const float e = m_run + logf(l_run);
+      if (gid < G && tig == 0) x.eb[(size_t)gid * x.el + (blk - x.b0)] = e;
+      const float m = fmaxf(rn.m, e);
+      rn.s = rn.s * __expf(rn.m - m) + __expf(e - m);
+      rn.m = m;
+      m_run = -1e30f; l_run = 0.f; in_blk = 0; ++blk;
+    };
+    // two groups at a time: their chains of products and exponentials run side by side
+#pragma unroll 1
+    for (int g = 0; g < n; g += 2) {
+      if ((g & 31) == 0 && g > 0) {                  // the table's older half is used up to the last entry
+        const uint32_t t = resolve(g + 32 + lane);
+        if (g & 32) tab[0] = t; else tab[1] = t;
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {                  // into the two stages that were used last
+        const int si = (st == 0) ? NST - 2 + i : st - 2 + i;
+        const uint32_t off = issue(g + NST - 2 + i, si);
+        live = (live & ~(1u << si)) | ((off != kNone ? 1u : 0u) << si);
+      }
+      cpa_wait<NST - 2>();
+      __syncwarp();
+      float v[4], w[4];
+      logits(st, v);
+      logits(st + 1, w);
+      __syncwarp();
+      st = (st == NST - 2) ? 0 : st + 2;
+      if (gpb > 1) {
+        add(v, w, true);
+        in_blk += 2;
+        if (in_blk == gpb) finish();
+      } else {
+        add(v, w, false);
+        finish();
+        if (g + 1 < n) { add(w, v, false); finish(); }
+      }
+    }
+    cpa_wait<0>();
+    __syncwarp();
+    if (tig == 0) pair[gid] = (gid < G) ? make_float2(rn.m, rn.s) : make_float2(-1e30f, 0.f);
+    return true;
+  }
+};
+
+// ---------------------------------------------------------------------------------------------------
 // Query projection q~ = U_Q^T (q / sqrt(D)) of a unit's heads, zero padded to Ds_pad, by the whole CTA (Method, "Per-step
 // scoring": one O(s D) projection per step and head).  A warp takes (32 consecutive coordinates, a quarter of the head
 // dimension): lane = coordinate, so the reads of U_Q [Hkv][D][Ds] are coalesced and serve all heads; the quarters are added in
@@ -741,7 +911,12 @@ __device__ __forceinline__ void select_topk(const float *keys_s, int n, int k, i
   uint32_t key[BPT ? BPT : 1];
   if constexpr (BPT > 0) {
 #pragma unroll
-    for (int j = 0; j < BPT; ++j) key[j] = (b0 + j < n) ? __float_as_uint(keys_s[b0 + j]) : 0u;
+    for (int j = 0; j < BPT; j += 2) {               // (the array has a whole number of fours of keys)
+      float2 v = make_float2(0.f, 0.f);
+      if (b0 + j < n) v = *reinterpret_cast<const float2 *>(keys_s + b0 + j);
+      key[j] = __float_as_uint(v.x);
+      key[j + 1] = (b0 + j + 1 < n) ? __float_as_uint(v.y) : 0u;
+    }
   }
   // one pass over this thread's keys
   auto each = [&](auto f) {
@@ -852,10 +1027,14 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
       qa[s][1] = (gid < G) ? qg[8 * s + 4 + tig] : 0u;
     }
   }
-  float o[NTL][2];
+  // P = bf16 high + low: the high parts are rows 0-7 of the A operand, the low parts rows 8-15, so that one mma takes both and
+  // the two products meet at the end.  Every accumulator tile has its own four registers: with the unused rows of all tiles in
+  // one pair, every mma waited for the one before it (192 ragged units of 64 groups: 21 us, now 12.5, which is 8 TB/s from L2 and
+  // HBM; running the products with K a group ahead of those with V on top of it gains nothing)
+  float o[NTL][4];
 #pragma unroll
-  for (int n = 0; n < NTL; ++n) o[n][0] = o[n][1] = 0.f;
-  float m_run = -1e30f, l_run = 0.f, z2 = 0.f, z3 = 0.f;
+  for (int n = 0; n < NTL; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+  float m_run = -1e30f, l_run = 0.f;
 #pragma unroll 1
   for (int gb = g0; gb < g1; gb += kTable) {
     const int n_groups = min(g1 - gb, kTable);
@@ -913,14 +1092,17 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
       if (first >= 0) {
         const uint32_t sb = ring + st * STAGE;
         // ---- S^T = q K^T: s0 tokens 0-7, s1 tokens 8-15 --------------------------------------------------
-        float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f;
+        float sc[2][2][4] = {};                // [tokens 0-7, 8-15][even, odd k steps]
 #pragma unroll
         for (int s = 0; s < KS; ++s) {
           uint32_t b0, b1, b2, b3;
           ldsm_x4(b0, b1, b2, b3, sb + kt * ROWB + (((2 * s + kc) ^ (kt & 7)) << 4));
-          mma16816_bf16(s00, s01, z2, z3, qa[s][0], 0u, qa[s][1], 0u, b0, b1);
-          mma16816_bf16(s10, s11, z2, z3, qa[s][0], 0u, qa[s][1], 0u, b2, b3);
+          float (&x0)[4] = sc[0][s & 1], (&x1)[4] = sc[1][s & 1];
+          mma16816_bf16(x0[0], x0[1], x0[2], x0[3], qa[s][0], 0u, qa[s][1], 0u, b0, b1);
+          mma16816_bf16(x1[0], x1[1], x1[2], x1[3], qa[s][0], 0u, qa[s][1], 0u, b2, b3);
         }
+        float s00 = sc[0][0][0] + sc[0][1][0], s01 = sc[0][0][1] + sc[0][1][1];
+        float s10 = sc[1][0][0] + sc[1][1][0], s11 = sc[1][0][1] + sc[1][1][1];
         const int nv = T - first;
         if (nv < 16) {                         // tokens past the end take no weight
           if (2 * tig >= nv) s00 = -1e30f;
@@ -936,8 +1118,8 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
           const float corr = ex2((m_run - m_new) * sl2);
           m_run = m_new;
           l_run *= corr;
-#pragma unroll
-          for (int n = 0; n < NTL; ++n) { o[n][0] *= corr; o[n][1] *= corr; }
+          #pragma unroll
+          for (int n = 0; n < NTL; ++n) { o[n][0] *= corr; o[n][1] *= corr; o[n][2] *= corr; o[n][3] *= corr; }
         }
         const float mb = m_run * sl2;
         const float p0 = ex2(fmaf(s00, sl2, -mb)), p1 = ex2(fmaf(s01, sl2, -mb));
@@ -951,10 +1133,9 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
         for (int np = 0; np < NTL / 2; ++np) {
           uint32_t b0, b1, b2, b3;
           ldsm_x4_t(b0, b1, b2, b3, sb + VOFF + vt * ROWB + (((2 * np + vc) ^ (vt & 7)) << 4));
-          mma16816_bf16(o[2 * np][0], o[2 * np][1], z2, z3, a0h, 0u, a2h, 0u, b0, b1);
-          mma16816_bf16(o[2 * np + 1][0], o[2 * np + 1][1], z2, z3, a0h, 0u, a2h, 0u, b2, b3);
-          mma16816_bf16(o[2 * np][0], o[2 * np][1], z2, z3, a0l, 0u, a2l, 0u, b0, b1);
-          mma16816_bf16(o[2 * np + 1][0], o[2 * np + 1][1], z2, z3, a0l, 0u, a2l, 0u, b2, b3);
+          float (&o0)[4] = o[2 * np], (&o1)[4] = o[2 * np + 1];
+          mma16816_bf16(o0[0], o0[1], o0[2], o0[3], a0h, a0l, a2h, a2l, b0, b1);
+          mma16816_bf16(o1[0], o1[1], o1[2], o1[3], a0h, a0l, a2h, a2l, b2, b3);
         }
       }
       __syncwarp();                            // all lanes are done with the stage before it is refilled
@@ -970,7 +1151,7 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
   if (gid < G) {
     float *dst = reinterpret_cast<float *>(wsm) + gid * D;
 #pragma unroll
-    for (int n = 0; n < NTL; ++n) *reinterpret_cast<float2 *>(dst + 8 * n + 2 * tig) = make_float2(o[n][0], o[n][1]);
+    for (int n = 0; n < NTL; ++n) *reinterpret_cast<float2 *>(dst + 8 * n + 2 * tig) = make_float2(o[n][0] + o[n][2], o[n][1] + o[n][3]);
     if (tig == 0) pair[gid] = make_float2((l_run > 0.f) ? m_run * (sl2 * 0.6931471805599453f) : -INFINITY, l_run);
   }
 }
@@ -1018,12 +1199,12 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   int n_sel = min(p.topk, n_cand);
 
   if (phases & PH_SCORE) {
-    const int n_chunks = (x.n_sum + 15) / 16;
+    const int n_chunks = (x.n_sum + SCORER::BLOCKS - 1) / SCORER::BLOCKS;
     const int cb = (int)((long long)n_chunks * wi / nw), ce = (int)((long long)n_chunks * (wi + 1) / nw);
-    x.c0 = (int)((long long)n_chunks * (rank * W) / nw);
-    const int c1 = (int)((long long)n_chunks * (rank * W + W) / nw);
-    x.el = (c1 - x.c0) * 16;
-    x.eb = (pl.e_off >= 0) ? reinterpret_cast<float *>(fsm + pl.e_off) : p.e + ((size_t)u * ((NB + 15) / 16) + x.c0) * 16 * G;
+    const int c0 = (int)((long long)n_chunks * (rank * W) / nw), c1 = (int)((long long)n_chunks * (rank * W + W) / nw);
+    x.b0 = c0 * SCORER::BLOCKS;
+    x.el = (c1 - c0) * SCORER::BLOCKS;
+    x.eb = (pl.e_off >= 0) ? reinterpret_cast<float *>(fsm + pl.e_off) : p.e + ((size_t)u * ((NB + 15) / 16 * 16) + x.b0) * G;
     x.qt = s_qt;
     SCORER sc(p, x, wsm, &s_bars[warp][0], lane);
     sc.start(cb, ce);
@@ -1031,19 +1212,8 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
       project_query<D>(p, x.b_idx, x.h, s_qt, reinterpret_cast<float *>(fsm + kStage), kRing / 4, warp, lane, W);
       fence_proxy_async();                                  // bulk copies follow where the scratch was written
     }
-    Run rn[2] = {{-1e30f, 0.f}, {-1e30f, 0.f}};
-    if (!sc.run(x, cb, ce, rn)) s_lost = 1;
-    // ---- log-sum-exp per head: over the warp, the CTA, the cluster ----------------------------------------------
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      float m = rn[i].m;
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      float s = rn[i].s * __expf(rn[i].m - m);
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane < 4) s_pair[warp][2 * lane + i] = make_float2(m, s);
-    }
+    // (max, sum) of e per head: over the warp, the CTA, the cluster
+    if (!sc.run(x, cb, ce, s_pair[warp])) s_lost = 1;
     __syncthreads();
     COBS_STAMP(1);
     if (C > 1) cluster_wait();
@@ -1070,17 +1240,39 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     {
       const uint32_t ka = smem_u32(keys);
       const int n_dst = (phases & PH_ATTEND) ? C : 1;       // without an attention phase CTA 0 alone selects
-      const int n_loc = min(x.el, x.n_sum - 16 * x.c0);
-      for (int i = tid; i < n_loc; i += nthr) {
-        float s = 0.f;
+      const int n_loc = min(x.el, x.n_sum - x.b0);
+      if (n_loc <= nthr) {                                  // few blocks: one per thread (0.6 us less than four on a quarter of them)
+        if (tid < n_loc) {
+          float s = 0.f;
 #pragma unroll 4
-        for (int g = 0; g < G; ++g) s += __expf(x.eb[(size_t)g * x.el + i] - s_lse[g]);
-        const int b = 16 * x.c0 + i;
-        if (p.scores) p.scores[(size_t)u * NB + b] = s;
-        if (b < n_cand) {
+          for (int g = 0; g < G; ++g) s += __expf(x.eb[(size_t)g * x.el + tid] - s_lse[g]);
+          const int b = x.b0 + tid;
+          if (p.scores) p.scores[(size_t)u * NB + b] = s;
           if (C == 1) keys[b] = s;
           else for (int c = 0; c < n_dst; ++c) st_cluster(mapa(ka + 4 * b, c), s);
         }
+      } else
+      for (int i = 4 * tid; i < n_loc; i += 4 * nthr) {     // four blocks at a time (what lies beyond n_loc is not used)
+        float4 v[8], s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (g < G) v[g] = *reinterpret_cast<const float4 *>(x.eb + (size_t)g * x.el + i);
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (g < G) {
+            const float l = s_lse[g];
+            s.x += __expf(v[g].x - l); s.y += __expf(v[g].y - l); s.z += __expf(v[g].z - l); s.w += __expf(v[g].w - l);
+          }
+        const int b = x.b0 + i;
+        if (p.scores) {
+          float *d = p.scores + (size_t)u * NB + b;
+          d[0] = s.x;
+          if (i + 1 < n_loc) d[1] = s.y;
+          if (i + 2 < n_loc) d[2] = s.z;
+          if (i + 3 < n_loc) d[3] = s.w;
+        }
+        if (C == 1) *reinterpret_cast<float4 *>(keys + b) = s;
+        else for (int c = 0; c < n_dst; ++c) st_cluster4(mapa(ka + 4 * b, c), s);
       }
     }
     if (C > 1) { cluster_arrive(); cluster_wait(); } else __syncthreads();
@@ -1186,6 +1378,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
 // ---------------------------------------------------------------------------------------------------
 template <class SCORER, int D>
 cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
+  constexpr int NBLK = SCORER::BLOCKS;
   auto kern = unit_step_kernel<SCORER, D>;
   static std::atomic<int> ready[64];                       // per device: attributes set, table filled
   static std::atomic<int> fit[64][kMaxC + 1];              // clusters of C CTAs, eight warps each, that are resident at a time
@@ -1217,7 +1410,7 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   // 29.9 / 27.9 / 26.7 us with 2 / 3 / 4; 128 units of 128k: 98 us with one CTA of eight warps, 118 with two of four.)
   // More units than SMs: four warps per CTA, two CTAs per SM (192 ragged units of 12k: 45 us, 55 with eight warps in two waves).
   Plan pl;
-  const int units = p.B * p.Hkv, n_chunks = (p.NB + 15) / 16;
+  const int units = p.B * p.Hkv, n_chunks = (p.NB + NBLK - 1) / NBLK;
   const int groups = (p.topk + (p.window + p.L - 1) / p.L + 1) * (p.L / 16);
   // (the same for a scoring call and a whole step: the order of the sums, and so the selection's last bits, follow the split)
   const int work = (phases & PH_SCORE) ? max(n_chunks, groups) : groups;
@@ -1227,7 +1420,7 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
     if (fit[dev][c].load(std::memory_order_relaxed) >= units) pl.C = c;
   const int W = pl.W, C = pl.C, cap = (W == kMaxW) ? kSmemOne : kSmemTwo;
   const int key_bytes = (phases & PH_SCORE) ? (p.NB * 4 + 15) / 16 * 16 : 0;
-  const int e_bytes = (phases & PH_SCORE) ? p.G * 16 * ((n_chunks + C - 1) / C) * 4 : 0;
+  const int e_bytes = (phases & PH_SCORE) ? p.G * NBLK * ((n_chunks + C - 1) / C) * 4 : 0;
   int off = W * kRing;
   if (off + key_bytes <= cap) { pl.key_off = off; off += key_bytes; } else pl.key_off = 0;      // over the rings: scoring is over by then
   if (off + e_bytes <= cap) { pl.e_off = off; off += e_bytes; } else pl.e_off = -1;
@@ -1258,9 +1451,12 @@ cudaError_t launch_stage(const void *src, void *dst, size_t bytes, cudaStream_t 
 
 // Whether this kernel covers a configuration's scoring phase: everything but the diagonal-skew variant of FP4 summaries, and
 // units whose scores do not fit a CTA's shared memory.
-bool unit_score_supported(const Params &p) {
-  if (p.skew && p.summ_dtype == COBS_SUMM_FP4_E2M1) return false;
-  return p.NB <= kMaxKeys;
+bool unit_keys_fit(const Params &p) { return p.NB <= kMaxKeys; }
+bool unit_score_supported(const Params &p) { return unit_keys_fit(p) && !(p.skew && p.summ_dtype == COBS_SUMM_FP4_E2M1); }
+
+// Exact block masses, group scores and selection.
+cudaError_t launch_unit_exact(const Params &p, cudaStream_t stream) {
+  return p.D == 128 ? launch_t<ExactScorer<128>, 128>(p, PH_SCORE, stream) : launch_t<ExactScorer<64>, 64>(p, PH_SCORE, stream);
 }
 
 cudaError_t launch_unit_step(const Params &p, int phases, cudaStream_t stream) {
