@@ -30,7 +30,6 @@ cudaError_t launch_append(const Params &p, const void *k_new, const void *v_new,
 cudaError_t launch_quantise(const float *xi, long long n_vectors, int Ds, int Ds_pad, int scale_dtype, void *codes,
                             void *scale, cudaStream_t stream);
 size_t build_smem_bytes(const Params &p);
-cudaError_t launch_stage(const void *src, void *dst, size_t bytes, cudaStream_t stream);
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -451,28 +450,20 @@ int32_t cobs_decode_step_host(const cobs_config *cfg, const void *q_host, const 
   float *out_dev = reinterpret_cast<float *>(base + w.out_stage);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t n = (size_t)cfg->batch * cfg->n_q_heads * cfg->head_dim, units = (size_t)cfg->batch * cfg->n_kv_heads;
-  // Pinned, device-mapped memory is read and written in place: the query by a small kernel that the step is chained to (a
-  // copy-engine transfer and the hand-over to it cost more than the 131 KB over the bus), the output rows and the selection
-  // by posted writes of the step kernel, which saves their copies after it.  Any other host memory goes through copies.
-  const void *q_map = mapped(q_host);
+  // Pinned, device-mapped memory is used in place by the cluster kernel: its CTAs fetch their unit's query from it once (2 KB;
+  // 131 KB through a copy or a staging kernel in front of the step took 6 us and more), output rows and selection are posted
+  // writes.  The other kernels read the query often and the selection back; they, and any other host memory, get copies.
+  Params p;
+  fill_params(p, cfg, workspace);
+  if ((st = set_summaries(p, cfg, summ)) != COBS_OK) return st;
+  const bool in_place = unit_score_supported(p) && !umma_score_supported(p);
+  const void *q_map = in_place ? mapped(q_host) : nullptr;
+  if (!q_map && cudaMemcpyAsync(q_dev, q_host, n * 2, cudaMemcpyHostToDevice, s) != cudaSuccess) return COBS_ERR_CUDA;
   float *out_map = static_cast<float *>(mapped(out_host));
-  if (q_map) {
-    if (launch_stage(q_map, q_dev, n * 2, s) != cudaSuccess) return COBS_ERR_CUDA;
-  } else if (cudaMemcpyAsync(q_dev, q_host, n * 2, cudaMemcpyHostToDevice, s) != cudaSuccess) {
-    return COBS_ERR_CUDA;
-  }
-  int32_t *sel_map = nullptr, *cnt_map = nullptr;
-  if (sel_idx_host_or_null) {
-    Params p;
-    fill_params(p, cfg, workspace);
-    if ((st = set_summaries(p, cfg, summ)) != COBS_OK) return st;
-    if (unit_score_supported(p) && !umma_score_supported(p)) {       // (the other paths read the selection back)
-      sel_map = static_cast<int32_t *>(mapped(sel_idx_host_or_null));
-      cnt_map = static_cast<int32_t *>(mapped(sel_cnt_host_or_null));
-    }
-  }
+  int32_t *sel_map = (in_place && sel_idx_host_or_null) ? static_cast<int32_t *>(mapped(sel_idx_host_or_null)) : nullptr;
+  int32_t *cnt_map = sel_map ? static_cast<int32_t *>(mapped(sel_cnt_host_or_null)) : nullptr;
   const bool sel_direct = sel_map && cnt_map;
-  st = cobs_decode_step(cfg, q_dev, kv, summ, out_map ? out_map : out_dev, nullptr, sel_direct ? sel_map : nullptr,
+  st = cobs_decode_step(cfg, q_map ? q_map : q_dev, kv, summ, out_map ? out_map : out_dev, nullptr, sel_direct ? sel_map : nullptr,
                         sel_direct ? cnt_map : nullptr, workspace, workspace_bytes, stream);
   if (st != COBS_OK) return st;
   if (!out_map && cudaMemcpyAsync(out_host, out_dev, n * sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)

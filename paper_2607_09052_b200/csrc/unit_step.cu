@@ -7,6 +7,7 @@
 // (about a microsecond each less than a counter in global memory with its fences), there is nothing to poll, no counter to
 // clear, no order in which CTAs must run, and a grid of any size.
 //
+//   query    each CTA fetches its unit's 2 KB of query once, into shared memory (the caller's may lie in host memory)
 //   score    the unit's 16-block chunks are dealt to the cluster's warps in contiguous ranges; a warp leaves e per block and
 //            head in its CTA's buffer and keeps a running (max, sum) per head
 //   lse      the CTAs exchange their (max, sum) pairs                                        (cluster barrier)
@@ -19,7 +20,8 @@
 // one sequence of 32k 31.9 -> 20.5, four of 32k with a subspace 37.0 -> 26.7, sixteen of 128k 115 -> 98 (80 % of the measured
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
 // summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
-// search: 17.1, 23.4, 95-98, 43.5, 16.9.
+// search: 17.1, 23.4, 95-98, 43.5, 16.9; with the attention's accumulators apart and the query in shared memory: 16.1, 20.9,
+// 93, 35.2, 16.4.
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
 // chunk is three contiguous pieces of the summary arrays, fetched by three bulk copies (cp.async.bulk, completion on an
@@ -69,8 +71,9 @@ constexpr int kTable = 128;                                  // 16-token groups 
 constexpr int kRing = 2 * kStage;                            // 26112 bytes per warp
 static_assert(kAttStages * kAttStage + kTable * 8 <= kRing, "the attention ring and its table must fit");
 constexpr int kCtaPart = 8192;                               // offset of the CTA's merged partial in warp 0's ring (its own partial: below)
-constexpr int kSmemOne = (227 - 8) * 1024;                   // dynamic shared memory of a CTA that has an SM to itself (static: 6.7 KB)
-constexpr int kSmemTwo = 108544;                             // of two CTAs per SM (four warps each)
+constexpr int kSmemOne = (227 - 9) * 1024;                   // dynamic shared memory of a CTA that has an SM to itself (static: 8960 bytes)
+constexpr int kSmemTwo = 106752;                             // of two CTAs per SM (four warps each)
+constexpr int kQRow = 128 + 8;                               // row stride of the query in shared memory (no bank conflicts)
 constexpr int kMaxKeys = 24576;                              // score keys that fit over the rings of four warps
 
 // how a launch lays out a CTA (chosen on the host, see launch_t)
@@ -127,6 +130,7 @@ struct Unit {
   int u, b_idx, h, n_sum;
   float *eb;                                                 // [G][el]: e of the CTA's blocks, the first of which is b0
   int el, b0;
+  const __nv_bfloat16 *q;                                    // [G][kQRow] the raw query in shared memory
   const float *qt;                                           // [G][Ds_pad] the subspace query in shared memory
 };
 
@@ -308,11 +312,10 @@ struct Scorer {
     uint32_t bq[FP4 ? NT : 1][KSQ][2];
     float m0 = 0.f, m1 = 0.f;
     {
-      const __nv_bfloat16 *qg = p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D;
 #pragma unroll
       for (int m = 0; m < KSM / 2; ++m) {
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (gid < G) v = *reinterpret_cast<const uint4 *>(qg + gid * D + (tig + 4 * m) * 8);
+        if (gid < G) v = *reinterpret_cast<const uint4 *>(x.q + gid * kQRow + (tig + 4 * m) * 8);
         bm[2 * m][0] = v.x; bm[2 * m][1] = v.y; bm[2 * m + 1][0] = v.z; bm[2 * m + 1][1] = v.w;
       }
       if (FP4) {
@@ -330,7 +333,7 @@ struct Scorer {
             e[j][4] = hi.x; e[j][5] = hi.y; e[j][6] = hi.z; e[j][7] = hi.w;
           } else {
             uint4 v = make_uint4(0, 0, 0, 0);
-            if (gid < G) v = *reinterpret_cast<const uint4 *>(qg + gid * D + tig * (WPT * 8) + j * 8);
+            if (gid < G) v = *reinterpret_cast<const uint4 *>(x.q + gid * kQRow + tig * (WPT * 8) + j * 8);
             e[j][0] = bf16_lo(v.x); e[j][1] = bf16_hi(v.x); e[j][2] = bf16_lo(v.y); e[j][3] = bf16_hi(v.y);
             e[j][4] = bf16_lo(v.z); e[j][5] = bf16_hi(v.z); e[j][6] = bf16_lo(v.w); e[j][7] = bf16_hi(v.w);
           }
@@ -629,11 +632,10 @@ struct RowScorer {
     const float inv_sqrt_d = 1.0f / sqrtf((float)D);
     const float ln_l = (float)(31 - __clz(p.L)) * 0.6931471805599453f;
     uint32_t bm[KS][4], bs[3][KS][4];               // the raw query; the subspace query in three bf16 terms
-    const __nv_bfloat16 *qg = p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D;
 #pragma unroll
     for (int m = 0; m < KS; ++m) {
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (gid < G) v = *reinterpret_cast<const uint4 *>(qg + gid * D + (tig + 4 * m) * 8);
+      if (gid < G) v = *reinterpret_cast<const uint4 *>(x.q + gid * kQRow + (tig + 4 * m) * 8);
       bm[m][0] = v.x; bm[m][1] = v.y; bm[m][2] = v.z; bm[m][3] = v.w;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -749,7 +751,7 @@ struct ExactScorer {
     const uint64_t pol = l2_evict_first_policy();
     const uint4 *kbase = reinterpret_cast<const uint4 *>(p.k_pages) + lane;
     uint32_t qa[KS][2];
-    const uint32_t *qg = reinterpret_cast<const uint32_t *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G + gid) * D);
+    const uint32_t *qg = reinterpret_cast<const uint32_t *>(x.q + gid * kQRow);
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
       qa[s][0] = (gid < G) ? qg[8 * s + tig] : 0u;
@@ -869,25 +871,25 @@ struct ExactScorer {
 // a fixed order.  qt: [G][Ds_pad] result; part: scratch of 4 KB per quarter, `stride` floats apart.
 // ---------------------------------------------------------------------------------------------------
 template <int D>
-__device__ __forceinline__ void project_query(const Params &p, int b_idx, int h, float *qt, float *part, int stride, int warp, int lane, int W) {
+__device__ __forceinline__ void project_query(const Params &p, const Unit &x, float *qt, float *part, int stride, int warp, int lane, int W) {
   constexpr int DQ = D / 4;
   const int nsb = (p.Ds_pad + 31) / 32, G = p.G;
   const float inv_sqrt_d = 1.0f / sqrtf((float)D);
   for (int t = warp; t < 4 * nsb; t += W) {
     const int sb = t >> 2, quarter = t & 3, s = sb * 32 + lane;
     const bool live = s < p.Ds;
-    const float *uq = p.u_q + ((size_t)h * D + quarter * DQ) * p.Ds + (live ? s : 0);
-    float x[DQ];
+    const float *uq = p.u_q + ((size_t)x.h * D + quarter * DQ) * p.Ds + (live ? s : 0);
+    float v[DQ];
 #pragma unroll
-    for (int j = 0; j < DQ; ++j) x[j] = live ? __ldg(uq + (size_t)j * p.Ds) : 0.f;
+    for (int j = 0; j < DQ; ++j) v[j] = live ? __ldg(uq + (size_t)j * p.Ds) : 0.f;
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
-      const __nv_bfloat16 *q = p.q + ((size_t)b_idx * p.Hq + h * G + g) * D + quarter * DQ;
+      const __nv_bfloat16 *q = x.q + g * kQRow + quarter * DQ;
       const float qv = (lane < DQ) ? __bfloat162float(q[lane]) * inv_sqrt_d : 0.f;
-      float v = 0.f;
+      float a = 0.f;
 #pragma unroll
-      for (int j = 0; j < DQ; ++j) v = fmaf(x[j], __shfl_sync(0xffffffffu, qv, j), v);
-      part[quarter * stride + g * 128 + s] = v;
+      for (int j = 0; j < DQ; ++j) a = fmaf(v[j], __shfl_sync(0xffffffffu, qv, j), a);
+      part[quarter * stride + g * 128 + s] = a;
     }
   }
   __syncthreads();
@@ -1020,7 +1022,7 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
   // query fragments: rows = heads (zero padded to 16), natural k order
   uint32_t qa[KS][2];
   {
-    const uint32_t *qg = reinterpret_cast<const uint32_t *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G + gid) * D);
+    const uint32_t *qg = reinterpret_cast<const uint32_t *>(x.q + gid * kQRow);
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
       qa[s][0] = (gid < G) ? qg[8 * s + tig] : 0u;
@@ -1167,6 +1169,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   __shared__ __align__(16) float2 s_cpair[kMaxC][8];       // per CTA of the cluster and head: (max, sum) of e
   __shared__ __align__(16) float2 s_opair[8];              // the CTA's (max, sum) of the attention logits
   __shared__ float s_lse[8];
+  __shared__ __align__(16) __nv_bfloat16 s_q[8 * kQRow];
   __shared__ __align__(16) float s_qt[8 * 128];
   __shared__ uint32_t s_cnt[2][2][kMaxW];
   __shared__ int s_scan[kMaxW];
@@ -1189,6 +1192,12 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   COBS_STAMP(0);
   Unit x;
   x.u = u; x.b_idx = u / p.Hkv; x.h = u - x.b_idx * p.Hkv;
+  x.q = s_q;
+  // the unit's query, once per CTA (it may lie in host memory): needed behind the next barrier
+  if (tid < G * (D / 8)) {
+    const int g = tid / (D / 8), c = tid - g * (D / 8);
+    *reinterpret_cast<uint4 *>(s_q + g * kQRow + 8 * c) = reinterpret_cast<const uint4 *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D)[tid];
+  }
   const int T = p.seq_lens[x.b_idx];
   x.n_sum = min(T / L, NB);
   const int ws = window_start(T, p.window, L);
@@ -1208,8 +1217,9 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     x.qt = s_qt;
     SCORER sc(p, x, wsm, &s_bars[warp][0], lane);
     sc.start(cb, ce);
+    __syncthreads();
     if (p.u_q) {                                            // (scratch: the second stages of four rings, not in use yet)
-      project_query<D>(p, x.b_idx, x.h, s_qt, reinterpret_cast<float *>(fsm + kStage), kRing / 4, warp, lane, W);
+      project_query<D>(p, x, s_qt, reinterpret_cast<float *>(fsm + kStage), kRing / 4, warp, lane, W);
       fence_proxy_async();                                  // bulk copies follow where the scratch was written
     }
     // (max, sum) of e per head: over the warp, the CTA, the cluster
@@ -1435,19 +1445,7 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   return e;
 }
 
-// The query from mapped host memory into the workspace: 16 bytes per thread, all of them on the bus at once.
-__global__ void __launch_bounds__(256) stage_kernel(const uint4 *src, uint4 *dst, int n) {
-  pdl_begin();
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i < n) dst[i] = src[i];
-}
-
 }  // namespace
-
-cudaError_t launch_stage(const void *src, void *dst, size_t bytes, cudaStream_t stream) {
-  const int n = (int)(bytes / 16);                         // (a whole number of rows of 128 bytes at least)
-  return launch_chained(stage_kernel, dim3((n + 255) / 256), dim3(256), 0, stream, static_cast<const uint4 *>(src), static_cast<uint4 *>(dst), n);
-}
 
 // Whether this kernel covers a configuration's scoring phase: everything but the diagonal-skew variant of FP4 summaries, and
 // units whose scores do not fit a CTA's shared memory.
