@@ -122,6 +122,12 @@ __device__ __forceinline__ void reduce_runs(const Run (&rn)[2], float2 *pair, in
   }
 }
 
+// the first of n items that falls to worker i of w: floor(n i / w) without a 64-bit division (w <= 128)
+__device__ __forceinline__ int share(int n, int i, int w) {
+  const unsigned q = (unsigned)n / (unsigned)w, r = (unsigned)n - q * (unsigned)w;
+  return (int)(q * (unsigned)i + r * (unsigned)i / (unsigned)w);
+}
+
 // what a warp needs to know about its unit
 struct Unit {
   int u, b_idx, h, n_sum;
@@ -1189,12 +1195,16 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   Unit x;
   x.u = u; x.b_idx = u / p.Hkv; x.h = u - x.b_idx * p.Hkv;
   x.q = s_q;
-  // the unit's query, once per CTA (it may lie in host memory): needed behind the next barrier
-  if (tid < G * (D / 8)) {
-    const int g = tid / (D / 8), c = tid - g * (D / 8);
-    *reinterpret_cast<uint4 *>(s_q + g * kQRow + 8 * c) = reinterpret_cast<const uint4 *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D)[tid];
-  }
+  // the unit's query, once per CTA (it may lie in host memory): needed behind the next barrier, stored only when the first copies
+  // of the summaries, which wait for the length, are on their way
   const int T = p.seq_lens[x.b_idx];
+  const bool has_q = tid < G * (D / 8);
+  uint4 qv = make_uint4(0u, 0u, 0u, 0u);
+  if (has_q) qv = reinterpret_cast<const uint4 *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D)[tid];
+  auto store_q = [&]() {
+    const int g = tid / (D / 8), c = tid - g * (D / 8);
+    if (has_q) *reinterpret_cast<uint4 *>(s_q + g * kQRow + 8 * c) = qv;
+  };
   x.n_sum = min(T / L, NB);
   const int ws = window_start(T, p.window, L);
   const int n_cand = (phases & PH_SCORE) ? min(ws / L, x.n_sum) : ws / L;
@@ -1205,14 +1215,15 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
 
   if (phases & PH_SCORE) {
     const int n_chunks = (x.n_sum + SCORER::BLOCKS - 1) / SCORER::BLOCKS;
-    const int cb = (int)((long long)n_chunks * wi / nw), ce = (int)((long long)n_chunks * (wi + 1) / nw);
-    const int c0 = (int)((long long)n_chunks * (rank * W) / nw), c1 = (int)((long long)n_chunks * (rank * W + W) / nw);
+    const int cb = share(n_chunks, wi, nw), ce = share(n_chunks, wi + 1, nw);
+    const int c0 = share(n_chunks, rank * W, nw), c1 = share(n_chunks, rank * W + W, nw);
     x.b0 = c0 * SCORER::BLOCKS;
     x.el = (c1 - c0) * SCORER::BLOCKS;
     x.eb = (pl.e_off >= 0) ? reinterpret_cast<float *>(fsm + pl.e_off) : p.e + ((size_t)u * ((NB + 15) / 16 * 16) + x.b0) * G;
     x.qt = s_qt;
     SCORER sc(p, x, wsm, &s_bars[warp][0], lane);
     sc.start(cb, ce);
+    store_q();
     __syncthreads();
     if (p.u_q) {                                            // (scratch: the second stages of four rings, not in use yet)
       project_query<D>(p, x, s_qt, reinterpret_cast<float *>(fsm + kStage), kRing / 4, warp, lane, W);
@@ -1304,6 +1315,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   } else {
     n_sel = max(0, min(n_sel, p.sel_cnt[u]));
     for (int i = tid; i < n_sel; i += nthr) s_sel[i] = p.sel_idx[(size_t)u * p.topk + i];
+    store_q();
     if (C > 1) cluster_wait();
     __syncthreads();
   }
@@ -1311,7 +1323,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   // ---- attention: the unit's groups dealt to the cluster's warps ---------------------------------------------------
   {
     const int n_groups = s_lost ? 0 : (n_sel + n_win) * (L >> 4);
-    attend_groups<D>(p, x, T, n_cand, ws / L, n_sel, s_sel, wsm, (int)((long long)n_groups * wi / nw), (int)((long long)n_groups * (wi + 1) / nw),
+    attend_groups<D>(p, x, T, n_cand, ws / L, n_sel, s_sel, wsm, share(n_groups, wi, nw), share(n_groups, wi + 1, nw),
                      s_pair[warp], lane);
   }
   __syncthreads();
