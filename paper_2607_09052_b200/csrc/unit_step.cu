@@ -21,7 +21,8 @@
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
 // summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
 // search: 17.1, 23.4, 95-98, 43.5, 16.9; with the attention's accumulators apart and the query in shared memory: 16.1, 20.9,
-// 93, 35.2, 16.4.
+// 93, 35.2, 16.4; with the merge by stores and the first loads together: 15.3, 19.8, 93, 35.2, 13.9.  (One exchange of pairs and
+// e, every CTA computing all scores, instead of pairs first and scores after: 15.4, 20.3, 93, 35.1, 13.6: not kept.)
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
 // chunk is three contiguous pieces of the summary arrays, fetched by three bulk copies (cp.async.bulk, completion on an
@@ -515,7 +516,7 @@ struct Scorer {
 // on any element; a block's rows are fetched by one bulk copy of the 16-byte units that hold them, in batches of as many rows
 // as fit a stage, and read back 16 bytes or (rows that are no multiple of 16 bytes) one element at a time.
 // (Reading them straight from global memory, one row of 16 blocks in flight per warp, took 1366 us for 2.4 GB of fp32 summaries,
-// 288 units; this way 688.  A single sequence of 2k does not gain: 16.9 us, 15.7 that way.)
+// 288 units; this way 688.)
 // ---------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void split3(float x, float y, uint32_t &a, uint32_t &b, uint32_t &c) {
   a = bf16x2(x, y);
@@ -589,6 +590,9 @@ struct RowScorer {
     if (bytes) bulk_g2s(dst, src, bytes, bar, pol);
   }
   __device__ __forceinline__ void start(int cb, int ce) {
+    // a single chunk has the whole ring: one wait instead of one per batch (one sequence of 2k: 15.5 -> 13.9 us; not with a
+    // subspace, whose query is projected in the second stage)
+    if (ce - cb == 1 && n_batches > 1 && !p.u_q && p.r * rowb <= kRing / 16 - PAD - 32 - MROW) { rows0 = p.r; n_batches = 1; }
     if (cb < ce) issue(cb, 0, 0);
   }
 
