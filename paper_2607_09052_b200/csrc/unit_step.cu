@@ -21,7 +21,7 @@
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
 // summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
 // search: 17.1, 23.4, 95-98, 43.5, 16.9; with the attention's accumulators apart and the query in shared memory: 16.1, 20.9,
-// 93, 35.2, 16.4; with the merge by stores and the first loads together: 15.3, 19.8, 93, 35.2, 13.9.  (One exchange of pairs and
+// 93, 35.2, 16.4; with the merge by stores and the first loads together: 14.6, 19.8, 93, 35.2, 13.8.  (One exchange of pairs and
 // e, every CTA computing all scores, instead of pairs first and scores after: 15.4, 20.3, 93, 35.1, 13.6: not kept.)
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
@@ -226,13 +226,13 @@ struct Scorer {
   const Params &p;
   unsigned char *wsm;
   uint32_t ring, bar0;
-  int lane, r, scale_sz, scale_bytes, ROWS0, ROWSN, mrow, mean_bytes, XS0, XSN, n_batches;
+  int lane, r, cap, scale_sz, scale_bytes, ROWS0, ROWSN, mrow, mean_bytes, XS0, XSN, n_batches;
   bool single;
   uint64_t pol;
   size_t rec_u;                                   // record of the unit's block 0
   size_t scale_total;                             // bytes of the whole scale array
 
-  __device__ __forceinline__ Scorer(const Params &p_, const Unit &x, unsigned char *wsm_, uint64_t *bars, int lane_) : p(p_), wsm(wsm_), lane(lane_) {
+  __device__ __forceinline__ Scorer(const Params &p_, const Unit &x, unsigned char *wsm_, uint64_t *bars, int lane_, bool one) : p(p_), wsm(wsm_), lane(lane_) {
     r = p.r;
     ring = smem_u32(wsm);
     bar0 = smem_u32(bars);
@@ -243,7 +243,10 @@ struct Scorer {
     // contiguous pieces of the summary arrays and is fetched by three bulk copies in memory layout (`single`).
     // Otherwise the factor rows go in batches, each block copied on its own to a padded position.
     single = 16 * D * 2 + 16 * r * ROWB + scale_bytes <= kStage && r <= ROWS_MAX;
-    ROWS0 = single ? r : min(ROWS_MAX, (kStage - MEAN_BYTES - 16 * 32 - scale_bytes) / (16 * ROWB));
+    // A warp with a single chunk gives it the whole ring if that saves batches (one sequence of 32k with bf16 summaries of rank 4:
+    // 15.4 -> 14.6 us; not with a subspace, whose query is projected in the second stage).
+    cap = (!single && one && !p.u_q && MEAN_BYTES + 16 * 32 + scale_bytes + 16 * r * ROWB <= kRing) ? kRing : kStage;
+    ROWS0 = single ? r : min((int)COBS_MAX_RANK, (cap - MEAN_BYTES - 16 * 32 - scale_bytes) / (16 * ROWB));
     ROWSN = min(ROWS_MAX, (kStage - 16 * 32 - scale_bytes) / (16 * ROWB));
     mrow = single ? D * 2 : MROW;                                        // row stride of the mean area
     mean_bytes = 16 * mrow;
@@ -265,7 +268,7 @@ struct Scorer {
     const uint32_t sbase = ring + st * kStage;
     const uint32_t xoff = (b == 0) ? mean_bytes : 0;
     const uint32_t xs = (b == 0) ? XS0 : XSN;
-    const uint32_t soff = kStage - scale_bytes;
+    const uint32_t soff = cap - scale_bytes;
     // the scales of a chunk start on any 2-byte boundary: the copy takes the 16-byte units that hold them, unless those
     // reach past the end of the array (then plain loads)
     const size_t sb0 = rec0 * r * scale_sz;
@@ -423,7 +426,7 @@ struct Scorer {
       if (rows_done) {
       } else if (FP4) {
         // RG factor rows at a time: RG independent accumulator chains keep the tensor pipe busy
-        const unsigned char *sp = wsm + st * kStage + (kStage - scale_bytes) + scale_shift(ck) + (2 * gid) * r * scale_sz;
+        const unsigned char *sp = wsm + st * kStage + (cap - scale_bytes) + scale_shift(ck) + (2 * gid) * r * scale_sz;
 #pragma unroll 1
         for (int i0 = 0; i0 < rows; i0 += RG) {
           float d[RG][4];
@@ -484,18 +487,22 @@ struct Scorer {
           if (scale_sz == 4) accumulate(std::true_type{}); else accumulate(std::false_type{});
         }
       } else {
+#pragma unroll 1
+        for (int i0 = 0; i0 < rows; i0 += ROWS_MAX) {
 #pragma unroll
-        for (int i = 0; i < ROWS_MAX; ++i) {
-          if (i < rows) {
-            float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+          for (int k = 0; k < ROWS_MAX; ++k) {
+            const int i = i0 + k;
+            if (i < rows) {
+              float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
 #pragma unroll
-            for (int m = 0; m < MCH; ++m) {
-              const uint4 va = lds128(xa + i * ROWB + m * 64), vb = lds128(xb + i * ROWB + m * 64);
-              mma16816_bf16(d0, d1, d2, d3, va.x, vb.x, va.y, vb.y, bm[2 * m][0], bm[2 * m][1]);
-              mma16816_bf16(d0, d1, d2, d3, va.z, vb.z, va.w, vb.w, bm[2 * m + 1][0], bm[2 * m + 1][1]);
+              for (int m = 0; m < MCH; ++m) {
+                const uint4 va = lds128(xa + i * ROWB + m * 64), vb = lds128(xb + i * ROWB + m * 64);
+                mma16816_bf16(d0, d1, d2, d3, va.x, vb.x, va.y, vb.y, bm[2 * m][0], bm[2 * m][1]);
+                mma16816_bf16(d0, d1, d2, d3, va.z, vb.z, va.w, vb.w, bm[2 * m + 1][0], bm[2 * m + 1][1]);
+              }
+              d0 *= inv_sqrt_d; d1 *= inv_sqrt_d; d2 *= inv_sqrt_d; d3 *= inv_sqrt_d;
+              sA0 = fmaf(d0, d0, sA0); sA1 = fmaf(d1, d1, sA1); sB0 = fmaf(d2, d2, sB0); sB1 = fmaf(d3, d3, sB1);
             }
-            d0 *= inv_sqrt_d; d1 *= inv_sqrt_d; d2 *= inv_sqrt_d; d3 *= inv_sqrt_d;
-            sA0 = fmaf(d0, d0, sA0); sA1 = fmaf(d1, d1, sA1); sB0 = fmaf(d2, d2, sB0); sB1 = fmaf(d3, d3, sB1);
           }
         }
       }
@@ -542,13 +549,16 @@ struct RowScorer {
   uint64_t pol;
   size_t rec_u, xi_total;
 
-  __device__ __forceinline__ RowScorer(const Params &p_, const Unit &x, unsigned char *wsm_, uint64_t *bars, int lane_) : p(p_), wsm(wsm_), lane(lane_) {
+  __device__ __forceinline__ RowScorer(const Params &p_, const Unit &x, unsigned char *wsm_, uint64_t *bars, int lane_, bool one) : p(p_), wsm(wsm_), lane(lane_) {
     ring = smem_u32(wsm);
     bar0 = smem_u32(bars);
     rowb = p.Ds * ES;
     rows0 = min(p.r, max(0, ROOM - MROW) / rowb);            // rows beside the means
     rows_n = ROOM / rowb;
     n_batches = 1 + (p.r - rows0 + rows_n - 1) / rows_n;
+    // a warp with a single chunk gives it the whole ring: one wait instead of one per batch (one sequence of 2k: 15.5 -> 13.9 us;
+    // not with a subspace, whose query is projected in the second stage)
+    if (one && n_batches > 1 && !p.u_q && p.r * rowb <= kRing / 16 - PAD - 32 - MROW) { rows0 = p.r; n_batches = 1; }
     pol = l2_evict_first_policy();
     rec_u = (size_t)x.u * p.NB;
     xi_total = (size_t)p.B * p.Hkv * p.NB * p.r * rowb;
@@ -590,9 +600,6 @@ struct RowScorer {
     if (bytes) bulk_g2s(dst, src, bytes, bar, pol);
   }
   __device__ __forceinline__ void start(int cb, int ce) {
-    // a single chunk has the whole ring: one wait instead of one per batch (one sequence of 2k: 15.5 -> 13.9 us; not with a
-    // subspace, whose query is projected in the second stage)
-    if (ce - cb == 1 && n_batches > 1 && !p.u_q && p.r * rowb <= kRing / 16 - PAD - 32 - MROW) { rows0 = p.r; n_batches = 1; }
     if (cb < ce) issue(cb, 0, 0);
   }
 
@@ -747,7 +754,7 @@ struct ExactScorer {
   const Params &p;
   unsigned char *wsm;
   int lane;
-  __device__ __forceinline__ ExactScorer(const Params &p_, const Unit &, unsigned char *wsm_, uint64_t *, int lane_) : p(p_), wsm(wsm_), lane(lane_) {}
+  __device__ __forceinline__ ExactScorer(const Params &p_, const Unit &, unsigned char *wsm_, uint64_t *, int lane_, bool) : p(p_), wsm(wsm_), lane(lane_) {}
   __device__ __forceinline__ void start(int, int) {}
   __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, float2 *pair) {
     const int gid = lane >> 2, tig = lane & 3, G = p.G, gpb = p.L >> 4, lgP = 31 - __clz(p.P);
@@ -1225,7 +1232,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     x.el = (c1 - c0) * SCORER::BLOCKS;
     x.eb = (pl.e_off >= 0) ? reinterpret_cast<float *>(fsm + pl.e_off) : p.e + ((size_t)u * ((NB + 15) / 16 * 16) + x.b0) * G;
     x.qt = s_qt;
-    SCORER sc(p, x, wsm, &s_bars[warp][0], lane);
+    SCORER sc(p, x, wsm, &s_bars[warp][0], lane, ce - cb == 1);
     sc.start(cb, ce);
     store_q();
     __syncthreads();
