@@ -21,7 +21,7 @@
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
 // summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
 // search: 17.1, 23.4, 95-98, 43.5, 16.9; with the attention's accumulators apart and the query in shared memory: 16.1, 20.9,
-// 93, 35.2, 16.4; with the merge by stores and the first loads together: 14.6, 19.8, 93, 35.2, 13.8.  (One exchange of pairs and
+// 93, 35.2, 16.4; with the merge by stores and the first loads together: 14.6, 19.8, 93, 35.2, 13.4.  (One exchange of pairs and
 // e, every CTA computing all scores, instead of pairs first and scores after: 15.4, 20.3, 93, 35.1, 13.6: not kept.)
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
@@ -999,6 +999,63 @@ __device__ __forceinline__ void select_topk(const float *keys_s, int n, int k, i
   __syncthreads();
 }
 
+// The same for up to 32 KPL keys by one warp, which holds them all: a round costs no barrier, and a barrier is what a round of
+// select_topk waits for.  Up to one key per thread of the CTA (16 steps of 16 sequences of 16k in blocks of 64: 731 -> 726 us; one sequence of 2k:
+// 13.9 -> 13.4); sixteen keys per lane are too many instructions for one warp (one sequence of 32k: 14.6 us, 15.9 that way), and
+// with four warps per CTA a barrier costs less (24 ragged sequences of 12k: 35.1 us, 35.3 with 256).
+template <int KPL>
+__device__ __forceinline__ void select_topk_warp(const float *keys_s, int n, int k, int *sel, int lane) {
+  static_assert(KPL % 4 == 0 && 32 * KPL < 1024, "counts of ten bits");
+  const int b0 = lane * KPL;
+  uint32_t key[KPL];
+#pragma unroll
+  for (int j = 0; j < KPL; j += 4) {                 // (the array has a whole number of fours of keys)
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b0 + j < n) v = *reinterpret_cast<const float4 *>(keys_s + b0 + j);
+    key[j] = __float_as_uint(v.x);
+    key[j + 1] = (b0 + j + 1 < n) ? __float_as_uint(v.y) : 0u;
+    key[j + 2] = (b0 + j + 2 < n) ? __float_as_uint(v.z) : 0u;
+    key[j + 3] = (b0 + j + 3 < n) ? __float_as_uint(v.w) : 0u;
+  }
+  const uint32_t ku = (uint32_t)k;
+  uint32_t theta = 0u;
+#pragma unroll 1
+  for (int bit = 30; bit >= 0; bit -= 2) {
+    const uint32_t ta = theta | (3u << bit), tb = theta | (2u << bit), tc = theta | (1u << bit);
+    uint32_t c = 0, d = 0;                           // (two chains)
+#pragma unroll
+    for (int j = 0; j < KPL; j += 2) {
+      c += (key[j] >= ta ? 1u : 0u) + (key[j] >= tb ? 1u << 10 : 0u) + (key[j] >= tc ? 1u << 20 : 0u);
+      d += (key[j + 1] >= ta ? 1u : 0u) + (key[j + 1] >= tb ? 1u << 10 : 0u) + (key[j + 1] >= tc ? 1u << 20 : 0u);
+    }
+    c = __reduce_add_sync(0xffffffffu, c + d);
+    const uint32_t na = c & 1023u, nb = (c >> 10) & 1023u, nc = c >> 20;
+    const uint32_t at = (na >= ku) ? na : (nb >= ku) ? nb : (nc >= ku) ? nc : 0u;
+    if (na >= ku) theta = ta; else if (nb >= ku) theta = tb; else if (nc >= ku) theta = tc;
+    if (at == ku) break;
+  }
+  int v = 0;
+#pragma unroll
+  for (int j = 0; j < KPL; ++j)
+    if (b0 + j < n) v += (key[j] > theta ? (1 << 16) : 0) + (key[j] == theta ? 1 : 0);
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, inc, 31);
+  const int need_eq = max(k - (total >> 16), 0), excl = inc - v;
+  int eq_rank = excl & 0xffff, pos = (excl >> 16) + min(eq_rank, need_eq);
+#pragma unroll
+  for (int j = 0; j < KPL; ++j)
+    if (b0 + j < n) {
+      bool keep = key[j] > theta;
+      if (key[j] == theta) { keep = eq_rank < need_eq; ++eq_rank; }
+      if (keep && pos < k) sel[pos++] = b0 + j;
+    }
+}
+
 // ---------------------------------------------------------------------------------------------------
 // Attention over groups [g0, g1) of the unit by one warp: slots below n_sel are selected blocks, then the window's.
 // Leaves acc [G][D] in the warp's ring and (max in natural log units, sum) per head in pair.
@@ -1309,6 +1366,12 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     // ---- top-k ------------------------------------------------------------------------------------------------------
     if (n_sel == n_cand) {
       for (int i = tid; i < n_sel; i += nthr) s_sel[i] = i;
+      __syncthreads();
+    } else if (n_cand <= nthr) {
+      if (warp == 0) {
+        if (n_cand <= 128) select_topk_warp<4>(keys, n_cand, n_sel, s_sel, lane);
+        else select_topk_warp<8>(keys, n_cand, n_sel, s_sel, lane);
+      }
       __syncthreads();
     } else if (n_cand <= 2 * nthr) {
       select_topk<2>(keys, n_cand, n_sel, s_sel, s_cnt, s_scan, tid, W);

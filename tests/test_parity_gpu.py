@@ -314,6 +314,16 @@ def test_unit_step_plan_edges(batch, hkv, G, D, nb, L, rank, sub, dtype, scale, 
     run_stage_s(wl, units=units if len(units) <= 32 else [units[0], units[1], units[len(units) // 2], units[-1]])
 
 
+# candidate counts at the edges of the selection by one warp (four and eight keys per lane) and at the first count beyond it
+@pytest.mark.parametrize("n_cand", [2, 31, 127, 128, 129, 255, 256, 257])
+def test_selection_by_one_warp_at_its_edges(n_cand):
+    L, window = 16, 32
+    lens = [n_cand * L + window, n_cand * L + window + 5]
+    wl = synth.Workload("warp", 2, 4, 2, 64, lens[0] + L, L, 16, rank=2, topk=max(1, n_cand // 3), window=window,
+                        summary_dtype="bf16", key_model="block_offset", shuffle_pages=True, seed=23, seq_lens=lens)
+    run_stage_s(wl)
+
+
 def test_ragged_lengths_and_degenerate_cases():
     L = 64
     # T < L (no summarised block), T inside the window only, partial last block, k larger than candidates
