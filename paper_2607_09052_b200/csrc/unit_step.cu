@@ -21,7 +21,7 @@
 // copy rate: 512 MB), 24 ragged ones of 12k (375 blocks, not a multiple of four: three launches before) 156 -> 45, fp32
 // summaries at 2k (three launches before) 36.4 -> 18.5.  With programmatic dependent launch and the early end of the top-k
 // search: 17.1, 23.4, 95-98, 43.5, 16.9; with the attention's accumulators apart and the query in shared memory: 16.1, 20.9,
-// 93, 35.2, 16.4; with the merge by stores and the first loads together: 14.6, 19.8, 93, 35.2, 13.4.  (One exchange of pairs and
+// 93, 35.2, 16.4; with the merge by stores and the first loads together and the window fetched ahead: 14.6, 19.1, 91, 34.4, 13.3.  (One exchange of pairs and
 // e, every CTA computing all scores, instead of pairs first and scores after: 15.4, 20.3, 93, 35.1, 13.6: not kept.)
 //
 // Data movement.  Every stream a warp consumes goes global -> shared into a ring that belongs to that warp alone.  Scoring: a
@@ -100,6 +100,10 @@ __device__ __forceinline__ void st_cluster2(uint32_t addr, float2 v) {
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
+
+__device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
+}
 
 // running (max, sum of exponentials) of one head
 struct Run { float m, s; };
@@ -1291,6 +1295,17 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     x.qt = s_qt;
     SCORER sc(p, x, wsm, &s_bars[warp][0], lane, ce - cb == 1);
     sc.start(cb, ce);
+    // Between the last scores and the first selected block HBM would be idle: the window's groups, known already, are fetched into
+    // L2 meanwhile (sixteen sequences of 128k 93.4 -> 91.1 us; 16 steps of sixteen of 16k 727 -> 687).  Lane i < 4 looks up the page
+    // of group nw i + wi: four groups of 8 KB per warp are the window of 512 tokens with eight warps per unit, and 38 MB in all.
+    uint32_t ahead = 0xffffffffu;
+    {
+      const int tok = ws + 16 * (nw * lane + wi), pslot = tok >> (31 - __clz(p.P));
+      if ((phases & PH_ATTEND) && lane < 4 && tok < T && pslot < p.mpp) {
+        const int pg = p.page_table[(size_t)x.b_idx * p.mpp + pslot];
+        if (pg >= 0 && pg < p.n_pages) ahead = (uint32_t)(((((size_t)pg * p.Hkv + x.h) * p.P + (tok & (p.P - 1))) * D) / 8);
+      }
+    }
     store_q();
     __syncthreads();
     if (p.u_q) {                                            // (scratch: the second stages of four rings, not in use yet)
@@ -1299,6 +1314,10 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     }
     // (max, sum) of e per head: over the warp, the CTA, the cluster
     if (!sc.run(x, cb, ce, s_pair[warp])) s_lost = 1;
+    if (ahead != 0xffffffffu) {
+      bulk_prefetch_l2(reinterpret_cast<const uint4 *>(p.k_pages) + ahead, 16 * D * 2);
+      bulk_prefetch_l2(reinterpret_cast<const uint4 *>(p.v_pages) + ahead, 16 * D * 2);
+    }
     __syncthreads();
     COBS_STAMP(1);
     if (C > 1) cluster_wait();
