@@ -103,6 +103,12 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Place of the 16-token group that begins at token `tok` (a multiple of 16) of page `pg`, KV head h, in the key or value pool, in
+// groups from the pool's start (16 D elements each: 2 or 4 KB, so that 32 bits reach 8 TB; pages hold 16 tokens or more).
+__device__ __forceinline__ uint32_t group_place(const Params &p, int pg, int h, int tok) {
+  return (uint32_t)((((size_t)pg * p.Hkv + h) * p.P + (tok & (p.P - 1))) >> 4);
+}
+
 // window start (tokens), aligned down to a block boundary
 __device__ __forceinline__ int window_start(int T, int window, int L) {
   int a = T - window;

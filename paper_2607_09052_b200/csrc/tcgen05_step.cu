@@ -571,7 +571,7 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
         const int pslot = tok0 >> lgP;                                // a length beyond the page-table row is not followed
         const int pg = (pslot < p.mpp) ? p.page_table[(size_t)b_idx * p.mpp + pslot] : -1;
         if (pg < 0 || pg >= p.n_pages) report(p.status, COBS_ERR_BOUNDS);
-        else { first = tok0; off = (uint32_t)(((((size_t)pg * p.Hkv + h) * P + (tok0 & (P - 1))) * D) / 8); }
+        else { first = tok0; off = group_place(p, pg, h, tok0); }
       }
       goff[g] = off;
       gtok[g] = first;
@@ -587,7 +587,7 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
       if (g < n_groups) {
         const int first = gtok[g];
         if (first >= 0) {
-          const uint32_t off = goff[g];
+          const size_t off = (size_t)goff[g] * (2 * D);
           const uint4 *ks = kbase + off, *vs = vbase + off;
           const uint32_t dst = ring + st * STAGE;
           const int nv = T - first;

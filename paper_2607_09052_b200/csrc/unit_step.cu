@@ -782,21 +782,21 @@ struct ExactScorer {
       cdst[j] = t * ROWB + ((c ^ (t & 7)) << 4);
     }
     const int kt = ((lane >> 4) & 1) * 8 + (lane & 7), kc = (lane >> 3) & 1;
-    // lane i holds the place of group 32 k + i (16-byte units from the pool's start; none: all ones), for two k at a time
+    // lane i holds the place of group 32 k + i (in groups from the pool's start; none: all ones), for two k at a time
     constexpr uint32_t kNone = 0xffffffffu;
     auto resolve = [&](int g) -> uint32_t {
       if (g >= n) return kNone;
       const int tok0 = b0 * p.L + g * 16, pslot = tok0 >> lgP;
       const int pg = (pslot < p.mpp) ? p.page_table[(size_t)x.b_idx * p.mpp + pslot] : -1;
       if (pg < 0 || pg >= p.n_pages) { report(p.status, COBS_ERR_BOUNDS); return kNone; }
-      return (uint32_t)(((((size_t)pg * p.Hkv + x.h) * p.P + (tok0 & (p.P - 1))) * D) / 8);
+      return group_place(p, pg, x.h, tok0);
     };
     uint32_t tab[2] = {resolve(lane), resolve(32 + lane)};
     auto issue = [&](int g, int st) {
       const uint32_t off = __shfl_sync(0xffffffffu, (g & 32) ? tab[1] : tab[0], g & 31);
       if (g < n && off != kNone) {
 #pragma unroll
-        for (int j = 0; j < NCP; ++j) cpa16(ring + st * STAGE + cdst[j], kbase + off + 32 * j, pol);
+        for (int j = 0; j < NCP; ++j) cpa16(ring + st * STAGE + cdst[j], kbase + (size_t)off * (2 * D) + 32 * j, pol);
       }
       cpa_commit();
       return off;
@@ -1128,7 +1128,7 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
         const int pslot = tok0 >> lgP;                                // a length beyond the page-table row is not followed
         const int pg = (pslot < p.mpp) ? p.page_table[(size_t)x.b_idx * p.mpp + pslot] : -1;
         if (pg < 0 || pg >= p.n_pages) report(p.status, COBS_ERR_BOUNDS);
-        else { first = tok0; off = (uint32_t)(((((size_t)pg * p.Hkv + x.h) * P + (tok0 & (P - 1))) * D) / 8); }
+        else { first = tok0; off = group_place(p, pg, x.h, tok0); }
       }
       goff[g] = off;
       gtok[g] = first;
@@ -1138,7 +1138,7 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
       if (g < n_groups) {
         const int first = gtok[g];
         if (first >= 0) {
-          const uint32_t off = goff[g];
+          const size_t off = (size_t)goff[g] * (2 * D);
           const uint4 *ks = kbase + off, *vs = vbase + off;
           const uint32_t dst = ring + st * STAGE;
           const int nv = T - first;
@@ -1303,7 +1303,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
       const int tok = ws + 16 * (nw * lane + wi), pslot = tok >> (31 - __clz(p.P));
       if ((phases & PH_ATTEND) && lane < 4 && tok < T && pslot < p.mpp) {
         const int pg = p.page_table[(size_t)x.b_idx * p.mpp + pslot];
-        if (pg >= 0 && pg < p.n_pages) ahead = (uint32_t)(((((size_t)pg * p.Hkv + x.h) * p.P + (tok & (p.P - 1))) * D) / 8);
+        if (pg >= 0 && pg < p.n_pages) ahead = group_place(p, pg, x.h, tok);
       }
     }
     store_q();
@@ -1315,8 +1315,8 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     // (max, sum) of e per head: over the warp, the CTA, the cluster
     if (!sc.run(x, cb, ce, s_pair[warp])) s_lost = 1;
     if (ahead != 0xffffffffu) {
-      bulk_prefetch_l2(reinterpret_cast<const uint4 *>(p.k_pages) + ahead, 16 * D * 2);
-      bulk_prefetch_l2(reinterpret_cast<const uint4 *>(p.v_pages) + ahead, 16 * D * 2);
+      bulk_prefetch_l2(p.k_pages + (size_t)ahead * (16 * D), 16 * D * 2);
+      bulk_prefetch_l2(p.v_pages + (size_t)ahead * (16 * D), 16 * D * 2);
     }
     __syncthreads();
     COBS_STAMP(1);

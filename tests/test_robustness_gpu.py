@@ -1,0 +1,57 @@
+"""Calls at the edges of what the entry points accept: very large pools, lengths that make no sense, buffers that overlap,
+calls that follow one another without a host synchronisation."""
+
+import pytest
+import torch
+
+from paper_2607_09052_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _binding():
+    from paper_2607_09052_b200 import binding
+    return binding
+
+
+def to_dev(inp):
+    return {k: (v.cuda() if isinstance(v, torch.Tensor) and k != "planted" else v) for k, v in inp.items()}
+
+
+def test_pool_beyond_64_gib():
+    """Pages whose bytes lie 64 GiB and more from the start of the pool: the same bits as from a small pool.  The first pages
+    of the large pool, where an offset of 32 bits in 16-byte units would end up, hold other keys."""
+    B = _binding()
+    page_bytes, n_far = 16 * 128 * 2, 1 << 24                     # 4 KiB pages: page 2^24 begins at 64 GiB
+    wl = synth.Workload("far", 1, 4, 1, 128, 24 * 64, 64, 16, rank=2, topk=5, window=100, summary_dtype="bf16",
+                        key_model="block_offset", shuffle_pages=True, seed=19)
+    if torch.cuda.mem_get_info()[0] < (n_far + 4096) * page_bytes + (2 << 30):
+        pytest.skip("needs 67 GB of free device memory")
+    inp = to_dev(synth.generate(wl))
+    cfg = B.make_config(wl)
+    n = inp["k_pages"].shape[0]
+    summ = B.SummaryBuffers(cfg, "cuda")
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, B.make_kv(inp), 0, wl.max_blocks, summ, ws)
+
+    def calls(pool, table):
+        kv = B.KV(pool.data_ptr(), pool.data_ptr(), table.data_ptr(), inp["seq_lens"].data_ptr(), pool.shape[0])
+        sel = torch.full((1, 1, wl.topk), -7, dtype=torch.int32, device="cuda")
+        cnt = torch.zeros((1, 1), dtype=torch.int32, device="cuda")
+        scores = torch.zeros((1, 1, wl.max_blocks), device="cuda")
+        outs = [torch.zeros((1, 4, 128), device="cuda") for _ in range(2)]
+        B.cobs_exact_select(cfg, inp["q"], kv, sel, cnt, scores, ws)
+        B.cobs_sparse_decode(cfg, inp["q"], kv, sel, cnt, outs[0], None, ws)
+        B.cobs_decode_step(cfg, inp["q"], kv, summ, outs[1], None, None, None, ws)
+        assert B.cobs_read_status(ws) == 0
+        return [sel, cnt, scores] + outs
+
+    want = calls(inp["k_pages"], inp["page_table"])
+    far = torch.empty((n_far + n, 1, 16, 128), dtype=torch.bfloat16, device="cuda")
+    far[:n] = inp["k_pages"].flip(0) * -1.0
+    far[n_far:] = inp["k_pages"]
+    got = calls(far, inp["page_table"] + n_far)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    del far
+    torch.cuda.empty_cache()
