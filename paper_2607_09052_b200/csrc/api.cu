@@ -203,6 +203,11 @@ static void *mapped(const void *host) {
   return nullptr;
 }
 
+static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return a && b && x < y + nb && y < x + na;
+}
+
 // Scoring and selection, with the attention or without: one launch.  The generic scoring and selection kernels are for what the
 // unit kernel does not cover.
 static cudaError_t launch_score_step(const Params &p, int phases, cudaStream_t s) {
@@ -453,11 +458,14 @@ int32_t cobs_decode_step_host(const cobs_config *cfg, const void *q_host, const 
   // Pinned, device-mapped memory is used in place by the cluster kernel: its CTAs fetch their unit's query from it once (2 KB;
   // 131 KB through a copy or a staging kernel in front of the step took 6 us and more), output rows and selection are posted
   // writes.  The other kernels read the query often and the selection back; they, and any other host memory, get copies.
+  // So does a query that shares memory with what is written: a unit may write before another has read its query.
   Params p;
   fill_params(p, cfg, workspace);
   if ((st = set_summaries(p, cfg, summ)) != COBS_OK) return st;
   const bool in_place = unit_score_supported(p) && !umma_score_supported(p);
-  const void *q_map = in_place ? mapped(q_host) : nullptr;
+  const bool q_alone = !overlap(q_host, n * 2, out_host, n * 4) && !overlap(q_host, n * 2, sel_idx_host_or_null, units * cfg->topk * 4) &&
+                       !overlap(q_host, n * 2, sel_cnt_host_or_null, units * 4);
+  const void *q_map = (in_place && q_alone) ? mapped(q_host) : nullptr;
   if (!q_map && cudaMemcpyAsync(q_dev, q_host, n * 2, cudaMemcpyHostToDevice, s) != cudaSuccess) return COBS_ERR_CUDA;
   float *out_map = static_cast<float *>(mapped(out_host));
   int32_t *sel_map = (in_place && sel_idx_host_or_null) ? static_cast<int32_t *>(mapped(sel_idx_host_or_null)) : nullptr;

@@ -55,3 +55,36 @@ def test_pool_beyond_64_gib():
         assert torch.equal(a, b)
     del far
     torch.cuda.empty_cache()
+
+
+def test_host_step_with_query_and_output_in_one_buffer():
+    """The query at the start of the pinned buffer that receives the output: the query is read before anything is written,
+    however many (sequence, KV head) units there are, as when it was copied to the device first."""
+    B = _binding()
+    wl = synth.Workload("alias", 96, 32, 8, 128, 16 * 64, 64, 64, rank=2, topk=4, window=100, summary_dtype="bf16",
+                        key_model="block_offset", seed=5)
+    inp = synth.generate(wl, "cuda")
+    cfg = B.make_config(wl)
+    kv = B.make_kv(inp)
+    summ = B.SummaryBuffers(cfg, "cuda")
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, kv, 0, wl.max_blocks, summ, ws)
+    q = inp["q"].cpu().pin_memory()
+    want = torch.zeros(q.shape).pin_memory()
+    B.cobs_decode_step_host(cfg, q, kv, summ, want, None, None, ws)
+    for at in (0, q.numel() // 2 - 64):                           # at the start of the output, and across its middle
+        buf = torch.zeros(q.shape).pin_memory()
+        inside = buf.view(-1)[at:at + q.numel() // 2].view(torch.bfloat16).view(q.shape)
+        inside.copy_(q)
+        B.cobs_decode_step_host(cfg, inside, kv, summ, buf, None, None, ws)
+        assert torch.equal(buf, want)
+    # the selection's arrays may lie over the query as well
+    sel, cnt = torch.zeros((96, 8, 4), dtype=torch.int32).pin_memory(), torch.zeros((96, 8), dtype=torch.int32).pin_memory()
+    out = torch.zeros_like(want)
+    B.cobs_decode_step_host(cfg, q, kv, summ, out, sel, cnt, ws)
+    q2 = q.clone().pin_memory()
+    over = q2.view(-1).view(torch.int32)
+    sel2, cnt2 = over[:sel.numel()].view(sel.shape), over[sel.numel():sel.numel() + cnt.numel()].view(cnt.shape)
+    B.cobs_decode_step_host(cfg, q2, kv, summ, out, sel2, cnt2, ws)
+    assert torch.equal(out, want) and torch.equal(sel2, sel) and torch.equal(cnt2, cnt)
+    assert B.cobs_read_status(ws) == 0
