@@ -56,11 +56,14 @@ struct Params {
 void count_launch(int n = 1);
 void count_tcgen05_launch();
 
-// Programmatic dependent launch: every kernel of the library begins with pdl_begin and is launched by launch_chained, so that
-// in a chain of calls on one stream (append, build, step; score, trim, attend; step after step) a kernel's CTAs are set up
-// while the last ones of the kernel before it still run.  The wait returns when that kernel has completed and its writes are
-// visible: nothing is read or written before it.  (A kernel launched without the attribute is not overtaken, nor does one
-// that does not say launch_dependents let its successor in early.)
+// Programmatic dependent launch: the kernels of the library's main path begin with pdl_begin and are launched by launch_chained
+// (or with the same attribute), so that in a chain of calls on one stream (append, build, step; score, trim, attend; step after
+// step) a kernel's CTAs are set up while the last ones of the kernel before it still run.  The wait returns when that kernel
+// has completed and its writes are visible: nothing is read or written before it, and nothing that an earlier kernel may have
+// written is read through the non-coherent path (ld.global.nc, __ldg), which asks for data that does not change while the
+// kernel is resident and is not ordered by the wait.  (A kernel launched without the attribute - the exact masses beyond the step
+// kernel's capacity, the tcgen05 variant, the conversion hook - is not overtaken, nor does one that does not say
+// launch_dependents let its successor in early.)
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   asm volatile("griddepcontrol.wait;\n" ::: "memory");

@@ -725,8 +725,8 @@ struct RowScorer {
         row_product(xa + i * rowb, xb + i * rowb, Ds, vec, !sub, d);
         float cA = 0.f, cB = 0.f;                    // (c / 6) / (1 / 2): folded into the sums that are halved below
         if (p.skew) {
-          if (ck * 16 + 2 * gid < x.n_sum) cA = __ldg(p.skew + rec * p.r + row0 + i) * (1.0f / 3.0f);
-          if (ck * 16 + 2 * gid + 1 < x.n_sum) cB = __ldg(p.skew + (rec + 1) * p.r + row0 + i) * (1.0f / 3.0f);
+          if (ck * 16 + 2 * gid < x.n_sum) cA = p.skew[rec * p.r + row0 + i] * (1.0f / 3.0f);
+          if (ck * 16 + 2 * gid + 1 < x.n_sum) cB = p.skew[(rec + 1) * p.r + row0 + i] * (1.0f / 3.0f);
         }
         const float d0 = d[0] * qs, d1 = d[1] * qs, d2 = d[2] * qs, d3 = d[3] * qs;
         sA0 = fmaf(d0 * d0, fmaf(cA, d0, 1.0f), sA0); sA1 = fmaf(d1 * d1, fmaf(cA, d1, 1.0f), sA1);
@@ -899,7 +899,7 @@ __device__ __forceinline__ void project_query(const Params &p, const Unit &x, fl
     const float *uq = p.u_q + ((size_t)x.h * D + quarter * DQ) * p.Ds + (live ? s : 0);
     float v[DQ];
 #pragma unroll
-    for (int j = 0; j < DQ; ++j) v[j] = live ? __ldg(uq + (size_t)j * p.Ds) : 0.f;
+    for (int j = 0; j < DQ; ++j) v[j] = live ? uq[(size_t)j * p.Ds] : 0.f;
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
       const __nv_bfloat16 *q = x.q + g * kQRow + quarter * DQ;

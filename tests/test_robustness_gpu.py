@@ -88,3 +88,57 @@ def test_host_step_with_query_and_output_in_one_buffer():
     B.cobs_decode_step_host(cfg, q2, kv, summ, out, sel2, cnt2, ws)
     assert torch.equal(out, want) and torch.equal(sel2, sel) and torch.equal(cnt2, cnt)
     assert B.cobs_read_status(ws) == 0
+
+
+def test_calls_in_a_row_without_host_synchronisation():
+    """Appends, rebuilds and steps, and subspace builds with one basis after another on one workspace, enqueued back to back:
+    every kernel is resident before the one in front of it has finished writing what it reads.  The same bits as with a
+    synchronisation behind every call."""
+    B = _binding()
+    from paper_2607_09052_b200.decode_loop import DecodeLoop
+    wl = synth.Workload("chain", 3, 8, 2, 128, 40 * 32, 32, 16, rank=4, topk=6, window=70, summary_dtype="bf16",
+                        key_model="block_offset", shuffle_pages=True, seed=3, seq_lens=[32 * 20 + 30, 32 * 11 + 29, 32 * 31])
+    cfg = B.make_config(wl)
+    gen = torch.Generator().manual_seed(4)
+    q, k, v = (torch.randn(shape, generator=gen).bfloat16().cuda() for shape in ((40, 3, 8, 128), (40, 3, 2, 128), (40, 3, 2, 128)))
+
+    def loop(sync):
+        inp = to_dev(synth.generate(wl))
+        summ = B.SummaryBuffers(cfg, "cuda", skew=True)
+        ws = B.alloc_workspace(cfg, "cuda")
+        B.cobs_build_summaries(cfg, B.make_kv(inp), 0, wl.max_blocks, summ, ws)
+        dl = DecodeLoop(wl, inp, summ, ws)
+        out = torch.zeros((40, 3, 8, 128), device="cuda")
+        torch.cuda.synchronize()
+        for i in range(40):
+            dl.step(q[i], k[i], v[i], out[i])
+            if sync:
+                torch.cuda.synchronize()
+        assert B.cobs_read_status(ws) == 0
+        return [out, summ.mean, summ.xi, summ.skew, inp["seq_lens"]]
+
+    for a, b in zip(loop(False), loop(True)):
+        assert torch.equal(a, b)
+
+    wl = synth.Workload("bases", 2, 8, 2, 128, 64 * 64, 64, 16, rank=4, topk=6, window=70, summary_dtype="fp32", sub_dim=85,
+                        key_model="block_offset", shuffle_pages=True, seed=6)
+    cfg = B.make_config(wl)
+    inp = to_dev(synth.generate(wl))
+    kv = B.make_kv(inp)
+    ws = B.alloc_workspace(cfg, "cuda")
+    bases = [torch.linalg.qr(torch.randn((2, 128, 85), generator=gen))[0].contiguous().cuda() for _ in range(6)]
+
+    def builds(sync):
+        summs = [B.SummaryBuffers(cfg, "cuda", u) for u in bases * 2]
+        torch.cuda.synchronize()
+        for s in summs:
+            B.cobs_build_summaries(cfg, kv, 0, wl.max_blocks, s, ws)
+            if sync:
+                torch.cuda.synchronize()
+        assert B.cobs_read_status(ws) == 0
+        return [s.xi for s in summs]
+
+    want = builds(True)
+    for _ in range(5):
+        for a, b in zip(builds(False), want):
+            assert torch.equal(a, b)
