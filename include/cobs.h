@@ -93,7 +93,8 @@ typedef struct {
   const int32_t *page_table;  /* [B][max_pages_per_seq]: page id of the i-th page of a sequence */
   const int32_t *seq_lens;    /* [B]: tokens in the cache, the current one included; 1 <= T <= min(NB*L + L - 1,
                                  max_pages_per_seq * P).  Tokens beyond the page-table row are not read: they are
-                                 skipped and COBS_ERR_BOUNDS is left in the status word */
+                                 skipped and COBS_ERR_BOUNDS is left in the status word.  A length below
+                                 zero counts as none */
   int64_t n_pages;            /* page ids are checked against this */
 } cobs_kv;
 

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kAThreads) adaptive_trim_kernel(Params p, floa
   const int b_idx = u / p.Hkv;
   const float *sc = p.scores + (size_t)u * p.NB;
   int32_t *out = p.sel_idx + (size_t)u * p.topk;
-  const int T = p.seq_lens[b_idx], cnt = p.sel_cnt[u];
+  const int T = tokens_of(p.seq_lens, b_idx), cnt = p.sel_cnt[u];
   int id = (item < p.topk) ? out[item] : -1;
   const int n_sum = min(T / p.L, p.NB);
   const int n_cand = min(window_start(T, p.window, p.L) / p.L, n_sum);

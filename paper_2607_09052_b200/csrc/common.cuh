@@ -112,6 +112,17 @@ __device__ __forceinline__ uint32_t group_place(const Params &p, int pg, int h, 
   return (uint32_t)((((size_t)pg * p.Hkv + h) * p.P + (tok & (p.P - 1))) >> 4);
 }
 
+// Tokens of a sequence in the cache.  A length below zero counts as none: blocks, candidates and groups are shared out in
+// unsigned arithmetic.
+__device__ __forceinline__ int tokens_of(const int32_t *seq_lens, int b) { return max(seq_lens[b], 0); }
+
+// The page that holds token `tok` of sequence b, or -1 when the page table's row does not reach it (a length beyond the row, or
+// one so large that token numbers wrap, is not followed).  The id itself is checked by the caller.
+__device__ __forceinline__ int page_of(const Params &p, int b, int tok) {
+  const unsigned slot = (unsigned)tok >> (31 - __clz(p.P));
+  return (tok >= 0 && slot < (unsigned)p.mpp) ? p.page_table[(size_t)b * p.mpp + slot] : -1;
+}
+
 // window start (tokens), aligned down to a block boundary
 __device__ __forceinline__ int window_start(int T, int window, int L) {
   int a = T - window;

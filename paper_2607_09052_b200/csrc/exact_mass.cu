@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kEWarps * 32) exact_mass_kernel(Params p) {
   for (long long it = (long long)blockIdx.x * kEWarps + warp; it < items; it += (long long)gridDim.x * kEWarps) {
     const int u = (int)(it / NB), blk = (int)(it - (long long)u * NB);
     const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
-    const int T = p.seq_lens[b_idx];
+    const int T = tokens_of(p.seq_lens, b_idx);
     if (blk >= min(T / L, NB)) continue;         // only full blocks have a mass here, as only they have summaries
     if (u != cur_u) {
       cur_u = u;
@@ -70,8 +70,7 @@ __global__ void __launch_bounds__(kEWarps * 32) exact_mass_kernel(Params p) {
     auto issue = [&](int g, int st) {
       if (g < gpb) {
         const int tok0 = blk * L + g * 16;
-        const int pslot = tok0 / P;                 // < mpp for every full block (mpp * P >= NB * L); checked all the same
-        const int pg = (pslot < p.mpp) ? p.page_table[(size_t)b_idx * p.mpp + pslot] : -1;
+        const int pg = page_of(p, b_idx, tok0);
         if (pg < 0 || pg >= p.n_pages) report(p.status, COBS_ERR_BOUNDS);
         else {
           const uint4 *ks = kbase + ((((size_t)pg * p.Hkv + h) * P + (tok0 % P)) * D) / 8;

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) score_generic_kernel(Params p, int blocks
   float *qs = smem;                 // [G][D]
   float *qt = smem + G * p.D;       // [G][Ds_pad]
   const int u = blockIdx.y, b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
-  int T = p.seq_lens[b_idx];
+  const int T = tokens_of(p.seq_lens, b_idx);
   int n_sum = min(T / p.L, p.NB);
   const int first = blockIdx.x * blocks_per_cta;
   if (first >= n_sum) return;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(Params p) {
 
   pdl_begin();
   const int u = blockIdx.x, b_idx = u / p.Hkv, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int T = p.seq_lens[b_idx];
+  const int T = tokens_of(p.seq_lens, b_idx);
   const int n_sum = min(T / p.L, p.NB);
   const int n_cand = min(window_start(T, p.window, p.L) / p.L, n_sum);
   const int G = p.G;

@@ -286,7 +286,7 @@ __device__ __forceinline__ void build_block(const Params &p, float *sm, int u, i
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int NW = kBuildThreads / 32;
   const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
-  const int T = p.seq_lens[b_idx];
+  const int T = tokens_of(p.seq_lens, b_idx);
   if (blk >= min(T / L, p.NB)) return;
   const size_t rec = (size_t)u * p.NB + blk;
   const int Dk4 = (Dk + 3) / 4 * 4;
@@ -847,7 +847,7 @@ cudaError_t launch_build(const Params &p, int block_begin, int block_end, int *f
 __global__ void __launch_bounds__(256) append_kernel(Params p, const uint4 *k_new, const uint4 *v_new, uint4 *k_pages, uint4 *v_pages, int32_t *seq_lens) {
   pdl_begin();
   const int b = blockIdx.x, T = seq_lens[b], d8 = p.D / 8;
-  const int pg = (T >= 0 && T < p.mpp * p.P) ? p.page_table[(size_t)b * p.mpp + T / p.P] : -1;
+  const int pg = page_of(p, b, T);
   if (pg < 0 || pg >= p.n_pages) {
     if (threadIdx.x == 0) report(p.status, COBS_ERR_BOUNDS);
     return;

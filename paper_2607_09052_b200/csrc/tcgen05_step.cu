@@ -343,7 +343,7 @@ __device__ void select_team(const Params &p, const int *seq_lens, int tid, int c
   // pieces, the real pass finds them close by.
   bool rehearsal = true;
   for (int u = blockIdx.x; u < units;) {
-    const int T = seq_lens[u / p.Hkv];
+    const int T = tokens_of(seq_lens, u / p.Hkv);
     const int n_sum = min(T / p.L, p.NB);
     const int n_cand = min(window_start(T, p.window, p.L) / p.L, n_sum);
     const int n_chunks = (n_sum + 15) / 16;
@@ -390,8 +390,8 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
   constexpr int STAGE = 2 * VOFF;
   constexpr int NCP = (16 * CH) / 32;         // cp.async per lane per operand per stage
   const int gid = lane >> 2, tig = lane & 3;
-  const int G = p.G, L = p.L, P = p.P, units = p.B * p.Hkv, n_splits = p.n_splits;
-  const int lgL = 31 - __clz(L), lgP = 31 - __clz(P), lgg = lgL - 4;      // L and P are powers of two: shifts, not divisions
+  const int G = p.G, L = p.L, units = p.B * p.Hkv, n_splits = p.n_splits;
+  const int lgL = 31 - __clz(L), lgg = lgL - 4;      // L is a power of two: shifts, not divisions
   const int gpb = L >> 4;
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(wsm);
   uint32_t *goff = reinterpret_cast<uint32_t *>(wsm + kAttStages * kAttStageBytes);
@@ -520,7 +520,7 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
     if (item >= n_items) break;
     const int u = item / n_splits, split = item - u * n_splits;
     const int b_idx = u / p.Hkv, h = u - b_idx * p.Hkv;
-    const int T = seq_lens[b_idx];
+    const int T = tokens_of(seq_lens, b_idx);
     const int ws = window_start(T, p.window, L);
     const int n_cand = ws >> lgL;
     const int n_win = (T - ws + L - 1) >> lgL;
@@ -568,8 +568,7 @@ __device__ void attend_phase(const Params &p, const int *seq_lens, unsigned char
       int first = -1;
       uint32_t off = 0;
       if (good && tok0 < T) {
-        const int pslot = tok0 >> lgP;                                // a length beyond the page-table row is not followed
-        const int pg = (pslot < p.mpp) ? p.page_table[(size_t)b_idx * p.mpp + pslot] : -1;
+        const int pg = page_of(p, b_idx, tok0);
         if (pg < 0 || pg >= p.n_pages) report(p.status, COBS_ERR_BOUNDS);
         else { first = tok0; off = group_place(p, pg, h, tok0); }
       }
@@ -849,7 +848,7 @@ __device__ void umma_producer(const Params &p, const int *seq_lens, const UmmaLi
     if (has) {
       const int c = l.start[w] + o;
       u = c / cpu; ck = c - u * cpu;
-      n_sum = min(seq_lens[u / p.Hkv] / p.L, NB);
+      n_sum = min(tokens_of(seq_lens, u / p.Hkv) / p.L, NB);
       valid = ck * kUBlocks < n_sum;
       tile = l.tile0[w] + (u - l.start[w] / cpu);
     }

@@ -761,7 +761,7 @@ struct ExactScorer {
   __device__ __forceinline__ ExactScorer(const Params &p_, const Unit &, unsigned char *wsm_, uint64_t *, int lane_, bool) : p(p_), wsm(wsm_), lane(lane_) {}
   __device__ __forceinline__ void start(int, int) {}
   __device__ __forceinline__ bool run(const Unit &x, int cb, int ce, float2 *pair) {
-    const int gid = lane >> 2, tig = lane & 3, G = p.G, gpb = p.L >> 4, lgP = 31 - __clz(p.P);
+    const int gid = lane >> 2, tig = lane & 3, G = p.G, gpb = p.L >> 4;
     const int b0 = cb * BLOCKS, b1 = min(ce * BLOCKS, x.n_sum), n = max(0, b1 - b0) * gpb;
     Run rn = {-1e30f, 0.f};                         // of head gid
     const float sl = 1.0f / sqrtf((float)D);
@@ -786,8 +786,7 @@ struct ExactScorer {
     constexpr uint32_t kNone = 0xffffffffu;
     auto resolve = [&](int g) -> uint32_t {
       if (g >= n) return kNone;
-      const int tok0 = b0 * p.L + g * 16, pslot = tok0 >> lgP;
-      const int pg = (pslot < p.mpp) ? p.page_table[(size_t)x.b_idx * p.mpp + pslot] : -1;
+      const int tok0 = b0 * p.L + g * 16, pg = page_of(p, x.b_idx, tok0);
       if (pg < 0 || pg >= p.n_pages) { report(p.status, COBS_ERR_BOUNDS); return kNone; }
       return group_place(p, pg, x.h, tok0);
     };
@@ -1075,8 +1074,8 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
   constexpr int STAGE = 2 * VOFF;
   constexpr int NCP = (16 * CH) / 32;         // cp.async per lane per operand per stage
   const int gid = lane >> 2, tig = lane & 3;
-  const int G = p.G, L = p.L, P = p.P;
-  const int lgL = 31 - __clz(L), lgP = 31 - __clz(P), lgg = lgL - 4;      // L and P are powers of two: shifts, not divisions
+  const int G = p.G, L = p.L;
+  const int lgL = 31 - __clz(L), lgg = lgL - 4;      // L is a power of two: shifts, not divisions
   const uint32_t ring = smem_u32(wsm);
   uint32_t *goff = reinterpret_cast<uint32_t *>(wsm + kAttStages * kAttStage);
   int *gtok = reinterpret_cast<int *>(goff + kTable);
@@ -1125,8 +1124,7 @@ __device__ __forceinline__ void attend_groups(const Params &p, const Unit &x, in
       int first = -1;
       uint32_t off = 0;
       if (good && tok0 < T) {
-        const int pslot = tok0 >> lgP;                                // a length beyond the page-table row is not followed
-        const int pg = (pslot < p.mpp) ? p.page_table[(size_t)x.b_idx * p.mpp + pslot] : -1;
+        const int pg = page_of(p, x.b_idx, tok0);
         if (pg < 0 || pg >= p.n_pages) report(p.status, COBS_ERR_BOUNDS);
         else { first = tok0; off = group_place(p, pg, x.h, tok0); }
       }
@@ -1269,7 +1267,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   x.q = s_q;
   // the unit's query, once per CTA (it may lie in host memory): needed behind the next barrier, stored only when the first copies
   // of the summaries, which wait for the length, are on their way
-  const int T = p.seq_lens[x.b_idx];
+  const int T = tokens_of(p.seq_lens, x.b_idx);
   const bool has_q = tid < G * (D / 8);
   uint4 qv = make_uint4(0u, 0u, 0u, 0u);
   if (has_q) qv = reinterpret_cast<const uint4 *>(p.q + ((size_t)x.b_idx * p.Hq + x.h * G) * D)[tid];
@@ -1300,9 +1298,9 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
     // of group nw i + wi: four groups of 8 KB per warp are the window of 512 tokens with eight warps per unit, and 38 MB in all.
     uint32_t ahead = 0xffffffffu;
     {
-      const int tok = ws + 16 * (nw * lane + wi), pslot = tok >> (31 - __clz(p.P));
-      if ((phases & PH_ATTEND) && lane < 4 && tok < T && pslot < p.mpp) {
-        const int pg = p.page_table[(size_t)x.b_idx * p.mpp + pslot];
+      const int tok = ws + 16 * (nw * lane + wi);
+      if ((phases & PH_ATTEND) && lane < 4 && tok < T) {
+        const int pg = page_of(p, x.b_idx, tok);
         if (pg >= 0 && pg < p.n_pages) ahead = group_place(p, pg, x.h, tok);
       }
     }

@@ -142,3 +142,62 @@ def test_calls_in_a_row_without_host_synchronisation():
     for _ in range(5):
         for a, b in zip(builds(False), want):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dtype,sub,skew", [("fp4", 0, False), ("bf16", 0, False), ("fp32", 0, False), ("fp4", 33, False), ("fp4", 0, True)])
+def test_lengths_that_make_no_sense(dtype, sub, skew):
+    """A negative length counts as an empty sequence in every call, one beyond the page table's row is reported and not
+    followed; the sequences beside them get what they get without them."""
+    B = _binding()
+    L, D, big = 32, 64, 2 ** 31 - 1
+    wl = synth.Workload("lens", 6, 8, 2, D, 70 * L, L, 16, rank=3, topk=7, window=100, summary_dtype=dtype, sub_dim=sub,
+                        key_model="block_offset", shuffle_pages=True, seed=8)
+    inp = to_dev(synth.generate(wl))
+    cfg = B.make_config(wl)
+    kv = B.make_kv(inp)
+    summ = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"), skew=skew)
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, kv, 0, wl.max_blocks, summ, ws)
+    shape = (6, 2, wl.topk)
+
+    def calls(lens):
+        inp["seq_lens"].copy_(torch.tensor(lens, dtype=torch.int32))
+        sel, cnt = torch.full(shape, -7, dtype=torch.int32, device="cuda"), torch.full(shape[:2], -7, dtype=torch.int32, device="cuda")
+        scores = torch.zeros((6, 2, wl.max_blocks), device="cuda")
+        out, lse = torch.zeros((3, 6, 8, D), device="cuda"), torch.zeros((3, 6, 8), device="cuda")
+        sel_x, cnt_x, sel_f, cnt_f = torch.full_like(sel, -7), torch.full_like(cnt, -7), torch.full_like(sel, -7), torch.full_like(cnt, -7)
+        B.cobs_score_select(cfg, inp["q"], summ, inp["seq_lens"], sel, cnt, scores, ws)
+        B.cobs_sparse_decode(cfg, inp["q"], kv, sel, cnt, out[0], lse[0], ws)
+        B.cobs_adaptive_trim(cfg, scores, inp["seq_lens"], 0.3, 1, sel, cnt, ws)
+        B.cobs_sparse_decode(cfg, inp["q"], kv, sel, cnt, out[1], lse[1], ws)
+        B.cobs_decode_step(cfg, inp["q"], kv, summ, out[2], lse[2], sel_f, cnt_f, ws)
+        B.cobs_exact_select(cfg, inp["q"], kv, sel_x, cnt_x, scores, ws)
+        s2 = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"), skew=skew)
+        B.cobs_build_summaries(cfg, kv, 0, wl.max_blocks, s2, ws)
+        # (outputs as their bits: an empty sequence's rows are not numbers)
+        return [t.view(torch.int32) for t in (sel, cnt, sel_f, cnt_f, sel_x, cnt_x)] + \
+               [t.view(torch.int32)[i] for t in (out, lse) for i in range(3)], [s2.mean, s2.xi, s2.scale]
+
+    want, built = calls([70 * L, 0, 0, 9, 51 * L + 3, 0])
+    assert B.cobs_read_status(ws) == 0
+    got, built2 = calls([70 * L, -1, -70 * L, 9, 51 * L + 3, -2 ** 31])
+    assert B.cobs_read_status(ws) == 0
+    for a, b in zip(got + built2, want + built):
+        assert torch.equal(a, b)
+    assert torch.all(got[1][[1, 2, 5]] == 0) and torch.all(got[0][[1, 2, 5]] == -1)
+    got, _ = calls([70 * L, big, 0, 9, 51 * L + 3, big - 15])
+    assert B.cobs_read_status(ws) == 6
+    B.cobs_reset_status(ws)
+    for a, b in zip(got, want):
+        assert torch.equal(a[[0, 2, 3, 4]], b[[0, 2, 3, 4]])
+
+    # and no token is appended where there is no place for it
+    lens = [70 * L, -1, big, 9, 51 * L + 3, -2 ** 31]
+    inp["seq_lens"].copy_(torch.tensor(lens, dtype=torch.int32))
+    k_new = torch.ones((6, 2, D), dtype=torch.bfloat16, device="cuda")
+    pool = inp["k_pages"].clone()
+    B.cobs_append_token(cfg, k_new, k_new, inp, ws)
+    assert B.cobs_read_status(ws) == 6
+    assert inp["seq_lens"].tolist() == [70 * L, -1, big, 10, 51 * L + 4, -2 ** 31]
+    changed = (inp["k_pages"] != pool).any(-1).sum()
+    assert int(changed) == 2 * 2
