@@ -20,7 +20,7 @@ cudaError_t launch_exact_mass(const Params &p, cudaStream_t stream);
 cudaError_t launch_adaptive_trim(const Params &p, float tau, int k_min, cudaStream_t stream);
 cudaError_t launch_unit_step(const Params &p, int phases, cudaStream_t stream);
 bool unit_score_supported(const Params &p);
-bool unit_keys_fit(const Params &p);
+bool unit_exact_supported(const Params &p);
 cudaError_t launch_unit_exact(const Params &p, cudaStream_t stream);
 cudaError_t launch_fused_umma(Params p, int phases, cudaStream_t stream);
 bool umma_score_supported(const Params &p);
@@ -209,7 +209,7 @@ static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
 }
 
 // Scoring and selection, with the attention or without: one launch.  The generic scoring and selection kernels are for what the
-// unit kernel does not cover.
+// unit kernel does not cover or is slower at (see unit_score_supported).
 static cudaError_t launch_score_step(const Params &p, int phases, cudaStream_t s) {
   if (umma_score_supported(p)) {
     const cudaError_t e = launch_fused_umma(p, phases, s);
@@ -367,7 +367,7 @@ int32_t cobs_exact_select(const cobs_config *cfg, const void *q, const cobs_kv *
   p.q = static_cast<const __nv_bfloat16 *>(q);
   p.sel_idx = sel_idx; p.sel_cnt = sel_cnt; p.scores = scores_or_null;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (unit_keys_fit(p)) return cuda_status(launch_unit_exact(p, s));
+  if (unit_exact_supported(p)) return cuda_status(launch_unit_exact(p, s));
   if (launch_exact_mass(p, s) != cudaSuccess) return COBS_ERR_CUDA;
   return cuda_status(launch_select(p, s));
 }

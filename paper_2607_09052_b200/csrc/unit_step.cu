@@ -1562,10 +1562,30 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
 
 }  // namespace
 
-// Whether this kernel covers a configuration's scoring phase: everything but the diagonal-skew variant of FP4 summaries, and
-// units whose scores do not fit a CTA's shared memory.
-bool unit_keys_fit(const Params &p) { return p.NB <= kMaxKeys; }
-bool unit_score_supported(const Params &p) { return unit_keys_fit(p) && !(p.skew && p.summ_dtype == COBS_SUMM_FP4_E2M1); }
+// Whether this kernel does a configuration's scoring: everything but the diagonal-skew variant of FP4 summaries, units whose scores
+// do not fit a CTA's shared memory, and one or two units with so much to score row by row (fp32 summaries, bf16 ones in a subspace
+// or with the skew) that sixteen SMs each take longer than the generic kernels' whole grid.  Elements of a unit's means and
+// factors, times generic / this kernel (both in one loop, and with L2 flushed before each pass):
+//   1 unit   fp32  4.7M .93 / 1.07   8.9M .80 / 1.08   9.4M .74 / .84   18M .83 / .74   36M .57 / .55      drawn at 8M
+//            bf16  12M 1.16 / 1.05   18M 1.25 / 1.00   24M .80 / .80   36M .72 / .83                       at 24M
+//   2 units  fp32  9M 1.16 / 1.12   14M .98 / .94   18M .99 / 1.06   27M .91 / .98   36M .80 / .87         at 24M
+//            bf16  24M 1.18 / 1.25   36M 1.11 / 1.14                       3 units  fp32  36M 1.07 / 1.21
+bool unit_score_supported(const Params &p) {
+  if (p.NB > kMaxKeys || (p.skew && p.summ_dtype == COBS_SUMM_FP4_E2M1)) return false;
+  const long long units = (long long)p.B * p.Hkv, elements = (long long)p.NB * (p.D + p.r * p.Ds);
+  const bool fp32 = p.summ_dtype == COBS_SUMM_FP32, rows = fp32 || (p.summ_dtype == COBS_SUMM_BF16 && (p.u_q || p.skew));
+  if (!rows || units > 2) return true;
+  return (units == 1) ? elements < (fp32 ? 8LL << 20 : 24LL << 20) : !fp32 || elements < 24LL << 20;
+}
+// The same for the exact masses: all but few units with many keys, whose clusters are a few dozen SMs against the whole grid of
+// exact_mass_kernel.  (One unit of 131 072 tokens, D 128, L 64, four heads: 24.6 us there, 36.6 here; of 65 536: 20.5 / 22.4; of 32 768:
+// 18.5 / 14.0.  Two of 131 072: 28.7 / 36.8; three: 32.8 / 37.3; four: 43.7 / 37.7.  Eight heads, whose selection costs that route more:
+// one unit of 98 304: 32.8 / 30.1, of 131 072: 32.8 / 36.9, two 37.3 / 37.2, three 43.0 / 37.2.  Blocks of 16, whose number does: one of
+// 131 072 with D 64 47.1 / 43.4.  Blocks of 128, 512 of them, a group of blocks per warp: 20.5 / 15.3; 1 024 of them: 20.5 / 25.1.)
+bool unit_exact_supported(const Params &p) {
+  const bool many = p.L >= 64 && p.NB >= 1024 && (long long)p.NB * p.L * p.D * 2 >= (16LL << 20) * (p.G > 4 ? 2 : 1);
+  return p.NB <= kMaxKeys && !(many && p.B * p.Hkv <= (p.G > 4 ? 2 : 3));
+}
 
 // Exact block masses, group scores and selection.
 cudaError_t launch_unit_exact(const Params &p, cudaStream_t stream) {
