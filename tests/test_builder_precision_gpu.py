@@ -43,3 +43,65 @@ def test_factors_do_not_lose_the_bits_of_the_mean(D, sub, rank, L, mean):
     n2 = (x * x).sum(-1)
     resid = (x @ sigma - n2[..., None] * x).norm(dim=-1) / (lam0[..., None] * n2.sqrt())
     assert float(resid.max()) <= 24 * 2.0 ** -24, float(resid.max())
+
+
+def degenerate_keys(kind, n, L, D, gen):
+    """n blocks of L keys [n, L, D] with fewer directions than factors, or with eigenvalues that coincide."""
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    if kind == "equal":                                  # two equal eigenvalues, everything else zero: exact in bf16
+        t = torch.arange(L, device="cuda") % 4
+        k = torch.zeros((n, L, D), device="cuda")
+        k[:, :, 5] = 2.0 * ((t == 0).float() - (t == 1).float())
+        k[:, :, D - 3] = 2.0 * ((t == 2).float() - (t == 3).float())
+        return k
+    if kind == "constant":
+        return rnd(n, 1, D).expand(n, L, D)
+    if kind == "zero":
+        return torch.zeros((n, L, D), device="cuda")
+    if kind == "three":                                  # three distinct keys
+        return rnd(n, 3, D)[:, torch.arange(L, device="cuda") % 3]
+    return rnd(n, L, 2) @ rnd(n, 2, D)                   # two directions and the rounding of their products
+
+
+@pytest.mark.parametrize("kind", ["equal"])
+@pytest.mark.parametrize("L,D,sub,rank,n", [(16, 64, 0, 4, 70), (32, 128, 0, 8, 40), (64, 128, 0, 4, 40), (64, 128, 0, 4, 5), (128, 64, 0, 3, 40),
+                                            (64, 128, 85, 4, 40), (128, 128, 85, 8, 9), (16, 128, 33, 16, 40)])
+def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
+    """Every block of the call degenerate, fewer of them than the careful kernel's CTAs have threads and more: the rank-r matrix
+    within the errors of an eigenvalue, zeros where there is no direction.  Blocks with two equal eigenvalues are those that
+    the one-warp kernel declines: it has marked them all (in the workspace's score area), and the careful kernel has done them."""
+    from paper_2607_09052_b200 import binding as B
+    wl = synth.Workload("degenerate", 4, 8, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
+                        key_model="iid", shuffle_pages=True, seed=7)
+    inp = synth.generate(wl, "cuda")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    keys = degenerate_keys(kind, 4 * 2 * n, L, D, gen).bfloat16().view(4, 2, n * L // 16, 16, D)
+    inp["k_pages"][inp["page_table"].long().view(-1)] = keys.transpose(1, 2).reshape(-1, 2, 16, D)
+    cfg = B.make_config(wl)
+    summ = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"))
+    summ.xi.fill_(255)
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, B.make_kv(inp), 0, wl.max_blocks, summ, ws)
+    assert B.cobs_read_status(ws) == 0
+    marks_at = (256 + 6 * 65535 * 4 + 255) // 256 * 256          # behind the status block and the counters
+    marks = ws[marks_at:marks_at + 4 * 8 * n].view(torch.int32)
+    if kind == "equal" and not sub:
+        assert int(marks.sum()) == 8 * n
+    elif kind in ("constant", "zero", "three"):
+        assert int(marks.sum()) == 0
+    _, xi, _ = B.summary_views(cfg, summ)
+    K = keys.view(4, 2, n, L, D).double()
+    K = K - K.mean(3, keepdim=True)
+    if sub:
+        K = torch.einsum("bhnld,hds->bhnls", K, inp["u_q"].double())
+    lam, v = torch.linalg.eigh(K.transpose(-1, -2) @ K / L)
+    x = xi.double()
+    if kind in ("constant", "zero"):
+        assert torch.all(xi == 0)
+        return
+    # at most the eigenvalues' own error for each direction that is left out, and for those that are not: 2^-20 of the largest
+    top = (v[..., -rank:] * lam[..., None, -rank:]) @ v[..., -rank:].transpose(-1, -2)
+    err = torch.linalg.matrix_norm(x.transpose(-1, -2) @ x - top, ord=2) / lam[..., -1]
+    assert float(err.max()) <= 4 * 2.0 ** -20, float(err.max())
+    prod = (x @ x.transpose(-1, -2)).abs() / lam[..., -1, None, None]
+    assert float(torch.triu(prod, 1).max()) <= 2.0 ** -17
