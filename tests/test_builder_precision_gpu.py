@@ -63,7 +63,7 @@ def degenerate_keys(kind, n, L, D, gen):
     return rnd(n, L, 2) @ rnd(n, 2, D)                   # two directions and the rounding of their products
 
 
-@pytest.mark.parametrize("kind", ["equal", "three", "two"])
+@pytest.mark.parametrize("kind", ["equal", "constant", "zero", "three", "two"])
 @pytest.mark.parametrize("L,D,sub,rank,n", [(16, 64, 0, 4, 70), (32, 128, 0, 8, 40), (64, 128, 0, 4, 40), (64, 128, 0, 4, 5), (128, 64, 0, 3, 40),
                                             (64, 128, 85, 4, 40), (128, 128, 85, 8, 9), (16, 128, 33, 16, 40)])
 def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
