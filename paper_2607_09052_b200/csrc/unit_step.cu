@@ -79,6 +79,7 @@ constexpr int kMaxKeys = 24576;                              // score keys that 
 // how a launch lays out a CTA (chosen on the host, see launch_t)
 struct Plan {
   int W, C;
+  int u0;                                                    // the launch's first unit
   int key_off;                                               // byte offset of the score keys in dynamic shared memory
   int e_off;                                                 // of the e buffer, or -1: it is in the workspace
 };
@@ -226,6 +227,9 @@ struct Scorer {
   static constexpr int ROWS_MAX = ROWS_CAP < COBS_MAX_RANK ? ROWS_CAP : COBS_MAX_RANK;   // rows a batch can hold at most
   static_assert((kStage - MEAN_BYTES - 16 * 32 - 16 * COBS_MAX_RANK * 4 - 16) / (16 * ROWB) >= 1, "stage too small");
   static constexpr int RG = 4;                    // FP4 factor rows decoded and multiplied together
+  static size_t unit_bytes(const Params &p) {     // what a unit's scores are computed from
+    return (size_t)p.NB * (D * 2 + p.r * (ROWB + (FP4 ? (p.scale_dtype == COBS_SCALE_FP16 ? 2 : 4) : 0)));
+  }
 
   const Params &p;
   unsigned char *wsm;
@@ -546,6 +550,7 @@ struct RowScorer {
   static constexpr int MROW = D * ES + PAD;
   static constexpr int ROOM = kStage / 16 - PAD - 32;       // bytes of a block's rows in a batch (the copy takes up to 15 more at either end)
   static_assert(ROOM >= D * ES, "a stage must hold a row of every block");
+  static size_t unit_bytes(const Params &p) { return (size_t)p.NB * (D + p.r * p.Ds) * ES; }
   const Params &p;
   unsigned char *wsm;
   uint32_t ring, bar0;
@@ -755,6 +760,7 @@ struct ExactScorer {
   static constexpr int CH = D / 8, KS = D / 16, ROWB = D * 2, STAGE = 16 * ROWB, NCP = (16 * CH) / 32;
   static constexpr int NST = (D == 128) ? 6 : 12;   // 16-token groups in the ring: the two being used, 16 to 20 KB on their way
   static_assert(NST * STAGE <= kRing && NST % 2 == 0, "the ring must fit");
+  static size_t unit_bytes(const Params &p) { return (size_t)p.NB * p.L * ROWB; }
   const Params &p;
   unsigned char *wsm;
   int lane;
@@ -1267,7 +1273,7 @@ __global__ void __launch_bounds__(kMaxW * 32, 1) unit_step_kernel(Params p, int 
   __shared__ int s_sel[COBS_MAX_TOPK];
   __shared__ int s_lost;                                   // a wait for copies ran out: the outputs are undefined, the rings not ours
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, W = pl.W, C = pl.C, nthr = W * 32;
-  const int u = blockIdx.x / C, rank = blockIdx.x - u * C;
+  const int u = pl.u0 + blockIdx.x / C, rank = blockIdx.x % C;
   const int G = p.G, L = p.L, NB = p.NB;
   if (C > 1) cluster_arrive();                             // (waited for before the first access to another CTA's memory)
   if (tid < 2 * 2 * kMaxW) (&s_cnt[0][0][0])[tid] = 0u;
@@ -1533,31 +1539,47 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   // Eight warps per CTA and the largest cluster with which all units are resident at once; no larger than gives every warp a
   // chunk or a group.  (8 units of 32k: 20.5 us with clusters of 4 to 10, 36.7 with 16, of which only seven fit; 32 units:
   // 29.9 / 27.9 / 26.7 us with 2 / 3 / 4; 128 units of 128k: 98 us with one CTA of eight warps, 118 with two of four.)
-  // More units than SMs: four warps per CTA, two CTAs per SM (192 ragged units of 12k: 45 us, 55 with eight warps in two waves).
-  Plan pl;
+  // More units than SMs: four warps per CTA, two CTAs per SM (192 ragged units of 12k: 45 us, 55 with eight warps in two waves); but
+  // three waves of eight warps rather than two of four whose second is half empty (320 units of 32k 85 -> 77 us, 440 88 -> 85, 448
+  // would be 89 -> 101; 304 to 440 units of 2k equal; ragged ones of 12k 50 -> 53 at 304, equal from 352 on).
   const int units = p.B * p.Hkv, n_chunks = (p.NB + NBLK - 1) / NBLK;
   const int groups = (p.topk + (p.window + p.L - 1) / p.L + 1) * (p.L / 16);
   // (the same for a scoring call and a whole step: the order of the sums, and so the selection's last bits, follow the split)
   const int work = (phases & PH_SCORE) ? max(n_chunks, groups) : groups;
-  pl.W = (units <= fit[dev][1].load(std::memory_order_relaxed)) ? kMaxW : kMaxW / 2;
-  pl.C = 1;
-  for (int c = 2; c <= kMaxC && pl.W == kMaxW && (c - 1) * pl.W < work; ++c)
-    if (fit[dev][c].load(std::memory_order_relaxed) >= units) pl.C = c;
-  const int W = pl.W, C = pl.C, cap = (W == kMaxW) ? kSmemOne : kSmemTwo;
-  const int key_bytes = (phases & PH_SCORE) ? (p.NB * 4 + 15) / 16 * 16 : 0;
-  const int e_bytes = (phases & PH_SCORE) ? p.G * NBLK * ((n_chunks + C - 1) / C) * 4 : 0;
-  int off = W * kRing;
-  if (off + key_bytes <= cap) { pl.key_off = off; off += key_bytes; } else pl.key_off = 0;      // over the rings: scoring is over by then
-  if (off + e_bytes <= cap) { pl.e_off = off; off += e_bytes; } else pl.e_off = -1;
-  at[0].val.clusterDim.x = (unsigned)C;
-  cfg.gridDim = dim3((unsigned)(units * C));
-  cfg.blockDim = dim3((unsigned)(W * 32));
-  cfg.dynamicSmemBytes = (size_t)off;
-  cfg.stream = stream;
-  cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kern, p, phases, pl);
-  count_launch();
-  return e;
+  const int full = max(1, fit[dev][1].load(std::memory_order_relaxed));      // CTAs of eight warps that are resident at a time: SMs
+  auto launch = [&](int u0, int n) -> cudaError_t {
+    Plan pl;
+    pl.u0 = u0;
+    pl.W = (n <= full || (n + full - 1) / full == 3) ? kMaxW : kMaxW / 2;
+    pl.C = 1;
+    for (int c = 2; c <= kMaxC && n <= full && (c - 1) * pl.W < work; ++c)
+      if (fit[dev][c].load(std::memory_order_relaxed) >= n) pl.C = c;
+    const int W = pl.W, C = pl.C, cap = (W == kMaxW) ? kSmemOne : kSmemTwo;
+    const int key_bytes = (phases & PH_SCORE) ? (p.NB * 4 + 15) / 16 * 16 : 0;
+    const int e_bytes = (phases & PH_SCORE) ? p.G * NBLK * ((n_chunks + C - 1) / C) * 4 : 0;
+    int off = W * kRing;
+    if (off + key_bytes <= cap) { pl.key_off = off; off += key_bytes; } else pl.key_off = 0;      // over the rings: scoring is over by then
+    if (off + e_bytes <= cap) { pl.e_off = off; off += e_bytes; } else pl.e_off = -1;
+    at[0].val.clusterDim.x = (unsigned)C;
+    cfg.gridDim = dim3((unsigned)(n * C));
+    cfg.blockDim = dim3((unsigned)(W * 32));
+    cfg.dynamicSmemBytes = (size_t)off;
+    cfg.stream = stream;
+    cfg.numAttrs = 2;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, p, phases, pl);
+    count_launch();
+    return err;
+  };
+  // Up to a quarter more units than SMs, with 1.2 MB or more to score each: one unit per SM, then the others in clusters.  (With four
+  // warps per CTA nearly every SM would have one such CTA.  160 / 184 units of 128k, 4 MB each: 147 -> 119 / 152 -> 135 us in a loop,
+  // 149 -> 144 / 156 -> 157 with L2 flushed before each; fp32 at 32k, 152 / 176 units: 115 -> 93 / 122 -> 96, flushed 128 -> 119 / 132 -> 121;
+  // exact masses of 32k, 152: 233 -> 209, 234 -> 225.  192 units of 128k: 152 -> 144, 160 -> 161.  With 0.8 MB to score, 64k, 152: 114 -> 97,
+  // 116 -> 124; with 0.3, 32k: 41 -> 44, 64 -> 72.)
+  if ((phases & PH_SCORE) && units > full && units <= full + full / 4 && SCORER::unit_bytes(p) >= 1200000) {
+    if ((e = launch(0, full)) != cudaSuccess) return e;
+    return launch(full, units - full);
+  }
+  return launch(0, units);
 }
 
 }  // namespace

@@ -142,7 +142,8 @@ def test_units_with_many_rows_to_score(dtype, sub, rank, D, hkv, skew, n):
 
 @pytest.mark.parametrize("n,hkv,L,D,G", [(3, 1, 16, 64, 2), (5000, 1, 16, 64, 2), (5000, 3, 16, 64, 2), (24576, 2, 16, 64, 2), (24577, 2, 16, 64, 2),
                                          (1023, 1, 64, 128, 4), (1024, 1, 64, 128, 4), (1025, 3, 64, 128, 4), (1024, 4, 64, 128, 4),
-                                         (2048, 2, 64, 128, 8), (2048, 3, 64, 128, 8), (1023, 1, 128, 64, 1), (1024, 3, 128, 64, 1)])
+                                         (2048, 2, 64, 128, 8), (2048, 3, 64, 128, 8), (1023, 1, 128, 64, 1), (1024, 3, 128, 64, 1),
+                                         (292, 152, 16, 128, 2), (300, 149, 16, 128, 1), (293, 185, 16, 128, 1), (293, 186, 16, 128, 1)])
 def test_exact_selection_of_long_units(n, hkv, L, D, G):
     """The exact block masses of long contexts, on both sides of the lines between the kernels that take them: against direct sums
     in 64 bits."""
