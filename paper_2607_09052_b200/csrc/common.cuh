@@ -64,9 +64,10 @@ void count_tcgen05_launch();
 // kernel is resident and is not ordered by the wait.  (A kernel launched without the attribute - the exact masses beyond the step
 // kernel's capacity, the tcgen05 variant, the conversion hook - is not overtaken, nor does one that does not say
 // launch_dependents let its successor in early.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  pdl_wait();
 }
 template <class... KArgs, class... Args>
 static cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {

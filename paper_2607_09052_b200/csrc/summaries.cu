@@ -789,7 +789,9 @@ __global__ void __launch_bounds__(kBuildThreads, (TL == 8) ? 2 : 4)
 build_kernel(Params p, int block_begin, int block_end, int solver, const int *flags, int n) {
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_flag[kBuildThreads];
-  pdl_begin();
+  // (with flags the next kernel is let in as this one's CTAs leave, not before: nearly all leave at once, and CTAs of the next one
+  // that are placed around them share SMs while others stay empty: builds of 128 blocks of 128 tokens, rank 4, in a row 174 -> 118 us)
+  if (flags) pdl_wait(); else pdl_begin();
   const int n_range = block_end - block_begin;
   if (!flags) {
     build_block<TL>(p, sm, blockIdx.x / n_range, block_begin + (int)(blockIdx.x % n_range), solver);
