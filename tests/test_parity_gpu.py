@@ -335,10 +335,11 @@ def test_ragged_lengths_and_degenerate_cases():
 
 
 def test_selection_exact_ties_for_every_blocks_per_thread_layout():
-    """The selection team spreads a unit's blocks 4, 8 or 16 per thread depending on the unit's block count.
-    Synthetic summaries with two kinds of block (every 16th block "hot", the rest "cold", identical within a kind)
+    """The selection spreads a unit's candidates over one warp or over the CTA, two or eight keys per thread, depending on
+    their number; these lengths lie in the layouts of four keys per lane (95 candidates), two (507 to 509) and eight per
+    thread (1020 and more).  (Both sides of every boundary, and four warps per CTA: test_selection_gpu.py.)  Synthetic summaries with two kinds of block (every 16th block "hot", the rest "cold", identical within a kind)
     make every score one of two values, exactly: the top-k must be all hot candidates plus the LOWEST-index cold
-    ones (ties -> lower index), for block counts on both sides of each layout boundary, in one batch."""
+    ones (ties -> lower index), in one batch."""
     B = _binding()
     L, D, G, NB, topk = 16, 64, 4, 2048, 48
     n_sums = [3, 100, 511, 512, 513, 1024, 1025, 2047, 2048]
@@ -549,8 +550,8 @@ def test_builder_writes_skew_scalars():
 
 
 def test_context_beyond_the_fused_selection_capacity():
-    """4096 blocks per unit: more than the step kernel's selection team holds (2048), so scoring and selection
-    take the generic kernels and only attention runs in the persistent kernel; same parity bar."""
+    """4096 blocks per unit: more than the step kernel's selection holds in registers (2048), so its top-k reads the keys
+    from shared memory in every round; same parity bar.  (Units beyond the step kernel itself: test_selection_gpu.py.)"""
     wl = synth.Workload("long", 1, 4, 1, 128, 4096 * 64, 64, 64, rank=4, topk=16, window=512, summary_dtype="fp4",
                         key_model="block_offset", planted=4, shuffle_pages=False, seed=41)
     run_stage_s(wl)
@@ -769,8 +770,8 @@ def test_length_beyond_the_page_table_is_reported_not_followed():
 
 def test_one_workspace_serves_calls_of_different_shapes():
     """A workspace as large as the largest of three shapes needs, used by their steps in a mixed order: every step
-    gives the bits it gives on a workspace of its own (the hand-off counters of the persistent kernel live at the same
-    places for every shape, and each launch clears what the previous one left, however many units that one had)."""
+    gives the bits it gives on a workspace of its own (no step leaves anything in the workspace that another depends on,
+    whatever the shapes)."""
     B = _binding()
 
     def setup(wl):
@@ -808,8 +809,8 @@ def test_one_workspace_serves_calls_of_different_shapes():
 
 
 def test_step_replays_from_a_cuda_graph():
-    """The fused step captured once and replayed: its hand-off counters alternate between two sets by themselves
-    (no host state), so odd and even replays give the bits of a plain call; the status word stays clear."""
+    """The fused step captured once and replayed: no state is kept between launches, on the host or in the workspace, so
+    every replay gives the bits of a plain call; the status word stays clear."""
     B = _binding()
     wl = WL["cfg2_32k"].replace(seq_len=8192)
     inp = to_dev(synth.generate(wl))
@@ -966,7 +967,8 @@ def test_builder_jacobi_route(case, monkeypatch):
 @pytest.mark.parametrize("solver", ["tridiagonal", "jacobi"])
 @pytest.mark.parametrize("rank,L,D", [(12, 64, 128), (16, 128, 64), (15, 32, 64)])
 def test_builder_ranks_above_eight(rank, L, D, solver, monkeypatch):
-    """More factors than the builder has warps: two eigenvectors per warp in the inverse iteration."""
+    """More than eight factors: two lanes per eigenvalue in the one-warp builder's counts, two eigenvectors per warp in the
+    careful kernel."""
     if solver == "jacobi":
         monkeypatch.setenv("COBS_BUILD_SOLVER", "jacobi")
     wl = synth.Workload("highrank", 1, 4, 2, D, 6 * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32",

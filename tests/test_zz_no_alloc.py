@@ -1,6 +1,5 @@
-"""cobs_sparse_decode_static: the attention step for callers that are not allowed to allocate device memory
-(its scratch is a fixed array inside the library).  It must give what cobs_sparse_decode gives, call after call,
-although every call reuses the same scratch and finds the previous call's leftovers in it."""
+"""cobs_sparse_decode_static: the attention step for callers that are not allowed to allocate device memory: it takes no
+workspace and holds no memory of its own.  It must give what cobs_sparse_decode gives, call after call."""
 
 import numpy as np
 import pytest
@@ -15,8 +14,7 @@ pytestmark = pytest.mark.gpu
 def test_static_scratch_variant_matches_workspace_variant_on_two_calls_in_a_row():
     from paper_2607_09052_b200 import binding as B
     base = synth.named_workloads()["cfg4_128k"]
-    # the second call has another batch, context and top-k: it finds the first call's counters and partials laid
-    # out differently in the shared scratch
+    # the second call has another batch, context and top-k
     for call, (seed, batch, seq_len, topk) in enumerate(((41, 3, 8192, 64), (42, 2, 4096, 24))):
         wl = base.replace(batch=batch, seq_len=seq_len, topk=topk)
         cfg = B.make_config(wl)
