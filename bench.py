@@ -444,7 +444,7 @@ def run_ours(args):
 
     peak, peak_kind = read_peaks()
     value = world * step_bytes / (ms_per_step * 1e-3) / 1e9
-    # the step is ONE launch of the persistent kernel, so its launch duration is the step time
+    # the step is ONE launch of the step kernel, so its launch duration is the step time
     kernels_per_step = launches / args.steps
     achieved = step_bytes / (ms_per_step * 1e-3) / 1e9 if world == 1 else value / world
     line = {
