@@ -1540,17 +1540,19 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   // chunk or a group.  (8 units of 32k: 20.5 us with clusters of 4 to 10, 36.7 with 16, of which only seven fit; 32 units:
   // 29.9 / 27.9 / 26.7 us with 2 / 3 / 4; 128 units of 128k: 98 us with one CTA of eight warps, 118 with two of four.)
   // More units than SMs: four warps per CTA, two CTAs per SM (192 ragged units of 12k: 45 us, 55 with eight warps in two waves); but
-  // three waves of eight warps rather than two of four whose second is half empty (320 units of 32k 85 -> 77 us, 440 88 -> 85, 448
-  // would be 89 -> 101; 304 to 440 units of 2k equal; ragged ones of 12k 50 -> 53 at 304, equal from 352 on).
+  // three waves of eight warps rather than two of four whose second is half empty, where there is work for eight (320 units of 32k
+  // 85 -> 77 us, 440 88 -> 85, 448 would be 89 -> 101; ragged ones of 12k 50 -> 53 at 304, equal from 352 on; 320 with fp32 summaries
+  // of 128 blocks 92 -> 84, of 64 it would be 71 -> 82).
   const int units = p.B * p.Hkv, n_chunks = (p.NB + NBLK - 1) / NBLK;
   const int groups = (p.topk + (p.window + p.L - 1) / p.L + 1) * (p.L / 16);
-  // (the same for a scoring call and a whole step: the order of the sums, and so the selection's last bits, follow the split)
-  const int work = (phases & PH_SCORE) ? max(n_chunks, groups) : groups;
+  // (the same for a scoring call and a whole step: the order of the sums, and so the selection's last bits, follow the split; a single
+  // chunk has no order)
+  const int work = (phases == PH_SCORE && n_chunks == 1) ? 1 : (phases & PH_SCORE) ? max(n_chunks, groups) : groups;
   const int full = max(1, fit[dev][1].load(std::memory_order_relaxed));      // CTAs of eight warps that are resident at a time: SMs
   auto launch = [&](int u0, int n) -> cudaError_t {
     Plan pl;
     pl.u0 = u0;
-    pl.W = (n <= full || (n + full - 1) / full == 3) ? kMaxW : kMaxW / 2;
+    pl.W = (n <= full || ((n + full - 1) / full == 3 && n_chunks >= kMaxW)) ? kMaxW : kMaxW / 2;
     pl.C = 1;
     for (int c = 2; c <= kMaxC && n <= full && (c - 1) * pl.W < work; ++c)
       if (fit[dev][c].load(std::memory_order_relaxed) >= n) pl.C = c;
@@ -1573,7 +1575,8 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
   // Up to a quarter more units than SMs, with 1.2 MB or more to score each: one unit per SM, then the others in clusters.  (With four
   // warps per CTA nearly every SM would have one such CTA.  160 / 184 units of 128k, 4 MB each: 147 -> 119 / 152 -> 135 us in a loop,
   // 149 -> 144 / 156 -> 157 with L2 flushed before each; fp32 at 32k, 152 / 176 units: 115 -> 93 / 122 -> 96, flushed 128 -> 119 / 132 -> 121;
-  // exact masses of 32k, 152: 233 -> 209, 234 -> 225.  192 units of 128k: 152 -> 144, 160 -> 161.  With 0.8 MB to score, 64k, 152: 114 -> 97,
+  // exact masses of 32k, 152: 233 -> 209, 234 -> 225.  192 units of 128k: 152 -> 144, 160 -> 161, of 64k with
+  // bf16 summaries 108 -> 114, 116 -> 146.  With 0.8 MB to score, 64k, 152: 114 -> 97,
   // 116 -> 124; with 0.3, 32k: 41 -> 44, 64 -> 72.)
   if ((phases & PH_SCORE) && units > full && units <= full + full / 4 && SCORER::unit_bytes(p) >= 1200000) {
     if ((e = launch(0, full)) != cudaSuccess) return e;
@@ -1585,17 +1588,21 @@ cudaError_t launch_t(const Params &p, int phases, cudaStream_t stream) {
 }  // namespace
 
 // Whether this kernel does a configuration's scoring: everything but the diagonal-skew variant of FP4 summaries, units whose scores
-// do not fit a CTA's shared memory, and one or two units with so much to score row by row (fp32 summaries, bf16 ones in a subspace
-// or with the skew) that sixteen SMs each take longer than the generic kernels' whole grid.  Elements of a unit's means and
-// factors, times generic / this kernel (both in one loop, and with L2 flushed before each pass):
+// do not fit a CTA's shared memory, and two kinds of call in which warps that score row by row (fp32 summaries, bf16 ones in a
+// subspace or with the skew) are too few for long: one or two units with so much to score that sixteen SMs each take longer than the
+// generic kernels' whole grid, and very many units of a single chunk, which one warp of each CTA scores.  Elements of a unit's
+// means and factors, step with generic scoring / with this kernel (in a loop, and with L2 flushed before each pass):
 //   1 unit   fp32  4.7M .93 / 1.07   8.9M .80 / 1.08   9.4M .74 / .84   18M .83 / .74   36M .57 / .55      drawn at 8M
 //            bf16  12M 1.16 / 1.05   18M 1.25 / 1.00   24M .80 / .80   36M .72 / .83                       at 24M
 //   2 units  fp32  9M 1.16 / 1.12   14M .98 / .94   18M .99 / 1.06   27M .91 / .98   36M .80 / .87         at 24M
+//   fp32, rank 4 / 8, 4 blocks: 512 units .91 / .76, 1 024 .76 / .66; 16 blocks: 512 1.08 / 1.03, 1 024 .97 / .90, 2 048 1.00 / .90;
+//   32 blocks: 1 024 1.18 / 1.11; bf16 in a subspace, 4 blocks: 1 024 1.04                                 at 64 units per block
 //            bf16  24M 1.18 / 1.25   36M 1.11 / 1.14                       3 units  fp32  36M 1.07 / 1.21
 bool unit_score_supported(const Params &p) {
   if (p.NB > kMaxKeys || (p.skew && p.summ_dtype == COBS_SUMM_FP4_E2M1)) return false;
   const long long units = (long long)p.B * p.Hkv, elements = (long long)p.NB * (p.D + p.r * p.Ds);
   const bool fp32 = p.summ_dtype == COBS_SUMM_FP32, rows = fp32 || (p.summ_dtype == COBS_SUMM_BF16 && (p.u_q || p.skew));
+  if (fp32 && p.NB <= 16 && units > 296 && units >= 64LL * p.NB) return false;
   if (!rows || units > 2) return true;
   return (units == 1) ? elements < (fp32 ? 8LL << 20 : 24LL << 20) : !fp32 || elements < 24LL << 20;
 }

@@ -11,9 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("batch,hkv,blocks,rank,dtype,sub", [
-    (149, 1, 140, 16, "fp32", 0), (23, 8, 140, 16, "fp32", 0), (37, 5, 140, 16, "fp32", 0), (31, 6, 140, 16, "fp32", 0),      # 149, 184, 185, 186 units
+    (149, 1, 140, 16, "fp32", 0), (23, 8, 140, 16, "fp32", 0), (185, 1, 140, 16, "fp32", 0), (31, 6, 140, 16, "fp32", 0),      # 149, 184, 185, 186 units
     (19, 8, 140, 16, "fp32", 64), (19, 8, 280, 16, "bf16", 0), (19, 8, 900, 16, "fp4", 0), (19, 8, 40, 16, "fp32", 0),
-    (37, 8, 40, 4, "fp4", 0), (297, 1, 40, 4, "bf16", 0), (111, 4, 40, 4, "fp4", 33), (89, 5, 40, 4, "fp4", 0)])               # 296, 297, 444, 445
+    (37, 8, 130, 4, "fp4", 0), (297, 1, 112, 4, "bf16", 0), (297, 1, 113, 4, "bf16", 0), (111, 4, 130, 4, "fp4", 33), (89, 5, 120, 4, "fp4", 0),      # 296 to 445
+    (128, 4, 8, 4, "fp32", 0), (511, 1, 8, 4, "fp32", 33), (74, 4, 4, 4, "fp32", 0), (99, 3, 4, 4, "fp32", 0), (64, 16, 16, 8, "fp32", 0), (64, 17, 17, 8, "fp32", 0)])
 def test_more_units_than_sms(batch, hkv, blocks, rank, dtype, sub):
     from paper_2607_09052_b200 import binding as B
     L = 16
