@@ -105,3 +105,45 @@ def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
     assert float(err.max()) <= 4 * 2.0 ** -20, float(err.max())
     prod = (x @ x.transpose(-1, -2)).abs() / lam[..., -1, None, None]
     assert float(torch.triu(prod, 1).max()) <= 2.0 ** -17
+
+
+@pytest.mark.parametrize("kind", ["flat", "decay", "spike", "ten", "pairs"])
+@pytest.mark.parametrize("L,D,sub,rank", [(128, 128, 0, 1), (128, 128, 0, 8), (128, 64, 0, 5), (128, 128, 85, 4)])
+def test_leading_directions_of_hard_spectra(L, D, sub, rank, kind):
+    """A flat spectrum, a steep one, one direction that outweighs all others, fewer directions than the solver iterates with, and
+    pairs of nearly equal eigenvalues: every factor an eigenvector to the rounding of its sums (the bound of the test above, twice
+    where the largest eigenvalue is a hundred times the next), none of the leading ones left out."""
+    from paper_2607_09052_b200 import binding as B
+    n = 48
+    wl = synth.Workload("hard", 2, 2, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
+                        key_model="iid", shuffle_pages=True, seed=11)
+    inp = synth.generate(wl, "cuda")
+    keys = inp["k_pages"].float()
+    j = torch.arange(D, device="cuda")
+    if kind == "decay":
+        keys *= 0.8 ** j
+    elif kind == "spike":
+        keys[..., 3] *= 10.0
+    elif kind == "ten":
+        keys *= j < 10
+    elif kind == "pairs":
+        keys *= 0.7 ** (j // 2)
+    inp["k_pages"] = keys.to(torch.bfloat16)
+    cfg = B.make_config(wl)
+    summ = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"))
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, B.make_kv(inp), 0, wl.max_blocks, summ, ws)
+    assert B.cobs_read_status(ws) == 0
+    _, xi, _ = B.summary_views(cfg, summ)
+    K = inp["k_pages"][inp["page_table"].long()].permute(0, 2, 1, 3, 4).reshape(2, 2, -1, L, D).double()
+    K = K - K.mean(3, keepdim=True)
+    if sub:
+        K = torch.einsum("bhnld,hds->bhnls", K, inp["u_q"].double())
+    sigma = K.transpose(-1, -2) @ K / L
+    lam = torch.linalg.eigvalsh(sigma).flip(-1)[..., :rank]
+    x = xi.double()
+    n2 = (x * x).sum(-1)
+    resid = (x @ sigma - n2[..., None] * x).norm(dim=-1) / (lam[..., :1] * n2.sqrt())
+    bound = (48 if kind == "spike" else 24) * 2.0 ** -24
+    assert float(resid.max()) <= bound, float(resid.max())
+    assert float(((n2 - lam).abs() / lam[..., :1]).max()) <= bound
