@@ -13,7 +13,7 @@
 // is the operand of the next without a shuffle.  G is symmetric, so its accumulators are the B operand in the same way.
 // Operands are split into f16 high and low parts (22 bits) and products are summed in fp32 (mma_split); the first round, which
 // only has to find the neighbourhood, takes the high parts alone.
-// Four warps (blocks of 128) hold every fourth tile each; V goes through shared memory for each product, one barrier.
+// Four warps (blocks of 128; blocks of 64 when there are few) hold every fourth tile each; V goes through shared memory for each product, one barrier.
 //
 // Measured at 128 tokens, three blocks per SM (cycles of one block; products with G, orthonormalisations): flat spectrum, rank 4:
 // 126 000 (20; 4), rank 8: 138 000 (25; 4), sixteen directions over noise, rank 8: 102 000 (10; 4), where the tridiagonal form took
@@ -28,9 +28,9 @@
 namespace cobs {
 namespace {
 
-template <int L>
+template <int L, int W_>
 struct Filter {
-  static constexpr int W = (L == 128) ? 4 : 1;        // warps per block
+  static constexpr int W = W_;                        // warps per block
   static constexpr int NT = L / 8 / W;                // 8-token tiles of a warp: tile a is tile W a + warp of the block
   static constexpr int KT = L / 16;                   // 16-token steps of a product
   // shared memory, in floats: G as B fragments (four warps: the low halves, the high ones stay in registers)
@@ -176,15 +176,15 @@ __device__ __forceinline__ void refine16(float (&u)[8], const float (&h)[8], con
   for (int i = 0; i < 8; ++i) u[i] = fmaf(t[i], 1.f / (4096.f * 256.f), u[i]);
 }
 
-// Writes w (unit vectors, token-major, [L][RP], zeros where a direction is null) to Wt and top[0..RP) (index or -1); true if the
-// block has to be left to the careful kernel.  A: the Gram matrix, rows 8 (W a + warp) + gid, columns 8 n + 2 tig + {0, 1}.
-// sm: Filter's G_FLOATS, free, and Wt may lie there; buf: V_FLOATS + X_FLOATS; ub: U_FLOATS.  null_at: eigenvalues up to it
+// w: unit vector gid at tokens 8 (W a + warp) + 2 tig + {0, 1}, zeros where a direction is null; top[0..RP): index or -1.  True if
+// the block has to be left to the careful kernel.  A: the Gram matrix, rows 8 (W a + warp) + gid, columns 8 n + 2 tig + {0, 1}.
+// sm: Filter's G_FLOATS, free; buf: V_FLOATS + X_FLOATS; ub: U_FLOATS.  null_at: eigenvalues up to it
 // count as none.
-template <int L, int RP>
-__device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], float *sm, float *buf, float *ub, float *Wt, int *top,
-                                             int r_eff, float null_at, int warp, int lane) {
-  using F = Filter<L>;
-  constexpr int W = F::W, NT = F::NT, KT = F::KT;
+template <int L, int RP, int W>
+__device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], float (&w)[Filter<L, W>::NT][2], float *sm, float *buf, float *ub,
+                                             int *top, int r_eff, float null_at, int warp, int lane) {
+  using F = Filter<L, W>;
+  constexpr int NT = F::NT, KT = F::KT;
   const int gid = lane >> 2, tig = lane & 3;
   auto sync = [&]() { if (W == 1) __syncwarp(); else __syncthreads(); };
   float *xbuf = buf + F::V_FLOATS;
@@ -248,21 +248,18 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
     }
   if (W == 1) __syncwarp();
 
-  // ---- start: fixed vectors of no structure (multiples of 1/4 below 4), for 16 tokens the unit vectors -------------------------------
+  // ---- start: fixed vectors of no structure (odd multiples of 1/8 below 4) ---------------------------------------------------------------
   float V[NT][4], Vp[NT][4], P[NT][4];
 #pragma unroll
   for (int a = 0; a < NT; ++a)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int vec = gid + 8 * (i >> 1), tok = 8 * (W * a + warp) + 2 * tig + (i & 1);
-      if (L == 16) V[a][i] = (vec == tok) ? 16.f : 0.f;
-      else {
-        uint32_t x = (uint32_t)(vec * 256 + tok + 1) * 0x9E3779B1u;
-        x ^= x >> 15;
-        x *= 0x85EBCA77u;
-        x ^= x >> 13;
-        V[a][i] = (float)(2 * (int)(x >> 27) - 31) * 0.125f;
-      }
+      uint32_t x = (uint32_t)(vec * 256 + tok + 1) * 0x9E3779B1u;
+      x ^= x >> 15;
+      x *= 0x85EBCA77u;
+      x ^= x >> 13;
+      V[a][i] = (float)(2 * (int)(x >> 27) - 31) * 0.125f;
       Vp[a][i] = 0.f;
     }
 
@@ -432,10 +429,10 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
   // this round, the small problem is solved.  What limits m: the leading direction's share of the other rows grows with it, and
   // takes their bits where it is left too large.
   constexpr float kCoarse = 4.f;                        // what vectors rounded to f16 can gain
-  constexpr float kTol = (L == 16) ? 1.2e-6f : 4e-7f, kTol1 = (L == 16) ? 3e-7f : 2e-7f;      // |G w - theta w| over theta, and over theta_1
+  constexpr float kTol = 4e-7f, kTol1 = 2e-7f;      // |G w - theta w| over theta, and over theta_1
   float b = mu + 0.6f * sqrtf(fmaxf(fro2 * (1.0f / (float)L) - mu * mu, 0.f));
-  float credit = 0.f, extra = 0.f, grown = 3.4f, parted = 1.f, s0 = 1.f, s1 = 1.f;      // (the first round lets vectors grow 30 times)
-  bool last = L == 16, failed = false;
+  float credit = 0.f, extra = 0.f, wider = 1.f, grown = 3.4f, parted = 1.f, s0 = 1.f, s1 = 1.f;      // (the first round lets vectors grow 30 times)
+  bool last = false, failed = false;
   int m = 5, k = 0, round = 0;
 #pragma unroll 1
   for (;;) {
@@ -447,7 +444,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
       f1 = __fdividef(4.0f, b); f2 = -2.0f; f3 = -1.0f;
     } else {
       f2 = -1.0f; f3 = 0.f;
-      if (round > 0 || L == 16) {
+      if (round > 0) {
         // Rayleigh quotients: the largest, the smallest, and the smallest of the first r rows but for rounding noise (the rows come
         // about in the order of their quotients)
         float d[4];
@@ -456,9 +453,11 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
         xsum(d);
         d[0] = __fdividef(d[0], fmaxf(d[2], 1e-20f)); d[1] = __fdividef(d[1], fmaxf(d[3], 1e-20f));
         const float d_max = rows_max(fmaxf(d[0], d[1])), noise = 2e-6f * d_max;
-        const float d_min = -rows_max(-fminf((d[2] > 0.f) ? d[0] : d_max, (d[3] > 0.f) ? d[1] : d_max));
+        const int live = (__popc(__ballot_sync(0xffffffffu, d[2] > 0.f)) + __popc(__ballot_sync(0xffffffffu, d[3] > 0.f))) >> 2;
+        const float least_live = -rows_max(-fminf((d[2] > 0.f) ? d[0] : d_max, (d[3] > 0.f) ? d[1] : d_max));
+        const float d_min = (live > r_eff + 3) ? least_live : 0.f;      // (rows left out of a solution are zero)
         const float d_r = fminf(1.f / rows_max((gid < r_eff && d[0] > noise) ? 1.f / d[0] : 0.f), d_max);
-        if (L > 16 && round == 1) credit = fminf(fmaxf(fmaf(-(float)m, __logf(cheb_damp(__fdividef(2.0f * d_r, b) - 1.0f)), -0.7f), 0.f), kCoarse);
+        if (round == 1) credit = fminf(fmaxf(fmaf(-(float)m, __logf(cheb_damp(__fdividef(2.0f * d_r, b) - 1.0f)), -0.7f), 0.f), kCoarse);
         if (last) {
           // ---- H = V G V^T, its eigenvectors -----------------------------------------------------------------------------------
           float s[8], g[8];
@@ -500,22 +499,17 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
 #pragma unroll 1
             for (int pass = 0; pass < 3; ++pass) refine16(u, s, g, lane);
             split16(u, 256.f, uh, ul);
-            uh[1] = uh[3] = ul[1] = ul[3] = 0u;         // eight vectors
           }
-          float X[NT][4];
-#pragma unroll
-          for (int a = 0; a < NT; ++a)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { X[a][i] = V[a][i]; Vp[a][i] = P[a][i]; }
-          rotate(uh, ul, X, 1.f, 1.f);
-          rotate(uh, ul, Vp, 1.f / 64.f, 1.f / 64.f);
+          // the basis turned into the eigenvectors' (times 256)
+          rotate(uh, ul, V, 1.f, 1.f);
+          rotate(uh, ul, P, 1.f / 64.f, 1.f / 64.f);
           float q[2];                                   // x . x, x . G x / 64
           {
             u64 t0 = 0ull, t1 = 0ull;
 #pragma unroll
             for (int a = 0; a < NT; ++a) {
-              t0 = fma2(pk(X[a][0], X[a][1]), pk(X[a][0], X[a][1]), t0);
-              t1 = fma2(pk(X[a][0], X[a][1]), pk(Vp[a][0], Vp[a][1]), t1);
+              t0 = fma2(pk(V[a][0], V[a][1]), pk(V[a][0], V[a][1]), t0);
+              t1 = fma2(pk(V[a][0], V[a][1]), pk(P[a][0], P[a][1]), t1);
             }
             q[0] = quad_sum(lo(t0) + hi(t0)); q[1] = quad_sum(lo(t1) + hi(t1));
             xsum(q);
@@ -524,7 +518,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
           float e2[1] = {0.f};
 #pragma unroll
           for (int a = 0; a < NT; ++a) {
-            const float e0 = fmaf(-th, X[a][0], Vp[a][0]), e1 = fmaf(-th, X[a][1], Vp[a][1]);
+            const float e0 = fmaf(-th, V[a][0], P[a][0]), e1 = fmaf(-th, V[a][1], P[a][1]);
             e2[0] = fmaf(e0, e0, fmaf(e1, e1, e2[0]));
           }
           e2[0] = quad_sum(e2[0]);
@@ -534,26 +528,34 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
           // null rule: a direction below 1e-12 of the mean squared key norm is stored as zeros
           const bool keep = gid < r_eff && th * 64.f > null_at * gs;
           const bool sane = th1 > 0.f && th1 < 1e30f;
-          const bool ok = sane && __all_sync(0xffffffffu, !keep || err <= fmaf(kTol, th, kTol1 * th1));
+          // (a direction of rounding noise is one as well as another)
+          const float allowed = wider * ((th > 1e-6f * th1) ? fmaf(kTol, th, kTol1 * th1) : 1e-6f * th1);
+          const bool ok = sane && __all_sync(0xffffffffu, !keep || err <= allowed);
           // Two equal eigenvalues: any basis of their plane is right, and the careful kernel has the say.
           const bool equal = keep && gid + 1 < r_eff && thn > 2.4e-7f * th1 && th - thn <= 9.6e-7f * th;
           ++round;
-          if (ok || !sane || L == 16 || round > 20) {
+          if (ok || !sane || round > 20) {
             failed = !ok || __any_sync(0xffffffffu, equal);
             const float wn = keep ? xn : 0.f;
 #pragma unroll
-            for (int a = 0; a < NT; ++a) { Vp[a][0] = X[a][0] * wn; Vp[a][1] = X[a][1] * wn; }
+            for (int a = 0; a < NT; ++a) { w[a][0] = V[a][0] * wn; w[a][1] = V[a][1] * wn; }
             if (warp == 0 && tig == 0 && gid < RP) top[gid] = keep ? gid : -1;
             break;
           }
-          const float w = warp_max(keep ? __fdividef(err, fmaf(kTol, th, kTol1 * th1)) : 0.f);
-          extra = fminf(extra + __logf(fminf(fmaxf(w, 1.f), 1e6f)) + 1.0f, 30.f);
+          const float far = warp_max(keep ? __fdividef(err, allowed) : 0.f);
+          extra = fminf(extra + __logf(fminf(fmaxf(far, 1.f), 1e6f)) + 1.0f, 30.f);
+          wider = fminf(1.5f * wider, 4.f);             // (what the rounding of the products leaves may be just above)
           last = false;
+#pragma unroll
+          for (int a = 0; a < NT; ++a)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) V[a][i] *= 1.f / 256.f;
+          continue;
         }
         b = fmaxf(fmaxf(d_min, 0.02f * d_r), 1e-5f * d_max);      // (lower, and the leading rows drown the others)
         const float ib = __fdividef(2.0f, b);
         const float xr = -__logf(cheb_damp(fmaf(d_r, ib, -1.0f))), x1 = fmaxf(-__logf(cheb_damp(fmaf(d_max, ib, -1.0f))), 0.5f);
-        const float need = __logf(1.0f / kTol) + 6.0f + extra;
+        const float need = __logf(1.0f / kTol) + 6.0f + 0.5f * __logf(__fdividef(d_max, d_r)) + extra;
         // The other rows' share of the leading direction is what the rounds so far have left: it may grow to some fifty times the
         // rows themselves, and in the rows that are wanted to no more than a few times.
         const float cap = fminf(__fdividef(fminf(grown + 4.f, 15.f), x1), __fdividef(parted + 1.5f, fmaxf(x1 - xr, 0.1f)));
@@ -595,12 +597,6 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
     }
   }
   sync();                                               // G and the sums have been read by all warps
-  if (gid < RP) {
-#pragma unroll
-    for (int a = 0; a < NT; ++a)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) Wt[(8 * (W * a + warp) + 2 * tig + i) * RP + gid] = Vp[a][i];
-  }
   return failed;
 }
 

@@ -108,13 +108,15 @@ def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
 
 
 @pytest.mark.parametrize("kind", ["flat", "decay", "spike", "ten", "pairs"])
-@pytest.mark.parametrize("L,D,sub,rank", [(128, 128, 0, 1), (128, 128, 0, 8), (128, 64, 0, 5), (128, 128, 85, 4)])
-def test_leading_directions_of_hard_spectra(L, D, sub, rank, kind):
+@pytest.mark.parametrize("L,D,sub,rank,n", [(128, 128, 0, 1, 48), (128, 128, 0, 8, 48), (128, 64, 0, 5, 48), (128, 128, 85, 4, 48),
+                                            (64, 128, 0, 8, 48), (64, 64, 24, 4, 48), (64, 128, 0, 5, 160), (64, 128, 0, 8, 301),
+                                            (64, 64, 0, 1, 443), (64, 128, 85, 4, 301)])
+def test_leading_directions_of_hard_spectra(L, D, sub, rank, n, kind):
     """A flat spectrum, a steep one, one direction that outweighs all others, fewer directions than the solver iterates with, and
     pairs of nearly equal eigenvalues: every factor an eigenvector to the rounding of its sums (the bound of the test above, twice
-    where the largest eigenvalue is a hundred times the next), none of the leading ones left out."""
+    where the largest eigenvalue is a hundred times the next), none of the leading ones left out.  4 n blocks: few, more, and
+    so many that each warp takes one, the last CTA not full."""
     from paper_2607_09052_b200 import binding as B
-    n = 48
     wl = synth.Workload("hard", 2, 2, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
                         key_model="iid", shuffle_pages=True, seed=11)
     inp = synth.generate(wl, "cuda")
