@@ -13,7 +13,7 @@
 // is the operand of the next without a shuffle.  G is symmetric, so its accumulators are the B operand in the same way.
 // Operands are split into f16 high and low parts (22 bits) and products are summed in fp32 (mma_split); the first round, which
 // only has to find the neighbourhood, takes the high parts alone.
-// Four warps (blocks of 128; blocks of 64 when there are few) hold every fourth tile each; V goes through shared memory for each product, one barrier.
+// Four warps hold every fourth tile each; V goes through shared memory for each product, one barrier.
 //
 // Measured at 128 tokens, three blocks per SM (cycles of one block; products with G, orthonormalisations): flat spectrum, rank 4:
 // 126 000 (20; 4), rank 8: 138 000 (25; 4), sixteen directions over noise, rank 8: 102 000 (10; 4), where the tridiagonal form took
@@ -28,15 +28,15 @@
 namespace cobs {
 namespace {
 
-template <int L, int W_>
+template <int L>
 struct Filter {
-  static constexpr int W = W_;                        // warps per block
+  static constexpr int W = 4;                         // warps per block
   static constexpr int NT = L / 8 / W;                // 8-token tiles of a warp: tile a is tile W a + warp of the block
   static constexpr int KT = L / 16;                   // 16-token steps of a product
-  // shared memory, in floats: G as B fragments (four warps: the low halves, the high ones stay in registers)
-  static constexpr int G_FLOATS = (W == 1) ? L * L : L * L / 2;
-  static constexpr int V_FLOATS = (W == 1) ? 0 : 2 * KT * 2 * 128;      // two buffers of V as A fragments
-  static constexpr int X_FLOATS = (W == 1) ? 0 : 2 * W * 32 * 8;        // two buffers of the warps' partial sums
+  // shared memory, in floats: the low halves of G as B fragments (the high ones stay in registers)
+  static constexpr int G_FLOATS = L * L / 2;
+  static constexpr int V_FLOATS = 2 * KT * 2 * 128;   // two buffers of V as A fragments
+  static constexpr int X_FLOATS = 2 * W * 32 * 8;     // two buffers of the warps' partial sums
   static constexpr int U_FLOATS = 256;
 };
 
@@ -180,27 +180,24 @@ __device__ __forceinline__ void refine16(float (&u)[8], const float (&h)[8], con
 // the block has to be left to the careful kernel.  A: the Gram matrix, rows 8 (W a + warp) + gid, columns 8 n + 2 tig + {0, 1}.
 // sm: Filter's G_FLOATS, free; buf: V_FLOATS + X_FLOATS; ub: U_FLOATS.  null_at: eigenvalues up to it
 // count as none.
-template <int L, int RP, int W>
-__device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], float (&w)[Filter<L, W>::NT][2], float *sm, float *buf, float *ub,
+template <int L, int RP>
+__device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], float (&w)[Filter<L>::NT][2], float *sm, float *buf, float *ub,
                                              int *top, int r_eff, float null_at, int warp, int lane) {
-  using F = Filter<L, W>;
-  constexpr int NT = F::NT, KT = F::KT;
+  using F = Filter<L>;
+  constexpr int W = F::W, NT = F::NT, KT = F::KT;
   const int gid = lane >> 2, tig = lane & 3;
-  auto sync = [&]() { if (W == 1) __syncwarp(); else __syncthreads(); };
   float *xbuf = buf + F::V_FLOATS;
   int xpar = 0, vpar = 0;
   // sums over the block's warps; two buffers, so that one barrier per call is enough
   auto xsum = [&](auto &v) {
-    if constexpr (W > 1) {
-      constexpr int N = sizeof(v) / sizeof(float);
-      float *b = xbuf + xpar * W * 256;
-      xpar ^= 1;
+    constexpr int N = sizeof(v) / sizeof(float);
+    float *b = xbuf + xpar * W * 256;
+    xpar ^= 1;
 #pragma unroll
-      for (int i = 0; i < N; ++i) b[warp * 256 + 32 * i + lane] = v[i];
-      __syncthreads();
+    for (int i = 0; i < N; ++i) b[warp * 256 + 32 * i + lane] = v[i];
+    __syncthreads();
 #pragma unroll
-      for (int i = 0; i < N; ++i) v[i] = (b[32 * i + lane] + b[256 + 32 * i + lane]) + (b[512 + 32 * i + lane] + b[768 + 32 * i + lane]);
-    }
+    for (int i = 0; i < N; ++i) v[i] = (b[32 * i + lane] + b[256 + 32 * i + lane]) + (b[512 + 32 * i + lane] + b[768 + 32 * i + lane]);
   };
 
   // ---- scale: the trace to [2^12, 2^13), so that elements and eigenvalues fit f16 with their low parts ---------------------------
@@ -211,7 +208,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
     for (int a = 0; a < NT; ++a)
 #pragma unroll
       for (int w = 0; w < W; ++w)
-        if ((W == 1 || warp == w) && tig == gid >> 1) t[0] += (gid & 1) ? hi(A[a][W * a + w]) : lo(A[a][W * a + w]);
+        if (warp == w && tig == gid >> 1) t[0] += (gid & 1) ? hi(A[a][W * a + w]) : lo(A[a][W * a + w]);
     t[0] = warp_sum(t[0]);
     xsum(t);
     const float tr = t[0];
@@ -233,20 +230,17 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
     fro2 = f[0];
   }
   // ---- G as B fragments -----------------------------------------------------------------------------------------------------------
-  uint2 gh[(W == 1) ? 1 : NT][(W == 1) ? 1 : KT];       // four warps: the high halves
-  uint4 *gb = reinterpret_cast<uint4 *>(sm) + lane;
+  uint2 gh[NT][KT];                                     // the high halves
   uint2 *gl = reinterpret_cast<uint2 *>(sm) + warp * (NT * KT * 32) + lane;
 #pragma unroll
   for (int kt = 0; kt < KT; ++kt)
 #pragma unroll
     for (int a = 0; a < NT; ++a) {
-      uint4 f;
-      split_f16(lo(A[a][2 * kt]), hi(A[a][2 * kt]), f.x, f.z);
-      split_f16(lo(A[a][2 * kt + 1]), hi(A[a][2 * kt + 1]), f.y, f.w);
-      if constexpr (W == 1) gb[(kt * NT + a) * 32] = f;
-      else { gh[a][kt] = make_uint2(f.x, f.y); gl[(kt * NT + a) * 32] = make_uint2(f.z, f.w); }
+      uint2 l;
+      split_f16(lo(A[a][2 * kt]), hi(A[a][2 * kt]), gh[a][kt].x, l.x);
+      split_f16(lo(A[a][2 * kt + 1]), hi(A[a][2 * kt + 1]), gh[a][kt].y, l.y);
+      gl[(kt * NT + a) * 32] = l;
     }
-  if (W == 1) __syncwarp();
 
   // ---- start: fixed vectors of no structure (odd multiples of 1/8 below 4) ---------------------------------------------------------------
   float V[NT][4], Vp[NT][4], P[NT][4];
@@ -281,44 +275,31 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
       else if constexpr (MODE == 1) mma_chain(c, h, l, bh0, bh1, bl0, bl1);
       else mma_f16(c, h[0], h[1], h[2], h[3], bh0, bh1);
     };
-    if constexpr (W == 1) {
+    // tile g of the block is half (g & 1) of step g / 2
+    unsigned char *vb = reinterpret_cast<unsigned char *>(buf + vpar * KT * 256);
+    vpar ^= 1;
 #pragma unroll
-      for (int kt = 0; kt < KT; ++kt) {
-        uint32_t h[4], l[4];
-        split_pair(V, 2 * kt, 1.f, 1.f, h, l);
+    for (int a = 0; a < NT; ++a) {
+      const int g = W * a + warp;
+      uint2 h, l;
+      split_f16(V[a][0], V[a][1], h.x, l.x);
+      split_f16(V[a][2], V[a][3], h.y, l.y);
+      unsigned char *d = vb + ((g >> 1) * 64 + lane) * 16 + (g & 1) * 8;
+      *reinterpret_cast<uint2 *>(d) = h;
+      if (FULL) *reinterpret_cast<uint2 *>(d + 512) = l;
+    }
+    __syncthreads();
 #pragma unroll
-        for (int a = 0; a < NT; ++a) {
-          const uint4 b = gb[(kt * NT + a) * 32];
-          step(P[a], h, l, b.x, b.y, b.z, b.w);
-        }
-      }
-    } else {
-      // tile g of the block is half (g & 1) of step g / 2
-      unsigned char *vb = reinterpret_cast<unsigned char *>(buf + vpar * KT * 256);
-      vpar ^= 1;
+    for (int kt = 0; kt < KT; ++kt) {
+      const uint4 vh = *reinterpret_cast<const uint4 *>(vb + (kt * 64 + lane) * 16);
+      uint4 vl = make_uint4(0u, 0u, 0u, 0u);
+      if (FULL) vl = *reinterpret_cast<const uint4 *>(vb + (kt * 64 + 32 + lane) * 16);
+      const uint32_t h[4] = {vh.x, vh.y, vh.z, vh.w}, l[4] = {vl.x, vl.y, vl.z, vl.w};
 #pragma unroll
       for (int a = 0; a < NT; ++a) {
-        const int g = W * a + warp;
-        uint2 h, l;
-        split_f16(V[a][0], V[a][1], h.x, l.x);
-        split_f16(V[a][2], V[a][3], h.y, l.y);
-        unsigned char *d = vb + ((g >> 1) * 64 + lane) * 16 + (g & 1) * 8;
-        *reinterpret_cast<uint2 *>(d) = h;
-        if (FULL) *reinterpret_cast<uint2 *>(d + 512) = l;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kt = 0; kt < KT; ++kt) {
-        const uint4 vh = *reinterpret_cast<const uint4 *>(vb + (kt * 64 + lane) * 16);
-        uint4 vl = make_uint4(0u, 0u, 0u, 0u);
-        if (FULL) vl = *reinterpret_cast<const uint4 *>(vb + (kt * 64 + 32 + lane) * 16);
-        const uint32_t h[4] = {vh.x, vh.y, vh.z, vh.w}, l[4] = {vl.x, vl.y, vl.z, vl.w};
-#pragma unroll
-        for (int a = 0; a < NT; ++a) {
-          uint2 bl = make_uint2(0u, 0u);
-          if (FULL) bl = gl[(kt * NT + a) * 32];
-          step(P[a], h, l, gh[a][kt].x, gh[a][kt].y, bl.x, bl.y);
-        }
+        uint2 bl = make_uint2(0u, 0u);
+        if (FULL) bl = gl[(kt * NT + a) * 32];
+        step(P[a], h, l, gh[a][kt].x, gh[a][kt].y, bl.x, bl.y);
       }
     }
   };
@@ -463,7 +444,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
           float s[8], g[8];
           gram16(V, P, 1.f, 1.f, 1.f / 64.f, 1.f / 64.f, s);
           gram16(V, V, 1.f, 1.f, 1.f, 1.f, g);
-          if (W == 1 || warp == 0) {
+          if (warp == 0) {
             u64 x[2] = {pk(s[0], s[1]), pk(s[2], s[3])}, y[2] = {pk(s[4], s[5]), pk(s[6], s[7])};
             const float thr = 8.f * d_r * d_r;          // (the squared norm of the r-th row is 16 d_r^2)
             const float null2 = 16.f * 5.8e-14f * d_max * d_max;      // 2^-22 of the largest is the error of any eigenvalue: none, then
@@ -490,7 +471,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
             o[q0 * 8] = mul2(x[0], v0); o[q0 * 8 + 4] = mul2(x[1], v0);
             o[q1 * 8] = mul2(y[0], v1); o[q1 * 8 + 4] = mul2(y[1], v1);
           }
-          sync();
+          __syncthreads();
           uint32_t uh[4], ul[4];
           {
             const u64 *o = reinterpret_cast<const u64 *>(ub) + gid * 8 + tig;
@@ -596,7 +577,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L, W>::NT][L / 8], 
       }
     }
   }
-  sync();                                               // G and the sums have been read by all warps
+  __syncthreads();                                      // G and the sums have been read by all warps
   return failed;
 }
 

@@ -114,8 +114,8 @@ def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
 def test_leading_directions_of_hard_spectra(L, D, sub, rank, n, kind):
     """A flat spectrum, a steep one, one direction that outweighs all others, fewer directions than the solver iterates with, and
     pairs of nearly equal eigenvalues: every factor an eigenvector to the rounding of its sums (the bound of the test above, twice
-    where the largest eigenvalue is a hundred times the next), none of the leading ones left out.  4 n blocks: few, more, and
-    so many that each warp takes one, the last CTA not full."""
+    where the largest eigenvalue is a hundred times the next), none of the leading ones left out.  4 n blocks: fewer than
+    are resident at a time, and more."""
     from paper_2607_09052_b200 import binding as B
     wl = synth.Workload("hard", 2, 2, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
                         key_model="iid", shuffle_pages=True, seed=11)
@@ -149,3 +149,28 @@ def test_leading_directions_of_hard_spectra(L, D, sub, rank, n, kind):
     bound = (48 if kind == "spike" else 24) * 2.0 ** -24
     assert float(resid.max()) <= bound, float(resid.max())
     assert float(((n2 - lam).abs() / lam[..., :1]).max()) <= bound
+
+
+@pytest.mark.parametrize("L,D,sub,rank,n,dtype", [(64, 128, 0, 8, 300, "fp32"), (64, 128, 0, 4, 230, "fp4"), (64, 64, 24, 4, 300, "fp32"), (64, 64, 0, 12, 40, "fp32"),
+                                                  (128, 128, 0, 8, 150, "fp32"), (128, 64, 0, 4, 130, "fp4"), (128, 128, 85, 4, 120, "fp32"),
+                                                  (32, 64, 0, 4, 300, "fp32"), (16, 64, 0, 4, 300, "bf16")])
+def test_a_block_has_the_same_bits_in_every_call(L, D, sub, rank, n, dtype):
+    """All 8 n blocks in one call, and again in calls of one block of every sequence and KV head, of a few, and of half of them: a
+    block's summary is a function of its keys.  (A decode loop builds the blocks of all sequences again whenever one fills.)"""
+    from paper_2607_09052_b200 import binding as B
+    wl = synth.Workload("bits", 2, 4, 4, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype=dtype, sub_dim=sub,
+                        key_model="iid", shuffle_pages=True, seed=17)
+    inp = synth.generate(wl, "cuda")
+    inp["k_pages"][::3, ..., 7] *= 20.0                   # some blocks with a channel that outweighs the others
+    cfg = B.make_config(wl)
+    ws = B.alloc_workspace(cfg, "cuda")
+    whole, parts = B.SummaryBuffers(cfg, "cuda", inp.get("u_q")), B.SummaryBuffers(cfg, "cuda", inp.get("u_q"))
+    kv = B.make_kv(inp)
+    B.cobs_build_summaries(cfg, kv, 0, n, whole, ws)
+    cuts = sorted({0, 1, 2, 5, 12, 25, n // 2, n})
+    for first, last in zip(cuts, cuts[1:]):
+        B.cobs_build_summaries(cfg, kv, first, last, parts, ws)
+    assert B.cobs_read_status(ws) == 0
+    for one, other in zip(B.summary_views(cfg, whole), B.summary_views(cfg, parts)):
+        if one is not None:
+            assert torch.equal(one.contiguous().view(torch.uint8), other.contiguous().view(torch.uint8))
