@@ -78,10 +78,23 @@ __device__ __forceinline__ void from_tiles(const float (&c)[2][4], float (&o)[8]
   o[0] = c[0][0]; o[1] = c[0][1]; o[2] = c[1][0]; o[3] = c[1][1];
   o[4] = c[0][2]; o[5] = c[0][3]; o[6] = c[1][2]; o[7] = c[1][3];
 }
-__device__ __forceinline__ void mul16_bt(const uint32_t (&ah)[4], const uint32_t (&al)[4], const uint32_t (&bh)[4], const uint32_t (&bl)[4], float (&o)[8]) {      // A B^T
+// A B^T; SYM: to the bit the transpose of B A^T (the mixed products are added before the high ones)
+template <bool SYM>
+__device__ __forceinline__ void mul16_bt(const uint32_t (&ah)[4], const uint32_t (&al)[4], const uint32_t (&bh)[4], const uint32_t (&bl)[4], float (&o)[8]) {
   float c[2][4];
-  mma_split<true>(c[0], ah, al, bh[0], bh[2], bl[0], bl[2]);
-  mma_split<true>(c[1], ah, al, bh[1], bh[3], bl[1], bl[3]);
+#pragma unroll
+  for (int n = 0; n < 2; ++n) {
+    if constexpr (!SYM) {
+      mma_split<true>(c[n], ah, al, bh[n], bh[2 + n], bl[n], bl[2 + n]);
+      continue;
+    }
+    float t[4];
+    mma_f16_zero(c[n], ah[0], ah[1], ah[2], ah[3], bl[n], bl[2 + n]);
+    mma_f16_zero(t, al[0], al[1], al[2], al[3], bh[n], bh[2 + n]);
+    add4(c[n], t);
+    mma_f16_zero(t, ah[0], ah[1], ah[2], ah[3], bh[n], bh[2 + n]);
+    add4(c[n], t);
+  }
   from_tiles(c, o);
 }
 __device__ __forceinline__ void diag16(const float (&s)[8], int lane, float &d0, float &d1) {      // elements gid and gid + 8
@@ -137,18 +150,20 @@ __device__ __forceinline__ bool jacobi_sweep(u64 (&x)[2], u64 (&y)[2], float thr
 // Rows u, nearly the eigenvectors of the pair (h, g): h u = lambda g u, g nearly 1, to the rounding of the products (T. Ogita,
 // K. Aishima, "Iterative refinement for symmetric eigenvalue decomposition", 2018): u_j += sum_i e_ij u_i with
 // e_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i), r = 1 - u g u^T, s = u h u^T; for close pairs, and on the diagonal,
-// r_ij / 2.  Both are made symmetric, since e_ij + e_ji has to be r_ij however close the pair.  (The rotations alone leave the
-// rounding of some fifty steps, 5e-7 of the largest eigenvalue.)  g: times 256.
-__device__ __forceinline__ void refine16(float (&u)[8], const float (&h)[8], const float (&g)[8], int lane) {
+// r_ij / 2.  Both are made symmetric, to the bit, and so is what decides between the two: e_ij + e_ji has to be r_ij however close
+// the pair (or the factors of four nearly equal eigenvalues come out 1e-4 off the right angle).  (The rotations alone leave the
+// rounding of some fifty steps, 5e-7 of the largest eigenvalue.)  g: times 256.  Returns the largest |e_ij| of the first n rows:
+// what is left after the pass is its square.
+__device__ __forceinline__ float refine16(float (&u)[8], const float (&h)[8], const float (&g)[8], int n, int lane) {
   const int gid = lane >> 2, tig = lane & 3;
   uint32_t uh[4], ul[4], th[4], tl[4];
   float t[8], s[8], r[8];
   auto form = [&](const float (&x)[8], float (&o)[8]) {      // 256 u x u^T, twice
     split16(x, 1.f, th, tl);
-    mul16_bt(uh, ul, th, tl, t);                        // 256 u x
+    mul16_bt<false>(uh, ul, th, tl, t);                 // 256 u x
     split16(t, 1.f / 256.f, th, tl);
-    mul16_bt(th, tl, uh, ul, o);
-    mul16_bt(uh, ul, th, tl, t);
+    mul16_bt<true>(th, tl, uh, ul, o);
+    mul16_bt<true>(uh, ul, th, tl, t);
 #pragma unroll
     for (int i = 0; i < 8; ++i) o[i] += t[i];
   };
@@ -157,13 +172,20 @@ __device__ __forceinline__ void refine16(float (&u)[8], const float (&h)[8], con
   form(g, r);
   float l0, l1;
   diag16(s, lane, l0, l1);
+  const float lmax = __shfl_sync(0xffffffffu, l0, 0);
+  float most = 0.f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int row = gid + 8 * (i >> 2), col = 8 * ((i >> 1) & 1) + 2 * tig + (i & 1);
     const float lc = __shfl_sync(0xffffffffu, ((i >> 1) & 1) ? l1 : l0, 4 * (2 * tig + (i & 1))), lr = (i >> 2) ? l1 : l0;
     const float ri = fmaf(r[i], -1.f / 131072.f, (row == col) ? 1.f : 0.f);
-    const float num = fmaf(lr, ri, s[i]), gap = lr - lc;
-    t[i] = (row == col || !(fabsf(num) < 0.25f * fabsf(gap))) ? 0.5f * ri : __fdividef(num, gap);
+    // e_ij = r_ij / 2 + f_ij, f_ij = -f_ji; a numerator of rounding noise does not tell two close directions apart
+    const float num = fmaf(0.5f * (lr + lc), ri, s[i]), gap = lr - lc, an = fabsf(num), ag = fabsf(gap);
+    const bool turn = row != col && an < 0.25f * ag && (an > 2.5e-7f * lmax || an < 1e-4f * ag);
+    t[i] = 0.5f * ri + (turn ? __fdividef(num, gap) : 0.f);
+    // (rows of rounding noise may be nearly parallel: in full steps they grow without bound)
+    if (row != col && row >= n && col >= n) t[i] = fminf(fmaxf(t[i], -0.12f), 0.12f);
+    if (row != col && row < n) most = fmaxf(most, fabsf(t[i]));
   }
   split16(t, 4096.f, th, tl);
 #pragma unroll
@@ -174,10 +196,11 @@ __device__ __forceinline__ void refine16(float (&u)[8], const float (&h)[8], con
   from_tiles(c, t);
 #pragma unroll
   for (int i = 0; i < 8; ++i) u[i] = fmaf(t[i], 1.f / (4096.f * 256.f), u[i]);
+  return warp_max(most);
 }
 
 // w: unit vector gid at tokens 8 (W a + warp) + 2 tig + {0, 1}, zeros where a direction is null; top[0..RP): index or -1.  True if
-// the block has to be left to the careful kernel.  A: the Gram matrix, rows 8 (W a + warp) + gid, columns 8 n + 2 tig + {0, 1}.
+// the block has to be left to the tridiagonal form.  A: the Gram matrix, rows 8 (W a + warp) + gid, columns 8 n + 2 tig + {0, 1}.
 // sm: Filter's G_FLOATS, free; buf: V_FLOATS + X_FLOATS; ub: U_FLOATS.  null_at: eigenvalues up to it
 // count as none.
 template <int L, int RP>
@@ -212,7 +235,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
     t[0] = warp_sum(t[0]);
     xsum(t);
     const float tr = t[0];
-    if (!(tr < 1e30f) || !(tr > 0.f)) return true;      // (uniform) infinite or not a number: for the careful kernel
+    if (!(tr < 1e30f) || !(tr > 0.f)) return true;      // (uniform) infinite or not a number
     gs = pow2(min(max(12 - ilog2(tr), -120), 120));
     mu = tr * gs * (1.0f / (float)L);
     const u64 g2 = pk(gs, gs);
@@ -412,9 +435,9 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
   constexpr float kCoarse = 4.f;                        // what vectors rounded to f16 can gain
   constexpr float kTol = 4e-7f, kTol1 = 2e-7f;      // |G w - theta w| over theta, and over theta_1
   float b = mu + 0.6f * sqrtf(fmaxf(fro2 * (1.0f / (float)L) - mu * mu, 0.f));
-  float credit = 0.f, extra = 0.f, wider = 1.f, grown = 3.4f, parted = 1.f, s0 = 1.f, s1 = 1.f;      // (the first round lets vectors grow 30 times)
+  float credit = 0.f, extra = 0.f, grown = 3.4f, parted = 1.f, s0 = 1.f, s1 = 1.f;      // (the first round lets vectors grow 30 times)
   bool last = false, failed = false;
-  int m = 5, k = 0, round = 0;
+  int m = 5, k = 0, round = 0, solves = 0;
 #pragma unroll 1
   for (;;) {
     if (last && k == 0) product(std::integral_constant<int, 2>{});
@@ -473,12 +496,15 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
           }
           __syncthreads();
           uint32_t uh[4], ul[4];
+          bool settled;                                 // (else the vectors need not be orthogonal to their rounding)
           {
             const u64 *o = reinterpret_cast<const u64 *>(ub) + gid * 8 + tig;
             const u64 t0 = o[0], t1 = o[4], t2 = o[64], t3 = o[68];
             float u[8] = {lo(t0), hi(t0), lo(t1), hi(t1), lo(t2), hi(t2), lo(t3), hi(t3)};
+            float e = 1.f;
 #pragma unroll 1
-            for (int pass = 0; pass < 3; ++pass) refine16(u, s, g, lane);
+            for (int pass = 0; pass < 6 && e > 5e-5f; ++pass) e = refine16(u, s, g, r_eff, lane);
+            settled = e < 3e-4f;
             split16(u, 256.f, uh, ul);
           }
           // the basis turned into the eigenvectors' (times 256)
@@ -510,13 +536,19 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
           const bool keep = gid < r_eff && th * 64.f > null_at * gs;
           const bool sane = th1 > 0.f && th1 < 1e30f;
           // (a direction of rounding noise is one as well as another)
-          const float allowed = wider * ((th > 1e-6f * th1) ? fmaf(kTol, th, kTol1 * th1) : 1e-6f * th1);
-          const bool ok = sane && __all_sync(0xffffffffu, !keep || err <= allowed);
+          const float allowed = (th > 1e-6f * th1) ? fmaf(kTol, th, kTol1 * th1) : 1e-6f * th1;
+          const bool ok = sane && settled && __all_sync(0xffffffffu, !keep || err <= allowed);
+          // A direction that is left out, or a faint one, stands for what the block has only if the others make up the trace, to its own
+          // rounding or to what may follow after the r-th: rows end below the pivot, or come out as another pair's, because rounding
+          // noise along the leading direction grows with it (one channel of deviation 100, rank 8: an eigenvalue 7e-6 of the largest missed).
+          const float rest = mu * (float)L / 64.f - 0.25f * warp_sum((gid < r_eff) ? fmaxf(th, 0.f) : 0.f);
+          const float least = -rows_max((gid < r_eff) ? -th : -th1), after = (least > 3e-4f * th1) ? 2.f * least : 0.f;
+          const bool lost = !(least > 1.5e-3f * th1) && !(rest <= fmaf(2e-7f, th1, 1.5e-7f / 64.f * (mu * (float)L)) + after);
           // Two equal eigenvalues: any basis of their plane is right, and the careful kernel has the say.
-          const bool equal = keep && gid + 1 < r_eff && thn > 2.4e-7f * th1 && th - thn <= 9.6e-7f * th;
+          const bool equal = keep && gid + 1 < r_eff && thn > 2.4e-7f * th1 && th - thn <= 2.4e-7f * th;
           ++round;
-          if (ok || !sane || round > 20) {
-            failed = !ok || __any_sync(0xffffffffu, equal);
+          if (ok || lost || !sane || round > 20 || ++solves == 3) {
+            failed = !ok || lost || __any_sync(0xffffffffu, equal);
             const float wn = keep ? xn : 0.f;
 #pragma unroll
             for (int a = 0; a < NT; ++a) { w[a][0] = V[a][0] * wn; w[a][1] = V[a][1] * wn; }
@@ -524,8 +556,7 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
             break;
           }
           const float far = warp_max(keep ? __fdividef(err, allowed) : 0.f);
-          extra = fminf(extra + __logf(fminf(fmaxf(far, 1.f), 1e6f)) + 1.0f, 30.f);
-          wider = fminf(1.5f * wider, 4.f);             // (what the rounding of the products leaves may be just above)
+          extra = fminf(extra + 1.5f * __logf(fminf(fmaxf(far, 1.f), 1e6f)) + 3.0f, 40.f);
           last = false;
 #pragma unroll
           for (int a = 0; a < NT; ++a)

@@ -69,7 +69,7 @@ def degenerate_keys(kind, n, L, D, gen):
 def test_blocks_of_fewer_directions_than_factors(L, D, sub, rank, n, kind):
     """Every block of the call degenerate, fewer of them than the careful kernel's CTAs have threads and more: the rank-r matrix
     within the errors of an eigenvalue, zeros where there is no direction.  Blocks with two equal eigenvalues are those that
-    the one-warp kernel declines: it has marked them all (in the workspace's score area), and the careful kernel has done them."""
+    the fast kernel declines: it has marked them all (in the workspace's score area), and the careful kernel has done them."""
     from paper_2607_09052_b200 import binding as B
     wl = synth.Workload("degenerate", 4, 8, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
                         key_model="iid", shuffle_pages=True, seed=7)
@@ -174,3 +174,117 @@ def test_a_block_has_the_same_bits_in_every_call(L, D, sub, rank, n, dtype):
     for one, other in zip(B.summary_views(cfg, whole), B.summary_views(cfg, parts)):
         if one is not None:
             assert torch.equal(one.contiguous().view(torch.uint8), other.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("kind", [0.5, 0.45, 0.4, 0.35, 0.3, "four600", "two", "one100", "token30", "bunch", "tied"])
+@pytest.mark.parametrize("L,D,sub,rank,n", [(64, 128, 0, 8, 12), (64, 128, 0, 4, 222), (64, 128, 85, 8, 222), (128, 128, 0, 4, 60),
+                                            (128, 128, 0, 8, 12), (128, 128, 85, 4, 12), (32, 128, 0, 8, 12)])
+def test_faint_directions_beside_strong_ones(L, D, sub, rank, n, kind):
+    """Directions down to a millionth of the largest eigenvalue, beside ones that outweigh them: standard deviations that fall by a
+    factor per channel, four channels 600 times the others, two of 1 000 and 32, one of 100, one key in a block 30 times the others; and
+    24 eigenvalues within 2 % of each other, four that are equal but for bf16's rounding.  Every eigenvalue comes out to the bound
+    of the tests above, 24 units of 2^-24 of the largest, factors are orthogonal to the same, and the rank-r matrix is as good as
+    twice that, but for what a residual of that size can turn the r-th direction where its neighbour is close."""
+    from paper_2607_09052_b200 import binding as B
+    wl = synth.Workload("faint", 2, 4, 4, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
+                        key_model="iid", shuffle_pages=False, seed=13)
+    inp = synth.generate(wl, "cuda")
+    nb = 8 * n
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    keys = inp["k_pages"][inp["page_table"].long()].permute(0, 2, 1, 3, 4).reshape(nb, L, D).float()
+    if isinstance(kind, float):
+        keys *= kind ** torch.arange(D, device="cuda")
+    elif kind == "four600":
+        keys[..., [3, 17, 18, 40]] *= 600.0
+    elif kind == "two":
+        keys[..., 3] *= 1000.0
+        keys[..., 17] *= 32.0
+    elif kind == "one100":
+        keys[..., 3] *= 100.0
+    elif kind == "token30":
+        keys[:, 5] *= 30.0
+    else:
+        m = min(24, L - 1) if kind == "bunch" else 4
+        rnd = torch.randn((nb, L, m), generator=gen, device="cuda")
+        u = torch.linalg.qr(torch.cat([torch.ones((nb, L, 1), device="cuda"), rnd], 2))[0][..., 1:]
+        s = torch.linspace(1.02 if kind == "bunch" else 1.0, 1.0, m, device="cuda").sqrt()
+        v = torch.linalg.qr(torch.randn((nb, D, m), generator=gen, device="cuda"))[0]
+        keys = (u * s) @ v.transpose(-1, -2) * 30.0
+    keys = keys.to(torch.bfloat16)
+    inp["k_pages"][inp["page_table"].long()] = keys.view(2, 4, n * L // 16, 16, D).transpose(1, 2)
+    cfg = B.make_config(wl)
+    summ = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"))
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, B.make_kv(inp), 0, wl.max_blocks, summ, ws)
+    assert B.cobs_read_status(ws) == 0
+    _, xi, _ = B.summary_views(cfg, summ)
+    some = torch.arange(0, nb, max(1, nb // 96), device="cuda")
+    K = keys[some].double()
+    K = K - K.mean(1, keepdim=True)
+    if sub:
+        K = K @ inp["u_q"].double()[some // n % 4]
+    sigma = K.transpose(-1, -2) @ K / L
+    lam, v = (t.cuda() for t in torch.linalg.eigh(sigma.cpu()))
+    top = lam[:, -1:]
+    x = xi.double().reshape(nb, rank, -1)[some]
+    n2 = (x * x).sum(-1)
+    bound = 24 * 2.0 ** -24
+    err = (n2 - lam.flip(-1)[:, :rank]).abs() / top
+    assert float(err.max()) <= bound, float(err.max())
+    prod = torch.triu((x @ x.transpose(-1, -2)).abs() / top[..., None], 1)
+    assert float(prod.max()) <= bound, float(prod.max())
+    want = (v[..., -rank:] * lam[:, None, -rank:]) @ v[..., -rank:].transpose(-1, -2)
+    off = torch.linalg.matrix_norm(x.transpose(-1, -2) @ x - want, ord=2) / top[:, 0]
+    gap = (lam[:, -rank] - lam[:, -rank - 1]) / top[:, 0]              # a residual of e turns the r-th direction by e / gap
+    most = 2 * bound + bound * lam[:, -rank] / top[:, 0] / gap.clamp_min(1e-12)
+    assert float((off / most).max()) <= 1.0, float((off / most).max())
+
+
+@pytest.mark.parametrize("L,D,sub,rank", [(64, 128, 0, 4), (64, 64, 24, 4), (128, 128, 0, 8), (128, 64, 0, 3), (128, 128, 85, 4)])
+def test_blocks_of_every_kind_in_one_call(L, D, sub, rank):
+    """Constant keys, two equal eigenvalues, steep and flat spectra, a key or a channel that outweighs the others, side by side in
+    ragged sequences: each kind takes its own way through the builder's kernels, and no other block notices."""
+    from paper_2607_09052_b200 import binding as B
+    n, lens = 45, [45 * L, 33 * L + 5, 3, 20 * L]
+    wl = synth.Workload("kinds", 4, 4, 2, D, n * L, L, 16, rank=rank, topk=2, window=L, summary_dtype="fp32", sub_dim=sub,
+                        key_model="iid", shuffle_pages=True, seed=23, seq_lens=lens)
+    inp = synth.generate(wl, "cuda")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    keys = torch.randn((8, n, L, D), generator=gen, device="cuda")
+    keys[:, 0::8] = degenerate_keys("equal", 1, L, D, gen)
+    keys[:, 1::8] = degenerate_keys("constant", 1, L, D, gen)
+    keys[:, 2::8] *= 0.4 ** torch.arange(D, device="cuda")
+    keys[:, 3::8, 5] *= 30.0
+    keys[:, 4::8, :, 7] *= 100.0
+    keys[:, 5::8] *= 0.8 ** torch.arange(D, device="cuda")
+    keys = keys.bfloat16()
+    inp["k_pages"][inp["page_table"].long()] = keys.view(4, 2, n * L // 16, 16, D).transpose(1, 2)
+    cfg = B.make_config(wl)
+    summ = B.SummaryBuffers(cfg, "cuda", inp.get("u_q"))
+    summ.xi.fill_(255)
+    ws = B.alloc_workspace(cfg, "cuda")
+    B.cobs_build_summaries(cfg, B.make_kv(inp), 0, n, summ, ws)
+    assert B.cobs_read_status(ws) == 0
+    mean, xi, _ = B.summary_views(cfg, summ)
+    K = keys.view(4, 2, n, L, D).double()
+    want_mean = K.mean(3)
+    K = K - want_mean[..., None, :]
+    if sub:
+        K = torch.einsum("bhnld,hds->bhnls", K, inp["u_q"].double())
+    lam = torch.linalg.eigvalsh((K.transpose(-1, -2) @ K / L).cpu()).cuda()
+    x = xi.double()
+    for b, t in enumerate(lens):
+        full = t // L
+        assert bool(torch.isnan(xi[b, :, full:]).all())               # (bytes of 255: nothing was written)
+        if not full:
+            continue
+        s = (b, slice(None), slice(0, full))
+        top = lam[s][..., -1:]
+        flat = top[..., 0] < 1e-9                                       # constant keys
+        assert torch.allclose(mean[s].double(), want_mean[s], rtol=0, atol=2.0 ** -20 * float(keys.abs().max()))
+        n2 = (x[s] * x[s]).sum(-1)
+        assert bool((n2[flat] == 0).all())
+        err = (n2 - lam[s].flip(-1)[..., :rank]).abs() / top
+        assert float(err[~flat].max()) <= 24 * 2.0 ** -24, float(err[~flat].max())
+        prod = torch.triu((x[s] @ x[s].transpose(-1, -2)).abs() / top[..., None], 1)
+        assert float(prod[~flat].max()) <= 24 * 2.0 ** -24, float(prod[~flat].max())
