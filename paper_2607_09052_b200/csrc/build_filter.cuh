@@ -4,21 +4,29 @@
 //   ->  its eigenvectors U by one-sided Jacobi rotations  ->  w = U V, each checked: |G w - theta w|
 //
 // A tridiagonal form takes L - 2 dependent reflections whatever is asked for; here the chain is as long as the r leading
-// directions need to stand out from the seventeenth on (6 to 20 products with G in all), and every product is a
+// directions need to stand out from the seventeenth on (7 to 40 products with G in all), and every product is a
 // contraction for the tensor pipe.  (Y. Zhou, Y. Saad, "A Chebyshev-Davidson algorithm for large symmetric eigenproblems",
 // 2007, for the filter; H. Rutishauser, "Simultaneous iteration method for symmetric matrices", 1970, for the scheme.)
 //
 // Layout.  Vectors are rows: V is 16 x L, and thread (gid, tig) holds rows gid and gid + 8, columns 8 g + 2 tig + {0, 1} of
 // every 8-token tile g, which is the accumulator of mma.sync m16n8k16 and, packed, its A operand: the result of one product
 // is the operand of the next without a shuffle.  G is symmetric, so its accumulators are the B operand in the same way.
-// Operands are split into f16 high and low parts (22 bits) and products are summed in fp32 (mma_split); the first round, which
+// Operands are split into f16 high and low parts (23 bits with the low part's sign, one less than fp32) and products are summed in fp32 (mma_split); the first round, which
 // only has to find the neighbourhood, takes the high parts alone.
 // Four warps hold every fourth tile each; V goes through shared memory for each product, one barrier.
 //
-// Measured at 128 tokens, three blocks per SM (cycles of one block; products with G, orthonormalisations): flat spectrum, rank 4:
-// 126 000 (20; 4), rank 8: 138 000 (25; 4), sixteen directions over noise, rank 8: 102 000 (10; 4), where the tridiagonal form took
-// 320 000.  A product is 2 200 cycles, an orthonormalisation 4 200, the small eigenproblem 33 000, of which the rotations of one
-// warp 22 000: latency, not the tensor pipe (20 products are 15 400 cycles of it).
+// Products with G and orthonormalisations of a block of 128 (medians; 1 % to 99 %), and time of 8 192 blocks, three per SM, by the
+// tridiagonal form and by this:
+//                                              rank 4                             rank 8
+//   flat spectrum                              21 (18-24); 4    3 130 -> 1 470 us    25 (22-30); 4     3 450 -> 1 700 us
+//   sixteen directions over noise               9 (8-11); 4     3 130 -> 1 160       11 (8-14); 4      3 460 -> 1 310
+//   one channel ten times the others           30 (26-34); 16   3 130 -> 2 490       33 (33-42); 17    3 460 -> 2 840
+//   thirty times                               32 (19-33); 17   3 130 -> 2 820       33 (22-35); 17    3 460 -> 3 610
+//   a hundred times (left to the other)         -               3 130 -> 3 630        -                3 450 -> 3 900
+//   24 eigenvalues within 5 % (the same)        -               3 130 -> 3 890        -                3 450 -> 4 150
+// A product is 2 200 cycles, an orthonormalisation 4 200, the small eigenproblem 33 000, of which the rotations of one warp 22 000:
+// latency, not the tensor pipe (20 products are 15 400 cycles of it).  168 registers for three blocks per SM, 350 bytes of them spilled
+// (in a subspace 255 for two, 116 bytes).
 #pragma once
 
 #include <type_traits>
@@ -252,6 +260,8 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
     xsum(f);
     fro2 = f[0];
   }
+  // (uniform) one direction holds nearly all of the trace: the others' eigenvalues are left to the tridiagonal form
+  if (r_eff > 1 && fro2 > 0.93f * ((float)L * mu) * ((float)L * mu)) return true;
   // ---- G as B fragments -----------------------------------------------------------------------------------------------------------
   uint2 gh[NT][KT];                                     // the high halves
   uint2 *gl = reinterpret_cast<uint2 *>(sm) + warp * (NT * KT * 32) + lane;
@@ -366,8 +376,9 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
     o0 = quad_sum(lo(t0) + hi(t0)); o1 = quad_sum(lo(t1) + hi(t1));
   };
   // V <- orthonormal rows (of length 16) of the same span: S = V V^T, rows of the inverse of its Cholesky factor by elimination.
-  // A pivot below 2e-5 of the row is too near the rounding of S to be used: nothing is eliminated with it, and the row stays as it
-  // is for the next round, or is left out of the solution (`final`).  n: squared norms of V's rows.
+  // What is left of a row's square, 256 to 1024 by the power of two that scales it, may be too near the rounding of S to be used:
+  // below kPivot (2e-5 to 8e-5 of it) nothing is eliminated with the row.  Less the earlier rows it goes on to the next round, or
+  // is left out of the solution (`final`), which then has to account for it.  n: squared norms of V's rows.
   auto orthonormalise = [&](const float (&n)[2], bool final) {
     constexpr float kPivot = 2e-2f;
     float s[8], m[8];
@@ -564,6 +575,10 @@ __device__ __forceinline__ bool filter_solve(u64 (&A)[Filter<L>::NT][L / 8], flo
             for (int i = 0; i < 4; ++i) V[a][i] *= 1.f / 256.f;
           continue;
         }
+        // Left to the tridiagonal form: wanted directions so far below the leading one that its rounding outgrows them, and sixteen
+        // directions too close to one another to be parted soon.
+        failed = d_max < 1.17f * d_min || (round > 4 && d_r < 2e-4f * d_max);
+        if (failed) break;
         b = fmaxf(fmaxf(d_min, 0.02f * d_r), 1e-5f * d_max);      // (lower, and the leading rows drown the others)
         const float ib = __fdividef(2.0f, b);
         const float xr = -__logf(cheb_damp(fmaf(d_r, ib, -1.0f))), x1 = fmaxf(-__logf(cheb_damp(fmaf(d_max, ib, -1.0f))), 0.5f);

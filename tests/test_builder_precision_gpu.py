@@ -288,3 +288,40 @@ def test_blocks_of_every_kind_in_one_call(L, D, sub, rank):
         assert float(err[~flat].max()) <= 24 * 2.0 ** -24, float(err[~flat].max())
         prod = torch.triu((x[s] @ x[s].transpose(-1, -2)).abs() / top[..., None], 1)
         assert float(prod[~flat].max()) <= 24 * 2.0 ** -24, float(prod[~flat].max())
+
+
+@pytest.mark.parametrize("kind", ["bunch", "one100"])
+def test_hard_spectra_take_no_multiple_of_the_time(kind):
+    """Blocks that the filter has no business with (24 eigenvalues within 2 % of each other; one channel 100 times the others) are
+    left to the tridiagonal form early: 8 192 blocks of 128 take at most 3.3 times what flat spectra take (measured 2.6 and 2.5; 7.5 and 4.1
+    when the filter saw them through first)."""
+    from paper_2607_09052_b200 import binding as B
+    L, n = 128, 256
+    wl = synth.Workload("time", 4, 8, 8, 128, n * L, L, 16, rank=4, topk=2, window=L, summary_dtype="fp4", key_model="iid",
+                        shuffle_pages=False, seed=13)
+    inp = synth.generate(wl, "cuda")
+    cfg = B.make_config(wl)
+    summ, ws, kv = B.SummaryBuffers(cfg, "cuda"), B.alloc_workspace(cfg, "cuda"), B.make_kv(inp)
+
+    def fastest():
+        times = []
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            B.cobs_build_summaries(cfg, kv, 0, n, summ, ws)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        return min(times)
+
+    flat = fastest()
+    if kind == "one100":
+        inp["k_pages"][..., 3] *= 100.0
+    else:
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        u = torch.linalg.qr(torch.cat([torch.ones((64, L, 1), device="cuda"), torch.randn((64, L, 24), generator=gen, device="cuda")], 2))[0][..., 1:]
+        v = torch.linalg.qr(torch.randn((64, 128, 24), generator=gen, device="cuda"))[0]
+        keys = ((u * torch.linspace(1.02, 1.0, 24, device="cuda").sqrt()) @ v.transpose(-1, -2) * 30.0).bfloat16()
+        keys = keys.repeat(4 * 8 * n // 64, 1, 1).view(4, 8, n * L // 16, 16, 128)
+        inp["k_pages"][inp["page_table"].long()] = keys.transpose(1, 2)
+    assert fastest() <= 3.3 * flat
