@@ -22,8 +22,8 @@
 //   sixteen directions over noise               9 (8-11); 4     3 130 -> 1 160       11 (8-14); 4      3 460 -> 1 310
 //   one channel ten times the others           30 (26-34); 16   3 130 -> 2 490       33 (33-42); 17    3 460 -> 2 840
 //   thirty times                               32 (19-33); 17   3 130 -> 2 820       33 (22-35); 17    3 460 -> 3 610
-//   a hundred times (left to the other)         -               3 130 -> 3 630        -                3 450 -> 3 900
-//   24 eigenvalues within 5 % (the same)        -               3 130 -> 3 890        -                3 450 -> 4 150
+//   a hundred times (left to the other)         -               3 130 -> 3 730        -                3 450 -> 4 030
+//   24 eigenvalues within 5 % (the same)        -               3 130 -> 3 980        -                3 450 -> 4 370
 // A product is 2 200 cycles, an orthonormalisation 4 200, the small eigenproblem 33 000, of which the rotations of one warp 22 000:
 // latency, not the tensor pipe (20 products are 15 400 cycles of it).  168 registers for three blocks per SM, 350 bytes of them spilled
 // (in a subspace 255 for two, 116 bytes).

@@ -63,8 +63,8 @@ __device__ __forceinline__ void add4(float (&c)[4], const float (&t)[4]) {
 // projection's sums taken the same way, 16 384 blocks of 64: 1.35 -> 1.38 ms.)
 template <bool ZERO = false>                          // (c = instead of c +=)
 __device__ __forceinline__ void mma_split(float (&c)[4], const uint32_t (&h)[4], const uint32_t (&l)[4], uint32_t bh0, uint32_t bh1, uint32_t bl0, uint32_t bl1) {
-  float t[4];
-  mma_f16_zero(t, h[0], h[1], h[2], h[3], bl0, bl1);
+  float t[4] = {0.f, 0.f, 0.f, 0.f};
+  mma_f16(t, h[0], h[1], h[2], h[3], bl0, bl1);
   mma_f16(t, l[0], l[1], l[2], l[3], bh0, bh1);
   mma_f16(t, h[0], h[1], h[2], h[3], bh0, bh1);
   if constexpr (ZERO) {
